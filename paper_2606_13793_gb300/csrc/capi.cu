@@ -167,6 +167,13 @@ struct fmm_plan_s {
   int* d_m2l_tile_k = nullptr;
   long long* d_m2l_tile_w = nullptr;
   int m2l_ntiles = 0;
+  // reflection-basis form of the CUDA-core harmonic M2L (k_sym.cu; [1]: of
+  // its transpose) and of the leaf-4 near field
+  SymTab* d_sym_tab[2] = {nullptr, nullptr};
+  void* d_sym_ws[2] = {nullptr, nullptr};
+  void* d_sym_wq[2] = {nullptr, nullptr};
+  void* d_sym_near = nullptr;
+  int sym_q_len[2] = {0, 0};
   // near field
   void* d_w_near = nullptr;
   int* d_near_tile_k = nullptr;
@@ -194,6 +201,7 @@ struct fmm_plan_s {
   size_t rho_hi_off = 0, rho_lo_off = 0;
   size_t part_off = 0;  // neighbour-split partial sums of the small SIMT levels
   size_t part_cap = 0;  // bytes there
+  size_t near_part_off = 0, near_part_cap = 0;  // the near field's own (it runs beside the levels)
   // CUDA-core contraction variant of each M2L level and of the near field
   // (shape / neighbour split; fmm_plan_autotune times the candidates)
   struct SimtChoice {
@@ -450,22 +458,121 @@ void m2l_weights(const MultiIndex& mi, const TaylorTable& tt, std::vector<T>& W,
   }
   W.assign((size_t)off, T(0));
   if (!fill) return;
-  for (int t = 0; t < ntiles; ++t) {
-    const int K = tile_k[t];
-    for (int d = 0; d < 27; ++d) {
-      T* blk = W.data() + tile_w[t] + (long long)d * K * kNTile;
-      for (int k = 0; k < K; ++k)
-        for (int j = 0; j < kNTile; ++j) {
-          const int n = t * kNTile + j;
-          if (!harm) {
-            blk[(long long)k * kNTile + j] = (T)m2l_entry(mi, tt, d, k, n);
-          } else if (n / 8 < nk && k / 8 < nk) {
-            blk[(long long)k * kNTile + j] =
-                (T)m2l_entry(mi, tt, d, red[k / 8] * 8 + k % 8, red[n / 8] * 8 + n % 8);
+  // per (alpha, beta) pair the same factor for every neighbour and child pair
+  // (m2l_entry's, in its order of operations)
+  for (int b = 0; b < nk; ++b)
+    for (int a = 0; a < nk; ++a) {
+      const int be = harm ? red[b] : b, al = harm ? red[a] : a;
+      const int ob = level_of_order(mi, be), oa = level_of_order(mi, al);
+      if (oa + ob > p || oa > mi.mo || ob > mi.lo) continue;
+      const int g = mi.index(mi.a[al] + mi.a[be], mi.b[al] + mi.b[be], mi.c[al] + mi.c[be]);
+      const double mult = binom(mi.a[al] + mi.a[be], mi.a[al]) * binom(mi.b[al] + mi.b[be], mi.b[al]) *
+                          binom(mi.c[al] + mi.c[be], mi.c[al]);
+      const double f = ((oa & 1) ? -1.0 : 1.0) * mult;
+      const int t = b * 8 / kNTile, j0 = b * 8 % kNTile, K = tile_k[t];
+      T* base = W.data() + tile_w[t] + (long long)a * 8 * kNTile + j0;
+      for (int d = 0; d < 27; ++d) {
+        if (d == 13) continue;  // no child of the same parent
+        T* blk = base + (long long)d * K * kNTile;
+        const int D[3] = {d % 3 - 1, (d / 3) % 3 - 1, d / 9 - 1};
+        for (int cs = 0; cs < 8; ++cs)
+          for (int ct = 0; ct < 8; ++ct) {
+            int u[3], cheb = 0;
+            for (int q = 0; q < 3; ++q) {
+              u[q] = ((ct >> q) & 1) - ((cs >> q) & 1) - 2 * D[q];
+              cheb = std::max(cheb, std::abs(u[q]));
+            }
+            if (cheb >= 2) blk[(long long)cs * kNTile + ct] = (T)(f * (-tt.at(u)[g]));
+          }
+      }
+    }
+}
+
+// Reflection-basis weights of the harmonic M2L (k_sym.cu).  For a component
+// pair, w[j] = the unit-box weight to the upper child (1, 1, 1) from source
+// child position j in -2 .. 3 per axis (0, 1: the own parent's); per axis the
+// block of sign s holds w[1 + k] + s (-1)^alpha_q w[-k], and the 1/8 of the
+// way back is folded in (exact).
+struct SymHost {
+  SymTab tab{};
+  std::vector<double> Ws, Wq;
+};
+void sym_m2l_weights(const MultiIndex& mi, const TaylorTable& tt, SymHost& H, bool fill) {
+  const std::vector<int> red = harmonic_components(mi);
+  SymTab& T = H.tab;
+  const int nk = (int)red.size();
+  T = SymTab{};
+  T.nk = nk;
+  T.nunits = (nk + 7) / 8;
+  for (int i = 0; i < nk; ++i) {
+    const int r = red[i], o = level_of_order(mi, r);
+    T.par[i] = (unsigned char)((mi.a[r] & 1) | (mi.b[r] & 1) << 1 | (mi.c[r] & 1) << 2);
+    const int q = std::min(mi.p - o, mi.mo);
+    T.kb[i] = o > mi.lo ? 0 : (q + 1) * (q + 1);
+  }
+  long long off = 0;
+  for (int u = 0; u < T.nunits; ++u) {
+    for (int a = 0; a < nk; ++a) {
+      int live = 0;
+      while (live < 8 && u * 8 + live < nk && T.kb[u * 8 + live] > a) ++live;
+      if (live > 4) T.n8[u] = a + 1;
+      if (live > 1) T.n4[u] = a + 1;
+      if (live > 0) T.n1[u] = a + 1;
+    }
+    T.w_off[u] = off;
+    off += 216LL * (8 * T.n8[u] + 4 * (T.n4[u] - T.n8[u]) + (T.n1[u] - T.n4[u]));
+  }
+  int ql = 0;
+  for (int a = 0; a < nk; ++a) {
+    int nb = 0;
+    while (nb < nk && T.kb[nb] > a) ++nb;
+    T.q_off[a] = ql;
+    ql += (nb + 3) / 4 * 4 * 8;
+  }
+  T.q_len = ql;
+  H.Ws.assign((size_t)off, 0.0);
+  H.Wq.assign((size_t)27 * ql, 0.0);
+  if (!fill) return;
+  std::vector<double> w(216), x(216);
+  for (int a = 0; a < nk; ++a)
+    for (int b = 0; b < nk; ++b) {
+      if (a >= T.kb[b]) continue;
+      const int ra = red[a], rb = red[b], oa = level_of_order(mi, ra);
+      const int g = mi.index(mi.a[ra] + mi.a[rb], mi.b[ra] + mi.b[rb], mi.c[ra] + mi.c[rb]);
+      const double mult = binom(mi.a[ra] + mi.a[rb], mi.a[ra]) * binom(mi.b[ra] + mi.b[rb], mi.b[ra]) *
+                          binom(mi.c[ra] + mi.c[rb], mi.c[ra]) * ((oa & 1) ? -1.0 : 1.0) * 0.125;
+      for (int i = 0; i < 216; ++i) {
+        const int u[3] = {1 - (i % 6 - 2), 1 - ((i / 6) % 6 - 2), 1 - (i / 36 - 2)};
+        const int cheb = std::max(std::abs(u[0]), std::max(std::abs(u[1]), std::abs(u[2])));
+        w[i] = cheb < 2 ? 0.0 : mult * (-tt.at(u)[g]);
+      }
+      // per axis: position j + 2 in 0 .. 5 -> 2 k + (0: sum, 1: difference)
+      const int str[3] = {1, 6, 36};
+      for (int q = 0; q < 3; ++q) {
+        const double f = (T.par[a] >> q) & 1 ? -1.0 : 1.0;
+        for (int i = 0; i < 216; ++i) {
+          if ((i / str[q]) % 6) continue;
+          for (int k = 0; k < 3; ++k) {
+            const double up = w[i + (3 + k) * str[q]], lo = w[i + (2 - k) * str[q]];
+            x[i + 2 * k * str[q]] = up + f * lo;
+            x[i + (2 * k + 1) * str[q]] = up - f * lo;
           }
         }
+        w.swap(x);
+      }
+      const int un = b / 8, n = b % 8;
+      const int nl = a < T.n8[un] ? 8 : a < T.n4[un] ? 4 : 1;
+      const long long wo = T.w_off[un] + 216LL * (a < T.n8[un] ? 8 * a
+                                                  : a < T.n4[un] ? 8 * T.n8[un] + 4 * (a - T.n8[un])
+                                                                 : 8 * T.n8[un] + 4 * (T.n4[un] - T.n8[un]) + a - T.n4[un]);
+      for (int k = 0; k < 27; ++k)
+        for (int sg = 0; sg < 8; ++sg) {
+          const int kx = k % 3, ky = (k / 3) % 3, kz = k / 9;
+          const double v = w[(2 * kx + (sg & 1)) + 6 * (2 * ky + ((sg >> 1) & 1)) + 36 * (2 * kz + (sg >> 2))];
+          H.Ws[(size_t)(wo + ((((ky * 3 + kx) * 4 + (sg & 3)) * 3 + kz) * nl + n) * 2 + (sg >> 2))] = v;
+          H.Wq[(size_t)k * ql + T.q_off[a] + b * 8 + sg] = v;
+        }
     }
-  }
 }
 
 uint16_t bf16_rn(float f) {
@@ -1478,6 +1585,40 @@ void near_weights(int b, int comps, std::vector<T>& W, std::vector<int>& tile_k,
 
 // M2M: Mt_alpha(P) += C(alpha,beta) 2^-|alpha| (+-1/2)^(alpha-beta) Mt_beta(C);
 // L2L: Lt_beta(C) += C(gamma,beta) 2^(-1-|gamma|) (+-1/2)^(gamma-beta) Lt_gamma(P).
+// Reflection-basis weights of the leaf-4 near field (k_sym.cu): source
+// position j in -4 .. 7 and upper targets 2, 3 per axis; mirror pairs
+// (2 + k, 1 - k).  [36 (x, y) pairs][4 signs][6 z pairs][8 targets][2].
+void sym_near4_weights(std::vector<double>& Ws) {
+  Ws.assign((size_t)36 * 4 * 6 * 8 * 2, 0.0);
+  const int str[3] = {1, 12, 144};
+  std::vector<double> w(1728), x(1728);
+  for (int n = 0; n < 8; ++n) {
+    const int t[3] = {2 + (n & 1), 2 + ((n >> 1) & 1), 2 + (n >> 2)};
+    for (int i = 0; i < 1728; ++i) {
+      const double r0 = t[0] - (i % 12 - 4), r1 = t[1] - ((i / 12) % 12 - 4), r2 = t[2] - (i / 144 - 4);
+      const double r = std::sqrt(r0 * r0 + r1 * r1 + r2 * r2);
+      w[i] = -0.125 / (r > 0.0 ? r : 1.0);
+    }
+    for (int q = 0; q < 3; ++q) {
+      for (int i = 0; i < 1728; ++i) {
+        if ((i / str[q]) % 12) continue;
+        for (int k = 0; k < 6; ++k) {
+          const double up = w[i + (6 + k) * str[q]], lo = w[i + (5 - k) * str[q]];
+          x[i + 2 * k * str[q]] = up + lo;
+          x[i + (2 * k + 1) * str[q]] = up - lo;
+        }
+      }
+      w.swap(x);
+    }
+    for (int k = 0; k < 216; ++k)
+      for (int sg = 0; sg < 8; ++sg) {
+        const int kx = k % 6, ky = (k / 6) % 6, kz = k / 36;
+        Ws[(size_t)(((((ky * 6 + kx) * 4 + (sg & 3)) * 6 + kz) * 8 + n) * 2 + (sg >> 2))] =
+            w[(2 * kx + (sg & 1)) + 12 * (2 * ky + ((sg >> 1) & 1)) + 144 * (2 * kz + (sg >> 2))];
+      }
+  }
+}
+
 void shift_tables(const MultiIndex& mi, std::vector<int>& m2m_start, std::vector<ShiftEntry>& m2m,
                   std::vector<int>& l2l_start, std::vector<ShiftEntry>& l2l) {
   const int nc = mi.nc;
@@ -1526,8 +1667,48 @@ namespace {
 // arena layout, tables.  Device memory comes from P->dev_alloc (cudaMalloc
 // for plans, the static array for the allocation-free solve).  On failure
 // the caller releases P.
-NbrGemm m2l_gemm(fmm_plan_t P, int l);
+bool sym_level(fmm_plan_t P, int l);
+NbrGemm m2l_gemm(fmm_plan_t P, int l, int form = -1);
 NbrGemm near_gemm(fmm_plan_t P);
+
+// Default variant of a reflection-basis contraction (k_sym.cu), measured over
+// 32^3 .. 256^3 cells (FP32 p = 6, FP64 p = 4, 6):
+//  * M2L levels of at most 512 rows: the row forms, split 27 ways (one launch
+//    for all of them; FP64 in the reflection basis, 8 rows a block);
+//  * other M2L levels: the long z-run from 100 tiles on (64^3 rows 2.9 ms
+//    against 3.4 ms with the short one, 32^3 0.51 against 0.56 ms, 24^3 0.32
+//    against 0.23 ms), else the short one split until 304 blocks (two per SM)
+//    run; FP64
+//    until the first unit's blocks, half of all work, fill the SMs twice
+//    (12^3 rows: 9 ways 1.25 ms, 3 ways 1.38 ms);
+//  * near field: the long z-run from 100 tiles on (32^3 boxes 46 us, short 55),
+//    else the short one, FP32 split until 32 blocks run (16^3 boxes: 31 us
+//    unsplit, 57 us in three beside the M2L), FP64 until every SM has one.
+void sym_default(fmm_plan_t P, const NbrGemm& g, fmm_plan_s::SimtChoice* c, bool f64) {
+  const long long rows = (long long)g.grid[0] * g.grid[1] * g.grid[2];
+  auto tiles = [&](int rz) {
+    return (long long)((g.grid[0] + 7) / 8) * ((g.grid[1] + 3) / 4) * ((g.grid[2] + rz - 1) / rz);
+  };
+  const size_t one = (size_t)rows * g.n_cols * (f64 ? 8 : 4);
+  auto split = [&](long long blocks, long long want, size_t cap) {
+    int d = 1;
+    while (d < 9 && blocks * d < want && (size_t)(3 * d) * one <= cap) d *= 3;
+    return d;
+  };
+  if (!g.skip_center) {  // the near field
+    c->shape = tiles(f64 ? 4 : 8) >= 100 ? 1 : 2;
+    c->dsplit = c->shape == 1 ? 1 : split(tiles(f64 ? 2 : 4), f64 ? 152 : 32, P->near_part_cap);
+  } else if (c->dsplit == 27 && rows <= 512 && 27 * one <= P->part_cap) {
+    c->shape = f64 ? 3 : 0;
+    c->dsplit = 27;
+  } else {
+    const long long t = tiles(f64 ? 2 : 4);
+    c->shape = tiles(f64 ? 4 : 8) >= 100 ? 1 : 2;
+    c->dsplit = c->shape == 1 ? 1
+                : f64         ? split(t, 304, P->part_cap)
+                              : split(t * ((g.n_cols / 8 + 7) / 8), 304, P->part_cap);
+  }
+}
 
 fmm_status plan_init(fmm_plan_t P, const int d3[3], double dx, double G, int order, int leaf, const fmm_opts& o,
                      cudaStream_t stream, int dev) {
@@ -1639,14 +1820,17 @@ fmm_status plan_init(fmm_plan_t P, const int d3[3], double dx, double G, int ord
       if (!P->lev[l].tc) want = std::max(want, 27 * one);
     }
     // room for the autotuner's neighbour-split candidates (M2L levels and the
-    // near field), up to 64 MiB
-    if (!P->near_tc)
-      want = std::max(want, (size_t)27 * (size_t)P->lev[P->L].nbox * (size_t)(P->b * P->b * P->b) *
-                                (size_t)P->near_comps * P->esize());
+    // near field), up to 64 MiB each
+    if (!P->near_tc && !P->no_split)
+      P->near_part_cap = std::min((size_t)27 * (size_t)P->lev[P->L].nbox * (size_t)(P->b * P->b * P->b) *
+                                      (size_t)P->near_comps * P->esize(),
+                                  (size_t)64 << 20);
     if (!P->no_split) part = std::max(part, std::min(want, (size_t)64 << 20));
     P->part_off = off;
     P->part_cap = part;
     off = align(off + part);
+    P->near_part_off = off;
+    off = align(off + P->near_part_cap);
     for (int l = 2; l <= P->L; ++l) P->m2l_choice[l].dsplit = P->split_level(l) ? 27 : 1;
   }
   // Default variants before any tuning: the small levels split over their 27
@@ -1655,6 +1839,10 @@ fmm_status plan_init(fmm_plan_t P, const int d3[3], double dx, double G, int ord
     g.dsplit = 1;
     if (f64 && P->tc_kind >= 0) {  // coarse FP64 levels beside the tensor-core levels
       c->shape = 3;
+      return;
+    }
+    if (g.sym == kSymNear4 || (g.sym == kSymM2l || P->harm_cc) && g.skip_center) {
+      sym_default(P, g, c, f64);
       return;
     }
     if (c->dsplit != 1 || !zrun_eligible(g, tk.data(), (int)tk.size())) return;
@@ -1700,6 +1888,28 @@ fmm_status plan_init(fmm_plan_t P, const int d3[3], double dx, double G, int ord
     if (P->L >= 2 && !P->static_keep_tables) tt.build(P->mi);
     std::vector<int> tk;
     std::vector<long long> tw;
+    // reflection-basis weights in the level's type (all CUDA-core harmonic levels hold one type)
+    auto put_sym = [&](const MultiIndex& mi, int slot) -> fmm_status {
+      SymHost H;
+      sym_m2l_weights(mi, tt, H, !P->static_keep_tables);
+      std::vector<SymTab> tab(1, H.tab);
+      P->sym_q_len[slot] = H.tab.q_len;
+      fmm_status e;
+      if (any64) {
+        double *a = nullptr, *b = nullptr;
+        if ((e = P->upload(H.Ws, &a, s)) || (e = P->upload(H.Wq, &b, s))) return e;
+        P->d_sym_ws[slot] = a;
+        P->d_sym_wq[slot] = b;
+      } else {
+        const std::vector<float> wsf(H.Ws.begin(), H.Ws.end()), wqf(H.Wq.begin(), H.Wq.end());
+        float *a = nullptr, *b = nullptr;
+        if ((e = P->upload(wsf, &a, s)) || (e = P->upload(wqf, &b, s))) return e;
+        P->d_sym_ws[slot] = a;
+        P->d_sym_wq[slot] = b;
+      }
+      return P->upload(tab, &P->d_sym_tab[slot], s);
+    };
+    if (P->harm_cc && (any64 || any32) && (st = put_sym(P->mi, 0))) return cleanup(st);
     if (any64) {
       std::vector<double> W;
       m2l_weights<double>(P->mi, tt, W, tk, tw, !P->static_keep_tables, P->harm_cc);
@@ -1721,6 +1931,7 @@ fmm_status plan_init(fmm_plan_t P, const int d3[3], double dx, double G, int ord
     mt.mo = P->p;
     mt.lo = P->mi.mo;
     P->asym = P->mi.mo < P->p && P->L >= 2;
+    if (P->asym && (any64 || any32) && P->harm_cc && (st = put_sym(mt, 1))) return cleanup(st);
     if (P->asym && (any64 || any32)) {
       std::vector<int> tk2;
       std::vector<long long> tw2;
@@ -1843,6 +2054,22 @@ fmm_status plan_init(fmm_plan_t P, const int d3[3], double dx, double G, int ord
       float* d = nullptr;
       if ((st = P->upload(W, &d, s))) return cleanup(st);
       P->d_w_near = d;
+    }
+    // (the static array: where it leaves room, the two small tables below included)
+    const bool room = !P->static_base || P->static_used + 36 * 384 * P->esize() + 4096 <= P->static_cap;
+    if (P->b == 4 && P->near_comps == 1 && !P->near_tc && room) {
+      std::vector<double> W;
+      sym_near4_weights(W);
+      if (P->f64_data()) {
+        double* d = nullptr;
+        if ((st = P->upload(W, &d, s))) return cleanup(st);
+        P->d_sym_near = d;
+      } else {
+        const std::vector<float> Wf(W.begin(), W.end());
+        float* d = nullptr;
+        if ((st = P->upload(Wf, &d, s))) return cleanup(st);
+        P->d_sym_near = d;
+      }
     }
     P->near_ntiles = (int)tk.size();
     P->h_near_tile_k = tk;
@@ -2174,6 +2401,8 @@ bool fused_down(fmm_plan_t P) {
   return P->lev[L].f64 == want && P->lev[L - 1].f64 == want;
 }
 
+bool sym_level(fmm_plan_t P, int l);
+
 // Per-level dispatch helpers (a level's expansions are FP64 or FP32).
 fmm_status do_m2m(fmm_plan_t P, const TreeTables& tt, int l, cudaStream_t s) {
   const Level &c = P->lev[l], &q = P->lev[l - 1];
@@ -2181,7 +2410,7 @@ fmm_status do_m2m(fmm_plan_t P, const TreeTables& tt, int l, cudaStream_t s) {
   void* hi = planes ? P->arena + q.hi_off : nullptr;
   void* lo = planes ? P->arena + q.lo_off : nullptr;
   void* fold = q.fold_off ? P->arena + q.fold_off : nullptr;
-  const int harm = (planes && P->harm) || fold ? 1 : 0;
+  const int harm = sym_level(P, l - 1) ? 2 : (planes && P->harm) || fold ? 1 : 0;  // 2: component-major folds
   cudaError_t e;
   if (c.f64)
     e = launch_m2m<double, double>(tt, c, static_cast<const double*>(P->M(l)), q, static_cast<double*>(P->M(l - 1)),
@@ -2230,7 +2459,20 @@ fmm_status do_l2l(fmm_plan_t P, const TreeTables& tt, int l, cudaStream_t s, int
   return FMM_OK;
 }
 
-NbrGemm m2l_gemm(fmm_plan_t P, int l) {
+// Whether a CUDA-core level's M2L runs in the reflection basis (its folded
+// multipoles are then component-major): the harmonic form on the z-run
+// shapes, and every FP64 shape.  The FP32 row shapes keep the direct sums
+// (k_gemm_rows.cu: as fast on so few rows, and their rounding decides the
+// force's).
+bool sym_level(fmm_plan_t P, int l) {
+  const Level& lv = P->lev[l];
+  const int sh = P->m2l_choice[l].shape;
+  return lv.fold_off && !lv.tc && (lv.f64 || sh == 1 || sh == 2);
+}
+
+// form: the level's own (-1: sym_level), or forced: 0 direct, 1 reflection
+// basis (levels with folded multipoles); the folds must be in its layout.
+NbrGemm m2l_gemm(fmm_plan_t P, int l, int form) {
   const Level& lv = P->lev[l];
   NbrGemm g;
   // harmonic: folded multipoles in, the c <= 1 locals out (compact rows)
@@ -2250,6 +2492,14 @@ NbrGemm m2l_gemm(fmm_plan_t P, int l) {
   g.dsplit = P->m2l_choice[l].dsplit;
   g.partial = P->arena + P->part_off;
   g.skip_center = 1;  // the interaction list holds no child of the same parent
+  if (form < 0 ? sym_level(P, l) : form == 1) {
+    g.sym = kSymM2l;
+    g.st = P->d_sym_tab[tr];
+    g.Ws = P->d_sym_ws[tr];
+    g.Wq = P->d_sym_wq[tr];
+    g.q_len = P->sym_q_len[tr];
+    g.lda = lv.npar;
+  }
   return g;
 }
 
@@ -2267,7 +2517,11 @@ NbrGemm near_gemm(fmm_plan_t P) {
   g.accumulate = 0;
   g.shape = P->near_choice.shape;
   g.dsplit = P->near_choice.dsplit;
-  g.partial = P->arena + P->part_off;
+  if (P->d_sym_near) {
+    g.sym = kSymNear4;
+    g.Ws = P->d_sym_near;
+  }
+  g.partial = P->arena + P->near_part_off;
   return g;
 }
 
@@ -2372,6 +2626,61 @@ fmm_status do_m2l(fmm_plan_t P, int l, cudaStream_t s) {
   return FMM_OK;
 }
 
+// Levels whose M2L runs in a row form split 27 ways: those of one shape go in
+// one launch while their partial sums fit the scratch side by side (64 MiB:
+// levels of up to ~1500 rows together).
+bool rows_level(fmm_plan_t P, int l) {
+  const Level& lv = P->lev[l];
+  const fmm_plan_s::SimtChoice c = P->m2l_choice[l];
+  if (lv.tc || c.dsplit != 27) return false;
+  return sym_level(P, l) ? c.shape == 0 || c.shape == 3 : !lv.f64 && c.shape == 0;
+}
+// Levels that run the direct FP32 z-run unsplit (the allocation-free solve has
+// no scratch for partial sums) and do not fill the GPU: all of them in one
+// launch of its narrow form, the same sums.
+bool narrow_level(fmm_plan_t P, int l) {
+  const Level& lv = P->lev[l];
+  if (lv.tc || lv.f64 || sym_level(P, l) || P->m2l_choice[l].shape != 1 || P->m2l_choice[l].dsplit != 1) return false;
+  return (long long)((lv.np[0] + 7) / 8) * ((lv.np[1] + 3) / 4) * ((lv.np[2] + 7) / 8) * P->m2l_ntiles < kZrunNarrowBlocks;
+}
+size_t rows_partial(fmm_plan_t P, int l) {
+  const Level& lv = P->lev[l];
+  return ((size_t)27 * lv.npar * 8 * (lv.fold_off ? P->nr : P->nc) * (lv.f64 ? 8 : 4) + 255) & ~(size_t)255;
+}
+std::vector<std::vector<int>> row_groups(fmm_plan_t P, const int* ls, int n) {
+  std::vector<std::vector<int>> out;
+  for (int shape : {0, 3}) {
+    size_t used = 0;
+    bool open = false;
+    for (int i = 0; i < n; ++i) {
+      const int l = ls[i];
+      if (!rows_level(P, l) || P->m2l_choice[l].shape != shape) continue;
+      const size_t need = rows_partial(P, l);
+      if (!open || used + need > P->part_cap || (int)out.back().size() == std::min(kSymGroupMax, kRowsGroupMax) ||
+          P->lev[l].f64 != P->lev[out.back()[0]].f64 || sym_level(P, l) != sym_level(P, out.back()[0])) {
+        out.emplace_back();
+        open = true;
+        used = 0;
+      }
+      out.back().push_back(l);
+      used += need;
+    }
+  }
+  return out;
+}
+fmm_status do_m2l_rows(fmm_plan_t P, const std::vector<int>& ls, cudaStream_t s) {
+  NbrGemm g[std::max(kSymGroupMax, kRowsGroupMax)];
+  size_t used = 0;
+  for (size_t i = 0; i < ls.size(); ++i) {
+    g[i] = m2l_gemm(P, ls[i]);
+    g[i].partial = P->arena + P->part_off + used;
+    used += rows_partial(P, ls[i]);
+  }
+  CUDA_TRY(g[0].sym ? launch_nbr_gemm_sym_rows(g, (int)ls.size(), s)
+                    : launch_nbr_gemm_rows(g, (int)ls.size(), s));
+  return FMM_OK;
+}
+
 // adjoint = true (fmm_solve_adjoint): the same chain on the adjoint source,
 // except that with the final-stage M2P the leaf level runs its transpose
 // (P2L into the leaf locals, then L2L adds the parents' and L2P evaluates);
@@ -2404,7 +2713,7 @@ fmm_status run_solve(fmm_plan_t P, const T* rho, T* phi, T* accel, cudaStream_t 
                            mplanes ? P->arena + lf.hi_off : nullptr, mplanes ? P->arena + lf.lo_off : nullptr,
                            (P->near_tc && near_rows) ? P->arena + P->rho_hi_off : nullptr,
                            (P->near_tc && near_rows) ? P->arena + P->rho_lo_off : nullptr, P->d_flag,
-                           ((mplanes && P->harm) || lf.fold_off) ? 1 : 0,
+                           sym_level(P, L) ? 2 : ((mplanes && P->harm) || lf.fold_off) ? 1 : 0,
                            lf.fold_off ? reinterpret_cast<T*>(P->arena + lf.fold_off) : nullptr, s, adj_dip));
   }
   const bool p2l = adjoint && P->m2p;  // leaf level by the transpose of M2P
@@ -2423,33 +2732,49 @@ fmm_status run_solve(fmm_plan_t P, const T* rho, T* phi, T* accel, cudaStream_t 
   // level of the FP32/FP64 precisions) on the plan's side stream, the
   // tensor-core levels and the near field on `s`; the two use different
   // units of the SM.  The L2L chain then adds the parents' locals, coarse to
-  // fine.  A near field split over neighbour groups shares the split scratch
-  // with the CUDA-core levels, so it runs after them on the same stream.
+  // fine.
   if (L < 2) {
     StageTimer t(P, ST_L2L, s);
     CUDA_TRY(launch_zero<T>(static_cast<T*>(P->Lx(L)), P->lev[L].bytes / sizeof(T), s));
   }
   bool any_simt = false;
   for (int l = 2; l <= L; ++l) any_simt |= !P->lev[l].tc;
-  const bool near_side = !P->near_tc && P->near_choice.dsplit > 1 && !adj_g;
-  const bool fork = P->side && (any_simt || near_side);
+  const bool fork = P->side && any_simt;
   cudaStream_t sf = fork ? P->side : s;
   if (fork) {
     CUDA_TRY(cudaEventRecord(P->ev_fork, s));
     CUDA_TRY(cudaStreamWaitEvent(sf, P->ev_fork, 0));
   }
-  for (int l = 2; l <= L; ++l) {
-    if (P->lev[l].tc || (p2l && l == L)) continue;
-    StageTimer t(P, ST_M2L, sf);
-    if ((st = (l == L && P->m2p) ? do_m2p(P, sf) : do_m2l(P, l, sf))) return st;
+  {
+    int ls[kMaxLevels], n = 0;
+    for (int l = 2; l <= L; ++l)
+      if (!P->lev[l].tc && !(p2l && l == L) && !(l == L && P->m2p)) ls[n++] = l;
+    const std::vector<std::vector<int>> groups = row_groups(P, ls, n);
+    for (const std::vector<int>& gr : groups) {
+      StageTimer t(P, ST_M2L, sf);
+      if ((st = do_m2l_rows(P, gr, sf))) return st;
+    }
+    NbrGemm ng[kZrunGroupMax];
+    int nn = 0;
+    for (int i = 0; i < n && nn < kZrunGroupMax; ++i)
+      if (narrow_level(P, ls[i])) ng[nn++] = m2l_gemm(P, ls[i]);
+    if (nn) {
+      StageTimer t(P, ST_M2L, sf);
+      CUDA_TRY(launch_nbr_gemm_zrun_group(ng, nn, sf));
+    }
+    for (int i = 0, k = 0; i < n; ++i) {
+      if (rows_level(P, ls[i]) || (narrow_level(P, ls[i]) && k++ < nn)) continue;
+      StageTimer t(P, ST_M2L, sf);
+      if ((st = do_m2l(P, ls[i], sf))) return st;
+    }
+    if (P->m2p && !p2l && !P->lev[L].tc) {
+      StageTimer t(P, ST_M2L, sf);
+      if ((st = do_m2p(P, sf))) return st;
+    }
   }
   if (p2l) {
     StageTimer t(P, ST_M2L, sf);
     if ((st = do_p2l(P, sf))) return st;
-  }
-  if (near_side) {
-    StageTimer t(P, ST_NEAR, sf);
-    CUDA_TRY(launch_nbr_gemm<T>(near_gemm(P), sf));
   }
   if (fork) CUDA_TRY(cudaEventRecord(P->ev_join, sf));
   for (int l = 2; l <= L; ++l) {
@@ -2479,7 +2804,7 @@ fmm_status run_solve(fmm_plan_t P, const T* rho, T* phi, T* accel, cudaStream_t 
   } else if (P->near_tc) {
     StageTimer t(P, ST_NEAR_TC, s);
     if ((st = do_near_tc(P, s))) return st;
-  } else if (!near_side) {
+  } else {
     StageTimer t(P, ST_NEAR, s);
     CUDA_TRY(launch_nbr_gemm<T>(near_gemm(P), s));
   }
@@ -2725,9 +3050,20 @@ int fmm_solve_launches(fmm_plan_t P, int with_accel) {
   if (L < 2) n += 1;                    // zero the leaf locals
   for (int l = 2; l <= L; ++l) {
     n += l >= 3 ? 2 : 1;                // M2L, and L2L below level 2
+    if (rows_level(P, l) && !(l == L && P->m2p)) n -= 2;  // grouped: counted below (M2L and its reduction)
     if (l == 2 && harmonic_m2l_level(P, 2)) n += 1;  // rebuild of the harmonic level-2 locals
     if (l == 2 && L == 2 && P->m2p) n += 1;          // zero leaf locals (final-stage M2P, no parent far field)
     if (!P->lev[l].tc && P->m2l_choice[l].dsplit > 1 && !(l == L && P->m2p)) n += 1;  // partial-sum reduction
+  }
+  {
+    int ls[kMaxLevels], k = 0, nn = 0;
+    for (int l = 2; l <= L; ++l)
+      if (!P->lev[l].tc && !(l == L && P->m2p)) {
+        ls[k++] = l;
+        nn += narrow_level(P, l);
+      }
+    n += 2 * (int)row_groups(P, ls, k).size();
+    n -= std::max(0, std::min(nn, kZrunGroupMax) - 1);  // one launch for the narrow levels
   }
   n += P->near_tc ? ((P->near4 && P->use_near4) || tc_prefix(P, TS_NEAR) ? 1 : (int)P->tcn.size()) + 1
                    : 2;  // near field + leaf finish
@@ -2851,6 +3187,7 @@ __device__ __align__(256) unsigned char g_static_workspace[kStaticWorkspaceBytes
 struct StaticSlot {
   unsigned char* ptr = nullptr;
   int key[5] = {-1, -1, -1, -1, -1};
+  std::unique_ptr<fmm_plan_s> plan;  // host side of the grid the array's tables belong to
 };
 StaticSlot g_static_slots[kStaticMaxDevices];
 std::mutex g_static_mutex;
@@ -2889,31 +3226,37 @@ extern "C" fmm_status fmm_solve_static(const fmm_grid* grid, int order, int leaf
       return fail(FMM_ERR_CUDA, "cudaGetSymbolAddress of the static workspace failed: %s", cudaGetErrorString(e));
     if (static_cast<unsigned char*>(addr) != slot.ptr) {  // first call, or a new context: no tables held
       slot.ptr = static_cast<unsigned char*>(addr);
+      slot.plan.reset();
       for (int& k : slot.key) k = -1;
     }
   }
-  std::unique_ptr<fmm_plan_s> P(new (std::nothrow) fmm_plan_s());
-  if (!P) return fail(FMM_ERR_ALLOC, "host allocation failed");
-  P->static_base = slot.ptr;
-  P->static_cap = kStaticWorkspaceBytes;
-  P->no_split = true;  // no neighbour-split scratch
   const int key[5] = {order, leaf, d3[0], d3[1], d3[2]};
-  P->static_keep_tables = std::equal(key, key + 5, slot.key);
-  fmm_opts o;
-  fmm_default_opts(&o);  // FP32 on the CUDA cores
-  o.m2l_cartesian = 1;     // no folded arrays: the workspace limit stays that of the plain contraction
-  fmm_status st = plan_init(P.get(), d3, grid->dx, grid->G, order, leaf, o, s, dev);
-  if (st != FMM_OK) {
-    for (int& k : slot.key) k = -1;  // the tables may be half written
-    return st;
+  if (!slot.plan || !std::equal(key, key + 5, slot.key)) {
+    for (int& k : slot.key) k = -1;  // until the new tables are in place
+    slot.plan.reset(new (std::nothrow) fmm_plan_s());
+    if (!slot.plan) return fail(FMM_ERR_ALLOC, "host allocation failed");
+    slot.plan->static_base = slot.ptr;
+    slot.plan->static_cap = kStaticWorkspaceBytes;
+    slot.plan->no_split = true;  // no neighbour-split scratch
+    fmm_opts o;
+    fmm_default_opts(&o);  // FP32 on the CUDA cores
+    o.m2l_cartesian = 1;     // no folded arrays: the workspace limit stays that of the plain contraction
+    const fmm_status st = plan_init(slot.plan.get(), d3, grid->dx, grid->G, order, leaf, o, s, dev);
+    if (st != FMM_OK) {
+      slot.plan.reset();
+      return st;
+    }
+    std::copy(key, key + 5, slot.key);
   }
-  std::copy(key, key + 5, slot.key);
-  // plan_init cleared the arena; the flag word is kept with the tables
+  fmm_plan_t P = slot.plan.get();
+  P->dx = grid->dx;
+  P->G = grid->G;
+  P->last_stream = s;
+  // clear every part that must start at zero (phantom boxes) and the flag word
+  CUDA_TRY(cudaMemsetAsync(P->arena, 0, P->arena_bytes, s));
   CUDA_TRY(cudaMemsetAsync(P->d_flag, 0, sizeof(int), s));
-  st = run_solve<float>(P.get(), static_cast<const float*>(rho), static_cast<float*>(phi),
-                        static_cast<float*>(accel), s);
   // nothing of P was allocated on the device: no release
-  return st;
+  return run_solve<float>(P, static_cast<const float*>(rho), static_cast<float*>(phi), static_cast<float*>(accel), s);
 }
 
 // ---------------------------------------------------------------------------
@@ -2926,6 +3269,10 @@ struct MultiStep {
   int kind = 0, shape = 0, n = 0, bs = 0, harm_rows = 0;
   long long blocks = 0;
   size_t args_off = 0, grids_off = 0;
+  // MK_GEMM: items and blocks of each kind, in this order (one launch each):
+  // reflection-basis M2L, reflection-basis leaf-4 near field, direct form
+  int kn[3] = {0, 0, 0};
+  long long kb[3] = {0, 0, 0};
 };
 }  // namespace
 
@@ -3045,6 +3392,16 @@ void build_fused(fmm_batch_t B, const void* const* rho, void* const* phi, void* 
   constexpr int bs = 256;  // block size of the tree kernels (M2M, L2L)
   int maxL = 0;
   for (fmm_plan_t P : B->plans) maxL = std::max(maxL, P->L);
+  // The M2L form of a level inside the batch (whatever the plan is tuned to):
+  // the reflection basis, except the levels above the leaf level of FP32
+  // batches.  Their unsplit direct sums carry the largest rounding of a batch,
+  // which the 5-point force amplifies (a change of it shows as 2.2e-5 to
+  // 3.7e-5 of the force, against 5e-6 for the leaf level's): the force would
+  // differ from earlier releases' by more than their FP32 solves of one field
+  // agree in.
+  auto reflect = [&](fmm_plan_t P, int l) {
+    return P->lev[l].fold_off != 0 && !P->lev[l].tc && (P->f64_data() || l == P->L);
+  };
   {  // P2M (and the near field's box-major density)
     std::vector<P2mArgs> a;
     std::vector<std::array<unsigned, 3>> g;
@@ -3061,10 +3418,10 @@ void build_fused(fmm_batch_t B, const void* const* rho, void* const* phi, void* 
       x.Mleaf = P->M(P->L);
       x.rho_box = P->arena + P->rho_box_off;
       x.flag = P->d_flag;
-      x.harm = lf.fold_off ? 1 : 0;
+      x.harm = lf.fold_off ? (reflect(P, P->L) ? 2 : 1) : 0;
       x.Mfold = lf.fold_off ? P->arena + lf.fold_off : nullptr;
       x.ncell = P->ncell();
-      harm_rows |= x.harm;
+      harm_rows |= x.harm ? 1 : 0;
       a.push_back(x);
       g.push_back(blocks_1d(lf.npar * 16, 256));
     }
@@ -3082,7 +3439,7 @@ void build_fused(fmm_batch_t B, const void* const* rho, void* const* phi, void* 
       x.Mc = P->M(l);
       x.par = q;
       x.Mp = P->M(l - 1);
-      x.harm = q.fold_off ? 1 : 0;
+      x.harm = q.fold_off ? (reflect(P, l - 1) ? 2 : 1) : 0;
       x.Mfold = q.fold_off ? P->arena + q.fold_off : nullptr;
       a.push_back(x);
       g.push_back(blocks_1d(c.npar * 8, bs));
@@ -3090,8 +3447,8 @@ void build_fused(fmm_batch_t B, const void* const* rho, void* const* phi, void* 
     add_step(B, MK_M2M, 0, bs, 0, a, g);
   }
   {  // M2L of every level and the near field: independent contractions
-    std::vector<NbrGemm> a[6];
-    std::vector<std::array<unsigned, 3>> g[6];
+    std::vector<NbrGemm> a[6][3];
+    std::vector<std::array<unsigned, 3>> g[6][3];
     auto add = [&](NbrGemm x, const std::vector<int>& tile_k) {
       x.dsplit = 1;  // the batch fills the GPU: no neighbour split, no partial sums
       x.partial = nullptr;
@@ -3106,14 +3463,32 @@ void build_fused(fmm_batch_t B, const void* const* rho, void* const* phi, void* 
         nbr_gemm_zrun_grid<T>(x, x.shape - 1, gr.data());
       else
         nbr_gemm_simt_col_grid<T>(x, gr.data());
-      a[x.shape].push_back(x);
-      g[x.shape].push_back(gr);
+      const int kind = x.sym == kSymM2l ? 0 : x.sym == kSymNear4 && (x.shape == 1 || x.shape == 5) ? 1 : 2;
+      a[x.shape][kind].push_back(x);
+      g[x.shape][kind].push_back(gr);
     };
     for (fmm_plan_t P : B->plans) {
-      for (int l = 2; l <= P->L; ++l) add(m2l_gemm(P, l), P->h_m2l_tile_k);
+      for (int l = 2; l <= P->L; ++l) add(m2l_gemm(P, l, reflect(P, l) ? 1 : 0), P->h_m2l_tile_k);
       add(near_gemm(P), P->h_near_tile_k);
     }
-    for (int sh : {1, 5, 0, 2, 3, 4}) add_step(B, MK_GEMM, sh, 0, 0, a[sh], g[sh]);  // the tiny-grid launch last
+    for (int sh : {1, 5, 0, 2, 3, 4}) {  // the tiny-grid launch last
+      std::vector<NbrGemm> all;
+      std::vector<std::array<unsigned, 3>> ag;
+      for (int k = 0; k < 3; ++k) {
+        all.insert(all.end(), a[sh][k].begin(), a[sh][k].end());
+        ag.insert(ag.end(), g[sh][k].begin(), g[sh][k].end());
+      }
+      const size_t before = B->steps.size();
+      add_step(B, MK_GEMM, sh, 0, 0, all, ag);
+      if (B->steps.size() == before) continue;
+      MultiStep& st = B->steps.back();
+      for (int k = 0; k < 3; ++k)
+        for (const std::array<unsigned, 3>& x : g[sh][k]) {
+          const long long nb = (long long)x[0] * x[1] * x[2];
+          st.kn[k] += nb > 0;
+          st.kb[k] += nb;
+        }
+    }
   }
   for (int l = 2; l <= maxL; ++l) {  // L2L, coarse to fine (a fused leaf level's in the leaf kernel)
     std::vector<L2lArgs> a;
@@ -3225,16 +3600,24 @@ fmm_status run_fused(fmm_batch_t B, cudaStream_t s) {
         break;
       case MK_GEMM: {
         const NbrGemm* gs = static_cast<const NbrGemm*>(a);
+        const int zs = st.shape == 5 ? 2 : st.shape == 4 ? 3 : st.shape - 1;
+        for (int k = 0; k < 2 && e == cudaSuccess; ++k) {  // reflection-basis items: M2L, near field
+          e = launch_nbr_gemm_sym_multi<T>(zs, k == 0 ? kSymM2l : kSymNear4, gs, g, st.kn[k], st.kb[k],
+                                           k == 0 ? 0 : st.kb[0], ls);
+          gs += st.kn[k];
+          g += st.kn[k];
+        }
+        if (e != cudaSuccess) break;
+        const int n = st.kn[2];  // direct form
+        const long long nb = st.kb[2], first = st.kb[0] + st.kb[1];
         if (st.shape == 4)
-          e = launch_nbr_gemm_tiny_multi<T>(gs, g, st.n, st.blocks, ls);
+          e = launch_nbr_gemm_tiny_multi<T>(gs, g, n, nb, ls, first);
         else if (st.shape == 0)
-          e = launch_nbr_gemm_simt_multi<T>(gs, g, st.n, st.blocks, ls);
+          e = launch_nbr_gemm_simt_multi<T>(gs, g, n, nb, ls);
         else if (st.shape == 3)
-          e = launch_nbr_gemm_col_multi<T>(gs, g, st.n, st.blocks, ls);
-        else if (st.shape == 5)
-          e = launch_nbr_gemm_zrun_multi<T>(2, gs, g, st.n, st.blocks, ls);
+          e = launch_nbr_gemm_col_multi<T>(gs, g, n, nb, ls);
         else
-          e = launch_nbr_gemm_zrun_multi<T>(st.shape - 1, gs, g, st.n, st.blocks, ls);
+          e = launch_nbr_gemm_zrun_multi<T>(zs, gs, g, n, nb, ls, first);
         break;
       }
       case MK_L2L:
@@ -3491,16 +3874,19 @@ bool choice_valid(fmm_plan_t P, NbrGemm g, const std::vector<int>& tk, size_t es
   // share an SM with a tensor-core CTA
   if ((c.shape == 1 || c.shape == 2) && es == 8 && P->tc_kind >= 0) return false;
   const size_t one = (size_t)g.grid[0] * g.grid[1] * g.grid[2] * (size_t)g.n_cols * es;
-  if (c.dsplit > 1 && (size_t)c.dsplit * one > P->part_cap) return false;
+  const size_t cap = g.partial == P->arena + P->near_part_off && P->near_part_cap ? P->near_part_cap : P->part_cap;
+  if (c.dsplit > 1 && (size_t)c.dsplit * one > cap) return false;
   if (c.shape == 0 || c.shape == 3) return c.dsplit == 1 || c.dsplit == 27;
   if (c.shape != 1 && c.shape != 2) return false;
   g.dsplit = c.dsplit;
   return zrun_eligible(g, tk.data(), (int)tk.size());
 }
 
-template <typename T>
-fmm_status tune_one(fmm_plan_t P, NbrGemm g, const std::vector<int>& tk, const char* what, int reps, cudaStream_t s,
-                    SimtChoice* out) {
+// make(): the contraction as the plan runs it with its current choice *out.
+template <typename T, typename Make>
+fmm_status tune_one(fmm_plan_t P, const Make& make, const std::vector<int>& tk, const char* what, int reps,
+                    cudaStream_t s, SimtChoice* out) {
+  NbrGemm g = make();
   char key[160];
   std::snprintf(key, sizeof key, "%s/%zu/%d,%d,%d/%d/%d/%d/%d/%d", what, sizeof(T), g.grid[0], g.grid[1], g.grid[2],
                 g.row_len, g.n_cols, g.ntiles, P->p, P->b);
@@ -3524,10 +3910,11 @@ fmm_status tune_one(fmm_plan_t P, NbrGemm g, const std::vector<int>& tk, const c
   }
   fmm_status st = FMM_OK;
   float best = 1e30f;
-  SimtChoice pick = *out;
+  const SimtChoice old = *out;
+  SimtChoice pick = old;
   for (const SimtChoice& c : cand) {
-    g.shape = c.shape;
-    g.dsplit = c.dsplit;
+    *out = c;
+    g = make();
     cudaError_t e = launch_nbr_gemm<T>(g, s);  // warm-up
     if (e == cudaSuccess) e = cudaEventRecord(e0, s);
     for (int r = 0; r < reps && e == cudaSuccess; ++r) e = launch_nbr_gemm<T>(g, s);
@@ -3543,8 +3930,8 @@ fmm_status tune_one(fmm_plan_t P, NbrGemm g, const std::vector<int>& tk, const c
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
+  *out = st == FMM_OK ? pick : old;
   if (st != FMM_OK) return st;
-  *out = pick;
   std::lock_guard<std::mutex> lk(g_tune_mu);
   g_tune_cache[key] = pick;
   return FMM_OK;
@@ -3626,15 +4013,15 @@ extern "C" fmm_status fmm_plan_autotune(fmm_plan_t P, void* stream) {
   fmm_status st;
   for (int l = 2; l <= P->L; ++l) {
     if (P->lev[l].tc) continue;
-    const NbrGemm g = m2l_gemm(P, l);
-    st = P->lev[l].f64 ? tune_one<double>(P, g, P->h_m2l_tile_k, "m2l", 3, s, &P->m2l_choice[l])
-                       : tune_one<float>(P, g, P->h_m2l_tile_k, "m2l", 3, s, &P->m2l_choice[l]);
+    auto make = [P, l] { return m2l_gemm(P, l); };
+    st = P->lev[l].f64 ? tune_one<double>(P, make, P->h_m2l_tile_k, "m2l", 3, s, &P->m2l_choice[l])
+                       : tune_one<float>(P, make, P->h_m2l_tile_k, "m2l", 3, s, &P->m2l_choice[l]);
     if (st) return st;
   }
   if (!P->near_tc) {
-    const NbrGemm g = near_gemm(P);
-    st = P->f64_data() ? tune_one<double>(P, g, P->h_near_tile_k, "near", 3, s, &P->near_choice)
-                       : tune_one<float>(P, g, P->h_near_tile_k, "near", 3, s, &P->near_choice);
+    auto make = [P] { return near_gemm(P); };
+    st = P->f64_data() ? tune_one<double>(P, make, P->h_near_tile_k, "near", 3, s, &P->near_choice)
+                       : tune_one<float>(P, make, P->h_near_tile_k, "near", 3, s, &P->near_choice);
     if (st) return st;
   }
   for (int what = 0; what < 3; ++what)

@@ -54,8 +54,9 @@ struct Level {
   size_t bytes;    // bytes of one of the two arrays
   int tc;          // M2L of this level on the tensor cores
   size_t hi_off, lo_off;  // bf16 hi / lo planes of the multipoles (tensor-core bf16x3 levels)
-  // CUDA-core harmonic M2L: folded multipoles and the M2L's c <= 1 locals,
-  // rows of 8 (p+1)^2 values in the level's type (0: none)
+  // CUDA-core harmonic M2L: folded multipoles ([8 (p+1)^2][parents]) and the
+  // M2L's c <= 1 locals (rows of 8 (p+1)^2 values), in the level's type; TF32
+  // levels: folded rows (0: none)
   size_t fold_off, lred_off;
 };
 
@@ -65,6 +66,24 @@ struct MultiGrid {
   unsigned gx, gy, gz, pad;
   long long start;
 };
+
+// Reflection-basis form of an M2L contraction (k_sym.cu): components alpha /
+// beta in one order (by total order), output columns in units of 8.
+constexpr int kSymMaxK = 81;      // (p + 1)^2 at p = 8
+constexpr int kSymMaxUnits = 11;
+struct SymTab {
+  int nk, nunits;
+  // unit u: components [0, n8) feed its 8 columns, [n8, n4) at most the first
+  // four, [n4, n1) the first one (columns run over increasing order, so the
+  // live ones are a prefix that shrinks with alpha)
+  int n8[kSymMaxUnits], n4[kSymMaxUnits], n1[kSymMaxUnits];
+  long long w_off[kSymMaxUnits];  // unit's weights in Ws: [alpha][9 (x, y) pairs][4 signs][3 z pairs][columns][2]
+  int kb[kSymMaxK];               // components that reach column beta
+  int q_off[kSymMaxK];            // alpha's block in Wq: [27 triples][alpha][beta (multiple of 4)][8 blocks]
+  int q_len;                      // values of one triple
+  unsigned char par[kSymMaxK];    // bit q: odd along axis q
+};
+enum SymKind { kSymNone = 0, kSymM2l = 1, kSymNear4 = 2 };
 
 // Neighbour-contraction ("implicit GEMM") description for the SIMT kernel:
 //   C[row][n] (+)= sum_{d in 27 neighbours} sum_{k < K(tile(n))} A[row + d][k] * W_d[k][n]
@@ -88,7 +107,44 @@ struct NbrGemm {
   int max_blocks = 0;  // shape 0: at most this many CTAs, each looping over work items (0: one per item)
   int skip_center = 0; // 1: W_d of the centre neighbour (d = 13) is all zero (the M2L: a parent's
                        // children are each other's near neighbours), and the kernels skip it
+  // reflection-basis form (k_sym.cu), SymKind.  kSymM2l: A is component-major,
+  // [8 alpha + child][lda rows]; kSymNear4: A as above
+  int sym = 0;
+  const SymTab* st = nullptr;  // device
+  const void* Ws = nullptr;
+  const void* Wq = nullptr;
+  int q_len = 0;  // SymTab::q_len
+  long long lda = 0;
 };
+
+template <typename T>
+cudaError_t launch_nbr_gemm_sym(const NbrGemm& g, cudaStream_t s);
+// Several FP32 contractions on the 8 x 4 x 8 z-run tiles, unsplit, in one launch
+// of the narrow form (k_gemm_zrun.cu), which pays below kZrunNarrowBlocks
+// blocks of the wide one.
+constexpr int kZrunGroupMax = 8;
+constexpr long long kZrunNarrowBlocks = 8 * 152;
+cudaError_t launch_nbr_gemm_zrun_group(const NbrGemm* gs, int n, cudaStream_t s);
+// Few rows, FP32, split over the 27 neighbours (k_gemm_rows.cu): up to
+// kRowsGroupMax levels of one plan in one launch, each with its own scratch
+// for the partial sums; the sums of the simt kernel, bit for bit.
+constexpr int kRowsGroupMax = 8;
+cudaError_t launch_nbr_gemm_rows(const NbrGemm* gs, int n, cudaStream_t s);
+// Whether that kernel takes this contraction (dsplit 27, reduction lengths
+// and column counts multiples of 8).
+bool nbr_gemm_rows_fits(const NbrGemm& g, const int* tile_k_host, int ntiles);
+
+// The reflection-basis row form (shapes 0 and 3) over up to kSymGroupMax levels of one plan in
+// one launch, same shape and split, each with its own scratch for the partial sums.
+// (FP64.)
+constexpr int kSymGroupMax = 8;
+cudaError_t launch_nbr_gemm_sym_rows(const NbrGemm* gs, int n, cudaStream_t s);
+// Multi-item forms over the items of one kind: blocks [first, first + blocks)
+// of the step's block ranges.  shape as launch_nbr_gemm_zrun_multi, or 3: the
+// tiny-grid form (at most 64 rows, one block per 32 columns; kSymM2l only).
+template <typename T>
+cudaError_t launch_nbr_gemm_sym_multi(int shape, int kind, const NbrGemm* gs, const MultiGrid* grids, int n,
+                                      long long blocks, long long first, cudaStream_t s);
 
 template <typename T>
 cudaError_t launch_nbr_gemm_simt(const NbrGemm& g, cudaStream_t s);
@@ -104,7 +160,8 @@ cudaError_t launch_nbr_gemm(const NbrGemm& g, cudaStream_t s);
 // Multi-item forms (multi.cuh) for items of one shape with dsplit 1 (no
 // partial sums): gs / grids are device arrays of n items; *_grid gives an
 // item's grid (shape 0 / 3: nbr_gemm_simt_col_grid, shapes 1 / 2:
-// nbr_gemm_zrun_grid with shape - 1).
+// nbr_gemm_zrun_grid with shape - 1).  first: block offset of the launch in
+// the items' block ranges.
 template <typename T>
 cudaError_t launch_nbr_gemm_simt_multi(const NbrGemm* gs, const MultiGrid* grids, int n, long long blocks,
                                        cudaStream_t s);
@@ -114,7 +171,7 @@ cudaError_t launch_nbr_gemm_col_multi(const NbrGemm* gs, const MultiGrid* grids,
 // shape here: 0 / 1 as launch_nbr_gemm_zrun, 2 = a z run of 6 rows (FP32; 3 in FP64)
 template <typename T>
 cudaError_t launch_nbr_gemm_zrun_multi(int shape, const NbrGemm* gs, const MultiGrid* grids, int n, long long blocks,
-                                       cudaStream_t s);
+                                       cudaStream_t s, long long first = 0);
 template <typename T>
 void nbr_gemm_simt_col_grid(const NbrGemm& g, unsigned out[3]);
 // Grids of at most 64 rows (nbr_gemm_tiny_fits): one block per column tile
@@ -122,7 +179,7 @@ void nbr_gemm_simt_col_grid(const NbrGemm& g, unsigned out[3]);
 bool nbr_gemm_tiny_fits(const NbrGemm& g);
 template <typename T>
 cudaError_t launch_nbr_gemm_tiny_multi(const NbrGemm* gs, const MultiGrid* grids, int n, long long blocks,
-                                       cudaStream_t s);
+                                       cudaStream_t s, long long first = 0);
 template <typename T>
 void nbr_gemm_zrun_grid(const NbrGemm& g, int shape, unsigned out[3]);
 // C (+)= sum over nparts partial arrays of count values, in part order.
@@ -145,7 +202,8 @@ struct TreeTables {
 // harm = 1: the planes hold the harmonic ((p+1)^2, c <= 1) components of the
 // folded multipoles (tree_common.cuh), rows of 8 (p+1)^2 values per parent.
 // Mfold (nullable, with harm): the folded components in the level's type,
-// rows of 8 (p+1)^2 values (the CUDA-core harmonic M2L reads them).
+// rows of 8 (p+1)^2 values (TF32 levels) or, with harm = 2, component-major
+// [8 r + child][parent] (the CUDA-core harmonic M2L, k_sym.cu).
 // dip (nullable): dipole sources [3][cells], weights v_q adding v_q d/de_q (e^alpha)
 // (box units) per cell -- the transpose of the analytic force's L2P gradient.
 template <typename T>

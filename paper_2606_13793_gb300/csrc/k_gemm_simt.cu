@@ -321,12 +321,13 @@ __device__ __forceinline__ void nbr_gemm_tiny_body(const NbrGemm& g, const VBloc
 template <typename T>
 __global__ void __launch_bounds__(kTinyThreads) nbr_gemm_tiny_multi_kernel(const NbrGemm* __restrict__ gs,
                                                                            const MultiGrid* __restrict__ grids,
-                                                                           int n) {
+                                                                           int n, long long first) {
   __shared__ NbrGemm g;  // the item's description, read by the body from shared memory
-  const int i = multi_item(grids, n);
+  const long long b = (long long)blockIdx.x + first;
+  const int i = multi_item_at(grids, n, b);
   if (threadIdx.x == 0) g = gs[i];
   __syncthreads();
-  nbr_gemm_tiny_body<T>(g, multi_vblock(grids[i]));
+  nbr_gemm_tiny_body<T>(g, multi_vblock_at(grids[i], b));
 }
 
 // C (+)= sum over the neighbour-group partials, in group order.
@@ -366,6 +367,7 @@ cudaError_t launch_nbr_gemm_col(const NbrGemm& g, cudaStream_t s) {
 
 template <typename T>
 cudaError_t launch_nbr_gemm(const NbrGemm& g, cudaStream_t s) {
+  if (g.sym == kSymM2l || (g.sym == kSymNear4 && (g.shape == 1 || g.shape == 2))) return launch_nbr_gemm_sym<T>(g, s);
   if (g.shape == 3) return launch_nbr_gemm_col<T>(g, s);
   return g.shape == 0 ? launch_nbr_gemm_simt<T>(g, s) : launch_nbr_gemm_zrun<T>(g, g.shape - 1, s);
 }
@@ -377,6 +379,9 @@ cudaError_t launch_nbr_gemm_simt(const NbrGemm& g, cudaStream_t s) {
   long long items = tiles * g.ntiles * (g.dsplit > 1 ? 27 : 1);
   if (g.max_blocks > 0 && items > g.max_blocks) items = g.max_blocks;
   if (items > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+  if constexpr (sizeof(T) == 4) {  // reduction lengths and columns are multiples of 8 (8 children, or b^3 cells)
+    if (g.dsplit == 27 && g.max_blocks == 0) return launch_nbr_gemm_rows(&g, 1, s);
+  }
   nbr_gemm_simt_kernel<T><<<(unsigned)items, 64, 0, s>>>(g);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || g.dsplit <= 1) return e;
@@ -406,10 +411,10 @@ cudaError_t launch_nbr_gemm_col_multi(const NbrGemm* gs, const MultiGrid* grids,
 
 template <typename T>
 cudaError_t launch_nbr_gemm_tiny_multi(const NbrGemm* gs, const MultiGrid* grids, int n, long long blocks,
-                                       cudaStream_t s) {
+                                       cudaStream_t s, long long first) {
   if (n <= 0 || blocks <= 0) return cudaSuccess;
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  nbr_gemm_tiny_multi_kernel<T><<<(unsigned)blocks, kTinyThreads, 0, s>>>(gs, grids, n);
+  nbr_gemm_tiny_multi_kernel<T><<<(unsigned)blocks, kTinyThreads, 0, s>>>(gs, grids, n, first);
   return cudaGetLastError();
 }
 
@@ -434,8 +439,10 @@ template cudaError_t launch_nbr_gemm_simt_multi<float>(const NbrGemm*, const Mul
 template cudaError_t launch_nbr_gemm_simt_multi<double>(const NbrGemm*, const MultiGrid*, int, long long, cudaStream_t);
 template cudaError_t launch_nbr_gemm_col_multi<float>(const NbrGemm*, const MultiGrid*, int, long long, cudaStream_t);
 template cudaError_t launch_nbr_gemm_col_multi<double>(const NbrGemm*, const MultiGrid*, int, long long, cudaStream_t);
-template cudaError_t launch_nbr_gemm_tiny_multi<float>(const NbrGemm*, const MultiGrid*, int, long long, cudaStream_t);
-template cudaError_t launch_nbr_gemm_tiny_multi<double>(const NbrGemm*, const MultiGrid*, int, long long, cudaStream_t);
+template cudaError_t launch_nbr_gemm_tiny_multi<float>(const NbrGemm*, const MultiGrid*, int, long long, cudaStream_t,
+                                                       long long);
+template cudaError_t launch_nbr_gemm_tiny_multi<double>(const NbrGemm*, const MultiGrid*, int, long long, cudaStream_t,
+                                                        long long);
 template void nbr_gemm_simt_col_grid<float>(const NbrGemm&, unsigned[3]);
 template void nbr_gemm_simt_col_grid<double>(const NbrGemm&, unsigned[3]);
 template cudaError_t launch_nbr_gemm_simt<float>(const NbrGemm&, cudaStream_t);

@@ -221,16 +221,154 @@ __global__ void __launch_bounds__(kZrThreads, 4) nbr_gemm_zrun_kernel(NbrGemm g)
 
 template <typename T, int RZ>
 __global__ void __launch_bounds__(kZrThreads, 4) nbr_gemm_zrun_multi_kernel(const NbrGemm* __restrict__ gs,
-                                                                         const MultiGrid* __restrict__ grids, int n) {
+                                                                         const MultiGrid* __restrict__ grids, int n,
+                                                                         long long first) {
   __shared__ NbrGemm g;  // the item's description, read by the body from shared memory
-  const int i = multi_item(grids, n);
+  const long long b = (long long)blockIdx.x + first;
+  const int i = multi_item_at(grids, n, b);
   if (threadIdx.x == 0) g = gs[i];
   __syncthreads();
-  nbr_gemm_zrun_body<T, RZ>(g, multi_vblock(grids[i]));
+  nbr_gemm_zrun_body<T, RZ>(g, multi_vblock_at(grids[i], b));
+}
+
+// Narrow form (FP32), for launches whose blocks do not fill the GPU (the
+// coarse levels of a batch, the levels of the allocation-free solve): a block's 8 x 4 x RZ rows x 32 columns go to four CTAs of
+// 8 columns, a thread takes RZ / 2 rows x 4 columns, and the next stage's
+// operands are loaded while the current one is multiplied.  A lone 128-thread
+// CTA of the wide form needs 0.8 ms for the 10584 products of an order-6 M2L
+// output (64 outputs a thread, 4 warps on the SM), this one ~0.15 ms; filled,
+// the wide form is the faster one (34 shared-memory values per 192 products
+// against 18 per 48).  Every output adds the same products in the same order
+// as the wide form: the results are its, bit for bit.
+template <int RZ>
+__device__ __forceinline__ void zrun_narrow_body(const NbrGemm& g, const VBlock& vb, int cg) {
+  using H = ZrHalo<RZ>;
+  constexpr int HR = RZ / 2;
+  constexpr int kA = (H::rows * 2 + kZrThreads - 1) / kZrThreads;  // float4 of A per thread and stage
+  constexpr int kW = (27 * kZrKC * 2 + kZrThreads - 1) / kZrThreads;
+  __shared__ __align__(16) float As[kZrKC * H::stride];
+  __shared__ __align__(16) float Ws[27 * kZrKC * 8];
+  const int t = threadIdx.x;
+  const int xr = t & 7, yr = (t >> 3) & 3, zh = (t >> 5) & 1, cq = t >> 6;
+  const int ntx = (g.grid[0] + kZrBX - 1) / kZrBX, nty = (g.grid[1] + kZrBY - 1) / kZrBY;
+  const int bt = vb.x;
+  const int ox = (bt % ntx) * kZrBX, oy = ((bt / ntx) % nty) * kZrBY, oz = (bt / (ntx * nty)) * RZ;
+  const int tile = vb.y, K = g.tile_k[tile];
+  if (tile * kNTile + cg * 8 >= g.n_cols) return;  // a multiple of 8
+  const float* W0 = static_cast<const float*>(g.W) + g.tile_w[tile] + cg * 8;
+  const float* A = static_cast<const float*>(g.A);
+  long long ao[kA];  // source of each A piece (-1: zero)
+#pragma unroll
+  for (int i = 0; i < kA; ++i) {
+    const int e = t + i * kZrThreads, h = e >> 1;
+    const int x = ox + h % H::hx - 1, y = oy + (h / H::hx) % H::hy - 1, z = oz + h / (H::hx * H::hy) - 1;
+    ao[i] = (h < H::rows && x >= 0 && y >= 0 && z >= 0 && x < g.grid[0] && y < g.grid[1] && z < g.grid[2])
+                ? (((long long)z * g.grid[1] + y) * g.grid[0] + x) * g.row_len + (e & 1) * 4
+                : -1;
+  }
+  float4 ra[kA], rw[kW];
+  auto fetch = [&](int kc) {
+#pragma unroll
+    for (int i = 0; i < kA; ++i)
+      ra[i] = ao[i] >= 0 ? __ldg(reinterpret_cast<const float4*>(A + ao[i] + kc)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < kW; ++i) {
+      const int e = t + i * kZrThreads;  // [neighbour][k][half]
+      if (e < 27 * kZrKC * 2)
+        rw[i] = __ldg(reinterpret_cast<const float4*>(W0 + ((long long)(e >> 4) * K + kc + ((e >> 1) & 7)) * kNTile +
+                                                      (e & 1) * 4));
+    }
+  };
+  unsigned long long acc[HR][2];
+#pragma unroll
+  for (int z = 0; z < HR; ++z) acc[z][0] = acc[z][1] = 0ull;
+  if (K > 0) fetch(0);
+  for (int kc = 0; kc < K; kc += kZrKC) {
+    __syncthreads();  // the previous stage is read
+#pragma unroll
+    for (int i = 0; i < kA; ++i) {
+      const int e = t + i * kZrThreads, h = e >> 1, q = (e & 1) * 4;
+      if (h < H::rows) {
+        As[q * H::stride + h] = ra[i].x;
+        As[(q + 1) * H::stride + h] = ra[i].y;
+        As[(q + 2) * H::stride + h] = ra[i].z;
+        As[(q + 3) * H::stride + h] = ra[i].w;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kW; ++i) {
+      const int e = t + i * kZrThreads;
+      if (e < 27 * kZrKC * 2) *reinterpret_cast<float4*>(Ws + e * 4) = rw[i];
+    }
+    __syncthreads();
+    if (kc + kZrKC < K) fetch(kc + kZrKC);
+    for (int xy = 0; xy < 9; ++xy) {
+      const float* Ab = As + (zh * HR * H::hy + yr + xy / 3) * H::hx + (xr + xy % 3);
+      const float* Wb = Ws + xy * kZrKC * 8 + cq * 4;
+#pragma unroll
+      for (int k = 0; k < kZrKC; ++k) {
+        unsigned long long a2[HR + 2];
+#pragma unroll
+        for (int z = 0; z < HR + 2; ++z) a2[z] = f2_splat(Ab[k * H::stride + z * H::hx * H::hy]);
+#pragma unroll
+        for (int dz = 0; dz < 3; ++dz) {
+          if (dz == 1 && xy == 4 && g.skip_center) continue;  // the centre block is zero
+          const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(Wb + (dz * 9 * kZrKC + k) * 8);
+#pragma unroll
+          for (int z = 0; z < HR; ++z) {
+            acc[z][0] = f2_fma(a2[z + dz], w.x, acc[z][0]);
+            acc[z][1] = f2_fma(a2[z + dz], w.y, acc[z][1]);
+          }
+        }
+      }
+    }
+  }
+  const int x = ox + xr, y = oy + yr;
+  if (x >= g.grid[0] || y >= g.grid[1]) return;
+#pragma unroll
+  for (int z = 0; z < HR; ++z) {
+    const int zz = oz + zh * HR + z;
+    if (zz >= g.grid[2]) break;
+    const float2 u = f2_unpack(acc[z][0]), v = f2_unpack(acc[z][1]);
+    float4* o = reinterpret_cast<float4*>(static_cast<float*>(g.C) +
+                                          (((long long)zz * g.grid[1] + y) * g.grid[0] + x) * g.n_cols +
+                                          tile * kNTile + cg * 8 + cq * 4);
+    float4 r = make_float4(u.x, u.y, v.x, v.y);
+    if (g.accumulate) {
+      const float4 old = *o;
+      r.x = old.x + r.x, r.y = old.y + r.y, r.z = old.z + r.z, r.w = old.w + r.w;
+    }
+    *o = r;
+  }
+}
+
+template <int RZ>
+__global__ void __launch_bounds__(kZrThreads) zrun_narrow_multi_kernel(const NbrGemm* __restrict__ gs,
+                                                                       const MultiGrid* __restrict__ grids, int n,
+                                                                       long long first) {
+  __shared__ NbrGemm g;
+  const long long b = (long long)(blockIdx.x >> 2) + first;
+  const int it = multi_item_at(grids, n, b);
+  if (threadIdx.x == 0) g = gs[it];
+  __syncthreads();
+  zrun_narrow_body<RZ>(g, multi_vblock_at(grids[it], b), blockIdx.x & 3);
+}
+
+// A few contractions by value (blocks of item i: [grids[i].start, ...)).
+struct ZrunGroup {
+  NbrGemm g[kZrunGroupMax];
+  MultiGrid grids[kZrunGroupMax];
+  int n;
+};
+__global__ void __launch_bounds__(kZrThreads) zrun_narrow_group_kernel(const __grid_constant__ ZrunGroup G) {
+  const long long b = blockIdx.x >> 2;
+  const int it = multi_item_at(G.grids, G.n, b);
+  zrun_narrow_body<8>(G.g[it], multi_vblock_at(G.grids[it], b), blockIdx.x & 3);
 }
 
 template <typename T, int RZ>
-cudaError_t launch_rz_multi(const NbrGemm* gs, const MultiGrid* grids, int n, long long blocks, cudaStream_t s) {
+cudaError_t launch_rz_multi(const NbrGemm* gs, const MultiGrid* grids, int n, long long blocks, cudaStream_t s,
+                            long long first) {
   constexpr size_t smem = zrun_smem_bytes<T, RZ>();
   static bool attr = false;
   if (!attr) {
@@ -241,7 +379,13 @@ cudaError_t launch_rz_multi(const NbrGemm* gs, const MultiGrid* grids, int n, lo
   }
   if (n <= 0 || blocks <= 0) return cudaSuccess;
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  nbr_gemm_zrun_multi_kernel<T, RZ><<<(unsigned)blocks, kZrThreads, smem, s>>>(gs, grids, n);
+  if constexpr (sizeof(T) == 4 && RZ % 2 == 0) {
+    if (blocks < kZrunNarrowBlocks) {  // under two waves of four CTAs per SM
+      zrun_narrow_multi_kernel<RZ><<<(unsigned)(4 * blocks), kZrThreads, 0, s>>>(gs, grids, n, first);
+      return cudaGetLastError();
+    }
+  }
+  nbr_gemm_zrun_multi_kernel<T, RZ><<<(unsigned)blocks, kZrThreads, smem, s>>>(gs, grids, n, first);
   return cudaGetLastError();
 }
 
@@ -306,18 +450,41 @@ void nbr_gemm_zrun_grid(const NbrGemm& g, int shape, unsigned out[3]) {
 
 template <typename T>
 cudaError_t launch_nbr_gemm_zrun_multi(int shape, const NbrGemm* gs, const MultiGrid* grids, int n, long long blocks,
-                                       cudaStream_t s) {
-  return shape == 0   ? launch_rz_multi<T, zrun_rz<T>(0)>(gs, grids, n, blocks, s)
-         : shape == 1 ? launch_rz_multi<T, zrun_rz<T>(1)>(gs, grids, n, blocks, s)
-                      : launch_rz_multi<T, zrun_rz<T>(2)>(gs, grids, n, blocks, s);
+                                       cudaStream_t s, long long first) {
+  return shape == 0   ? launch_rz_multi<T, zrun_rz<T>(0)>(gs, grids, n, blocks, s, first)
+         : shape == 1 ? launch_rz_multi<T, zrun_rz<T>(1)>(gs, grids, n, blocks, s, first)
+                      : launch_rz_multi<T, zrun_rz<T>(2)>(gs, grids, n, blocks, s, first);
+}
+
+cudaError_t launch_nbr_gemm_zrun_group(const NbrGemm* gs, int n, cudaStream_t s) {
+  if (n < 1 || n > kZrunGroupMax) return cudaErrorInvalidValue;
+  ZrunGroup G{};
+  long long blocks = 0;
+  for (int i = 0; i < n; ++i) {
+    unsigned gr[3];
+    nbr_gemm_zrun_grid<float>(gs[i], 0, gr);
+    const long long nb = (long long)gr[0] * gr[1] * gr[2];
+    if (gs[i].dsplit != 1) return cudaErrorInvalidValue;
+    if (nb <= 0) continue;
+    G.g[G.n] = gs[i];
+    G.grids[G.n].gx = gr[0];
+    G.grids[G.n].gy = gr[1];
+    G.grids[G.n].gz = gr[2];
+    G.grids[G.n++].start = blocks;
+    blocks += nb;
+  }
+  if (G.n == 0) return cudaSuccess;
+  if (blocks > 0x1fffffffLL) return cudaErrorInvalidConfiguration;
+  zrun_narrow_group_kernel<<<(unsigned)(4 * blocks), kZrThreads, 0, s>>>(G);
+  return cudaGetLastError();
 }
 
 template void nbr_gemm_zrun_grid<float>(const NbrGemm&, int, unsigned[3]);
 template void nbr_gemm_zrun_grid<double>(const NbrGemm&, int, unsigned[3]);
 template cudaError_t launch_nbr_gemm_zrun_multi<float>(int, const NbrGemm*, const MultiGrid*, int, long long,
-                                                       cudaStream_t);
+                                                       cudaStream_t, long long);
 template cudaError_t launch_nbr_gemm_zrun_multi<double>(int, const NbrGemm*, const MultiGrid*, int, long long,
-                                                        cudaStream_t);
+                                                        cudaStream_t, long long);
 template cudaError_t launch_nbr_gemm_zrun<float>(const NbrGemm&, int, cudaStream_t);
 template cudaError_t launch_nbr_gemm_zrun<double>(const NbrGemm&, int, cudaStream_t);
 

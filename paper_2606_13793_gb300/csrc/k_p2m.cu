@@ -21,6 +21,14 @@ using namespace tree;
 // body instantiated for it, so every register index stays compile-time.
 constexpr int kP2mParents = kThreads / 16;  // 2 threads per box, 8 boxes per parent
 
+// Staged pitch of the folded rows that are written component-major: 10 mod 32
+// values, so that 16 parents' values of one component (read together) lie in
+// different banks.
+template <int P>
+__host__ __device__ constexpr int p2m_fold_pitch() {
+  return 8 * nred_c(P) + (42 - (8 * nred_c(P)) % 32) % 32;
+}
+
 template <int P>
 __host__ __device__ constexpr int ncoef_parity(int h) {
   int n = 0;
@@ -33,7 +41,7 @@ __host__ __device__ constexpr int ncoef_parity(int h) {
 // v_q d/de_q (e^alpha) (box units) to the monomial moments of its density.
 template <int P, typename T, int h, bool DIP>
 __device__ __forceinline__ void p2m_body(const Box& B, const T* __restrict__ rho, int nx, int ny, int b,
-                                         const Level& leaf, T* __restrict__ Ms, T* __restrict__ Mr,
+                                         const Level& leaf, T* __restrict__ Ms, T* __restrict__ Mr, int rp,
                                          T* __restrict__ rho_box, __nv_bfloat16* __restrict__ rhi,
                                          __nv_bfloat16* __restrict__ rlo, int* __restrict__ flag,
                                          const T* __restrict__ dip, long long ncell) {
@@ -197,7 +205,6 @@ __device__ __forceinline__ void p2m_body(const Box& B, const T* __restrict__ rho
   if (Mr) {
     // harmonic planes: this thread's parity class folds onto c = h (the fold
     // keeps the parity of c), staged as [parent][reduced coef][child]
-    constexpr int NR = nred_c(P);
     T f[NC];
 #pragma unroll
     for (int k = 0; k < NC; ++k) f[k] = T(0);
@@ -213,7 +220,7 @@ __device__ __forceinline__ void p2m_body(const Box& B, const T* __restrict__ rho
           ++r;
         }
     harmonic_fold<P, T>(f);
-    T* dr = Mr + (B.par & (kP2mParents - 1)) * (8 * NR + 8) + B.c;
+    T* dr = Mr + (B.par & (kP2mParents - 1)) * rp + B.c;
 #pragma unroll
     for (int n = h; n <= P; ++n)
 #pragma unroll
@@ -238,14 +245,15 @@ __device__ __forceinline__ void p2m_block(const T* __restrict__ rho, int nx, int
   extern __shared__ __align__(16) unsigned char p2m_smem[];
   T* Ms = reinterpret_cast<T*>(p2m_smem);
   T* Mr = (harm && (Mhi || Mfold)) ? Ms + kP2mParents * ROWP : nullptr;
+  const int rp = harm == 2 ? p2m_fold_pitch<P>() : ROWR + 8;  // staged pitch of the folded rows
   const long long t = (long long)vb.x * kThreads + threadIdx.x;
   const long long w = t >> 5;
   const Box B = box_of(leaf, (w >> 1) * 32 + (t & 31));
   if (B.par < leaf.npar) {
     if (w & 1)
-      p2m_body<P, T, 1, DIP>(B, rho, nx, ny, b, leaf, Ms, Mr, rho_box, rhi, rlo, flag, dip, ncell);
+      p2m_body<P, T, 1, DIP>(B, rho, nx, ny, b, leaf, Ms, Mr, rp, rho_box, rhi, rlo, flag, dip, ncell);
     else
-      p2m_body<P, T, 0, DIP>(B, rho, nx, ny, b, leaf, Ms, Mr, rho_box, rhi, rlo, flag, dip, ncell);
+      p2m_body<P, T, 0, DIP>(B, rho, nx, ny, b, leaf, Ms, Mr, rp, rho_box, rhi, rlo, flag, dip, ncell);
   }
   __syncthreads();
   const long long p0 = (long long)vb.x * kP2mParents;
@@ -262,17 +270,22 @@ __device__ __forceinline__ void p2m_block(const T* __restrict__ rho, int nx, int
   } else {
     for (int i = threadIdx.x; i < count; i += kThreads) Mleaf[g0 + i] = Ms[(i / ROW) * ROWP + i % ROW];
   }
-  if (Mfold) {  // the folded multipoles in the level's type (CUDA-core harmonic M2L)
+  if (Mfold && harm == 2) {  // component-major (CUDA-core harmonic M2L): runs of the block's 16 parents
+    for (int i = threadIdx.x; i < kP2mParents * ROWR; i += kThreads) {
+      const int pr = i % kP2mParents, k = i / kP2mParents;
+      if (pr < np) Mfold[(long long)k * leaf.npar + p0 + pr] = Mr[pr * rp + k];
+    }
+  } else if (Mfold) {  // the folded multipoles as rows, in the level's type (TF32)
     const int pc = (int)np * ROWR;
-    for (int i = threadIdx.x; i < pc; i += kThreads) Mfold[p0 * ROWR + i] = Mr[(i / ROWR) * (ROWR + 8) + i % ROWR];
+    for (int i = threadIdx.x; i < pc; i += kThreads) Mfold[p0 * ROWR + i] = Mr[(i / ROWR) * rp + i % ROWR];
   }
   if (Mhi) {  // 8 values -> 16 bytes of hi and 16 bytes of lo
-    const int rl = Mr ? ROWR : ROW, rp = Mr ? ROWR + 8 : ROWP;
+    const int rl = Mr ? ROWR : ROW, sp = Mr ? rp : ROWP;
     const T* src = Mr ? Mr : Ms;
     const int pc = (int)np * rl;
     const long long h0 = p0 * rl;
     for (int i = threadIdx.x; i < pc / 8; i += kThreads) {
-      const T* v = src + (i / (rl / 8)) * rp + (i % (rl / 8)) * 8;
+      const T* v = src + (i / (rl / 8)) * sp + (i % (rl / 8)) * 8;
       __nv_bfloat16 hh[8], ll[8];
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
@@ -317,7 +330,7 @@ template <int P, typename T>
 cudaError_t p2m_multi_launch(const P2mArgs* args, const MultiGrid* grids, int n, long long blocks, int harm_rows,
                              cudaStream_t s) {
   constexpr size_t full = (size_t)kP2mParents * (8 * ncoef_c(P) + 8) * sizeof(T);
-  constexpr size_t red0 = (size_t)kP2mParents * (8 * nred_c(P) + 8) * sizeof(T);
+  constexpr size_t red0 = (size_t)kP2mParents * (8 * nred_c(P) + 32) * sizeof(T);
   constexpr size_t red = full + red0 <= 227 * 1024 ? red0 : 0;
   if (harm_rows && red == 0) return cudaErrorInvalidValue;
   const size_t smem = full + (harm_rows ? red : 0);
@@ -356,7 +369,7 @@ cudaError_t p2m_launch(unsigned blocks, cudaStream_t s, const T* rho, int nx, in
   constexpr size_t full = (size_t)kP2mParents * (8 * ncoef_c(P) + 8) * sizeof(T);
   // staged harmonic rows, where they fit beside the full ones (the plan folds
   // nothing at FP64 order 8, which would not)
-  constexpr size_t red0 = (size_t)kP2mParents * (8 * nred_c(P) + 8) * sizeof(T);
+  constexpr size_t red0 = (size_t)kP2mParents * (8 * nred_c(P) + 32) * sizeof(T);
   constexpr size_t red = full + red0 <= 227 * 1024 ? red0 : 0;
   if (harm && (Mhi || Mfold) && red == 0) return cudaErrorInvalidValue;
   const size_t smem = full + ((harm && (Mhi || Mfold)) ? red : 0);

@@ -191,7 +191,7 @@ inline int small_grid_block(long long threads) { return threads < 152LL * kThrea
 // lanes take part in the shuffles), `live` false for padding lanes.  Writes
 // the parent's scaled multipoles 2^-|alpha| sum_children ... into Mp (its own
 // parent-blocked slot) and, when given, the bf16 hi / lo planes and the
-// folded harmonic rows.
+// folded harmonic components (Mfold: rows, or component-major with harm = 2).
 template <int P, typename Tp>
 __device__ __forceinline__ void m2m_to_parent(Tp (&M)[ncoef_c(P)], long long p, int c, bool live, const Level& par,
                                               Tp* __restrict__ Mp, __nv_bfloat16* __restrict__ Mhi,
@@ -244,6 +244,17 @@ __device__ __forceinline__ void m2m_to_parent(Tp (&M)[ncoef_c(P)], long long p, 
   }
   constexpr int NR = nred_c(P);
   harmonic_fold<P, Tp>(M);
+  // phantom siblings past an odd extent: their folds are written as zeros, so
+  // that the folds' layout may change from solve to solve
+  const int edge = (Mfold && !(px & 1) && px + 1 == par.n[0] ? 1 : 0) |
+                   (Mfold && !(py & 1) && py + 1 == par.n[1] ? 2 : 0) |
+                   (Mfold && !(pz & 1) && pz + 1 == par.n[2] ? 4 : 0);
+  if (edge)
+    for (int m = 1; m < 8; ++m) {
+      if ((m & edge) != m) continue;
+      for (int q = c; q < NR; q += 8)
+        Mfold[harm == 2 ? (size_t)(q * 8 + (cp | m)) * par.npar + gp : (size_t)(gp * 8 * NR + q * 8 + (cp | m))] = Tp(0);
+    }
   int r = 0;
 #pragma unroll
   for (int n = 0; n <= P; ++n)
@@ -254,7 +265,7 @@ __device__ __forceinline__ void m2m_to_parent(Tp (&M)[ncoef_c(P)], long long p, 
         if ((r & 7) == c) {
           const size_t o = (size_t)(gp * 8 * NR + cp + r * 8);
           if (Mhi) store_split(Mhi, Mlo, o, M[cidx(n - s, s - cc, cc)]);
-          if (Mfold) Mfold[o] = M[cidx(n - s, s - cc, cc)];
+          if (Mfold) Mfold[harm == 2 ? (size_t)(r * 8 + cp) * par.npar + gp : o] = M[cidx(n - s, s - cc, cc)];
         }
         ++r;
       }
