@@ -3423,7 +3423,7 @@ void build_fused(fmm_batch_t B, const void* const* rho, void* const* phi, void* 
       x.ncell = P->ncell();
       harm_rows |= x.harm ? 1 : 0;
       a.push_back(x);
-      g.push_back(blocks_1d(lf.npar * 16, 256));
+      g.push_back(blocks_1d(lf.npar * 16, sizeof(T) == 8 ? kP2mThreadsF64 : 256));
     }
     add_step(B, MK_P2M, 0, 256, harm_rows, a, g);
   }

@@ -243,8 +243,9 @@ cudaError_t launch_near_tc4(const NearTcLaunch& L, const void* map_hi, const voi
 // Multi-item forms (batched solves, multi.cuh): args and grids are device
 // arrays of n items sorted by first block; blocks = the launch's total, bs
 // the block size every item's grid was computed with.
-// P2M of one leaf level (launch_p2m's arguments; boxes of kThreads / 2 per
-// block: grid = ceil(npar * 16 / kThreads) blocks of kThreads).
+// P2M of one leaf level (launch_p2m's arguments; two threads per box: grid =
+// ceil(npar * 16 / bs) blocks of bs = 256 threads, FP64 kP2mThreadsF64).
+constexpr int kP2mThreadsF64 = 64;
 struct P2mArgs {
   const void* rho;
   int nx, ny, b;

@@ -38,6 +38,16 @@ __device__ __forceinline__ T fd_weight(int j, int off, int n) {
 
 constexpr int kFdTX = 32, kFdTY = 8, kFdZC = 32;
 
+// Planes a block walks along z: kFdZC, fewer where the grid would not give
+// every SM two blocks (a block's walk is a chain of barriers: 64^3 cells 20 us
+// with 16 blocks of 32 planes), at least 4 (each block also reads 4 halo
+// planes).
+int fd_planes(long long xy_blocks, int nz) {
+  int zc = kFdZC;
+  while (zc > 4 && xy_blocks * ((nz + zc - 1) / zc) < 2 * 152) zc /= 2;
+  return zc;
+}
+
 // 32 x 8 columns of cells per block, walking kFdZC cells along z: the z
 // neighbours come from a 5-value register window per column, the x-y
 // neighbours from a shared-memory tile with a 2-cell halo whose centre is the
@@ -45,7 +55,7 @@ constexpr int kFdTX = 32, kFdTY = 8, kFdZC = 32;
 // double-buffered, so one barrier per plane.
 template <typename T>
 __global__ void __launch_bounds__(kFdTX* kFdTY) fd_accel_tiled_kernel(const T* __restrict__ phi, int nx, int ny,
-                                                                      int nz, T inv_dx, T* __restrict__ accel) {
+                                                                      int nz, T inv_dx, T* __restrict__ accel, int zc) {
   constexpr int HX = kFdTX + 4, HY = kFdTY + 4;
   constexpr int kHalo = HX * HY - kFdTX * kFdTY;  // 176 halo cells per plane
   __shared__ T tile[2][HY][HX];
@@ -53,7 +63,7 @@ __global__ void __launch_bounds__(kFdTX* kFdTY) fd_accel_tiled_kernel(const T* _
   const long long plane = (long long)nx * ny;
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int tid = ty * kFdTX + tx;
-  const int x0 = blockIdx.x * kFdTX, y0 = blockIdx.y * kFdTY, z0 = blockIdx.z * kFdZC;
+  const int x0 = blockIdx.x * kFdTX, y0 = blockIdx.y * kFdTY, z0 = blockIdx.z * zc;
   const int x = x0 + tx, y = y0 + ty;
   const bool inside = x < nx && y < ny;
   const long long col = (long long)y * nx + x;
@@ -87,7 +97,7 @@ __global__ void __launch_bounds__(kFdTX* kFdTY) fd_accel_tiled_kernel(const T* _
     const int zz = z0 - 2 + q;
     w[q + 1] = (inside && zz >= 0 && zz < nz) ? phi[(long long)zz * plane + col] : T(0);
   }
-  const int z1 = min(z0 + kFdZC, nz);
+  const int z1 = min(z0 + zc, nz);
   for (int z = z0; z < z1; ++z) {
     const int buf = (z - z0) & 1;
 #pragma unroll
@@ -123,14 +133,14 @@ __global__ void __launch_bounds__(kFdTX* kFdTY) fd_accel_tiled_kernel(const T* _
 // of each tile row.
 constexpr int kFd4TX = 4 * kFdTX;  // cells per tile row
 __device__ __forceinline__ void fd_accel_vec4_body(const float* __restrict__ phi, int nx, int ny, int nz,
-                                                  float inv_dx, float* __restrict__ accel, const VBlock& vb) {
+                                                  float inv_dx, float* __restrict__ accel, const VBlock& vb, int zc) {
   constexpr int HX = kFd4TX + 8, HY = kFdTY + 4, C0 = 4;  // tile row: halo at C0-2, C0-1 and C0+128, C0+129
   __shared__ __align__(16) float tile[2][HY][HX];
   const long long n = (long long)nx * ny * nz;
   const long long plane = (long long)nx * ny;
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int tid = ty * kFdTX + tx;
-  const int x0 = vb.x * kFd4TX, y0 = vb.y * kFdTY, z0 = vb.z * kFdZC;
+  const int x0 = vb.x * kFd4TX, y0 = vb.y * kFdTY, z0 = vb.z * zc;
   const int x = x0 + 4 * tx, y = y0 + ty;
   const bool inside = x < nx && y < ny;  // nx % 4 == 0: all four cells
   const long long col = (long long)y * nx + x;
@@ -179,7 +189,7 @@ __device__ __forceinline__ void fd_accel_vec4_body(const float* __restrict__ phi
   float4 h4;
   float h1;
   load_halo(z0, h4, h1);
-  const int z1 = min(z0 + kFdZC, nz);
+  const int z1 = min(z0 + zc, nz);
   for (int z = z0; z < z1; ++z) {
     const int buf = (z - z0) & 1;
 #pragma unroll
@@ -225,8 +235,8 @@ __device__ __forceinline__ void fd_accel_vec4_body(const float* __restrict__ phi
 
 __global__ void __launch_bounds__(kFdTX* kFdTY, 3) fd_accel_vec4_kernel(const float* __restrict__ phi, int nx, int ny,
                                                                      int nz, float inv_dx,
-                                                                     float* __restrict__ accel) {
-  fd_accel_vec4_body(phi, nx, ny, nz, inv_dx, accel, native_vblock());
+                                                                     float* __restrict__ accel, int zc) {
+  fd_accel_vec4_body(phi, nx, ny, nz, inv_dx, accel, native_vblock(), zc);
 }
 
 // The stencils of many solves in one launch (batched solves; FP32 rows of a
@@ -238,7 +248,7 @@ __global__ void __launch_bounds__(kFdTX* kFdTY, 3) fd_accel_vec4_multi_kernel(co
   if (threadIdx.x == 0 && threadIdx.y == 0) x = a[i];
   __syncthreads();
   fd_accel_vec4_body(static_cast<const float*>(x.phi), x.nx, x.ny, x.nz, (float)x.inv_dx, static_cast<float*>(x.accel),
-                     multi_vblock(g[i]));
+                     multi_vblock(g[i]), kFdZC);
 }
 
 // Grid: x blocks over a row, y = row index, z = slice (32-bit indexing).
@@ -328,15 +338,17 @@ cudaError_t launch_fd_accel(const T* phi, const int dims[3], double inv_dx, T* a
   }
   if (sizeof(T) == 4 && dims[0] % 4 == 0 && (reinterpret_cast<uintptr_t>(phi) & 15) == 0 &&
       (reinterpret_cast<uintptr_t>(accel) & 15) == 0) {
-    dim3 grid((unsigned)((dims[0] + kFd4TX - 1) / kFd4TX), (unsigned)((dims[1] + kFdTY - 1) / kFdTY),
-              (unsigned)((dims[2] + kFdZC - 1) / kFdZC));
+    dim3 grid((unsigned)((dims[0] + kFd4TX - 1) / kFd4TX), (unsigned)((dims[1] + kFdTY - 1) / kFdTY));
+    const int zc = fd_planes((long long)grid.x * grid.y, dims[2]);
+    grid.z = (unsigned)((dims[2] + zc - 1) / zc);
     fd_accel_vec4_kernel<<<grid, dim3(kFdTX, kFdTY), 0, s>>>(reinterpret_cast<const float*>(phi), dims[0], dims[1],
-                                                             dims[2], (float)inv_dx, reinterpret_cast<float*>(accel));
+                                                             dims[2], (float)inv_dx, reinterpret_cast<float*>(accel), zc);
     return cudaGetLastError();
   }
-  dim3 grid((unsigned)((dims[0] + kFdTX - 1) / kFdTX), (unsigned)((dims[1] + kFdTY - 1) / kFdTY),
-            (unsigned)((dims[2] + kFdZC - 1) / kFdZC));
-  fd_accel_tiled_kernel<T><<<grid, dim3(kFdTX, kFdTY), 0, s>>>(phi, dims[0], dims[1], dims[2], (T)inv_dx, accel);
+  dim3 grid((unsigned)((dims[0] + kFdTX - 1) / kFdTX), (unsigned)((dims[1] + kFdTY - 1) / kFdTY));
+  const int zc = fd_planes((long long)grid.x * grid.y, dims[2]);
+  grid.z = (unsigned)((dims[2] + zc - 1) / zc);
+  fd_accel_tiled_kernel<T><<<grid, dim3(kFdTX, kFdTY), 0, s>>>(phi, dims[0], dims[1], dims[2], (T)inv_dx, accel, zc);
   return cudaGetLastError();
 }
 

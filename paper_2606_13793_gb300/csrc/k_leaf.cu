@@ -23,7 +23,7 @@ __device__ __forceinline__ void leaf_finish_body(const Level& leaf, const T* __r
                                                  const T* __restrict__ m2p, int nx, int ny, int b, T scale,
                                                  T* __restrict__ phi, const VBlock& vb, const LeafDownArgs<T>& down) {
   constexpr int NC = ncoef_c(P);
-  const long long t = (long long)vb.x * kThreads + threadIdx.x;
+  const long long t = (long long)vb.x * blockDim.x + threadIdx.x;
   const Box B = box_of(leaf, t);
   if (!B.real) return;
   T L[NC];
@@ -323,7 +323,8 @@ cudaError_t launch_leaf_finish(const TreeTables& t, const Level& leaf, const T* 
   const long long threads = leaf.npar * 8;
   if (threads == 0) return cudaSuccess;
   const LeafDownArgs<T> none{};
-  FMM_ORDER_SWITCH(t.p, (leaf_finish_kernel<PP, T><<<grid_threads(threads), kThreads, 0, s>>>(
+  const int bs = small_grid_block(threads);  // few boxes: warp-sized blocks on more SMs
+  FMM_ORDER_SWITCH(t.p, (leaf_finish_kernel<PP, T><<<(unsigned)((threads + bs - 1) / bs), bs, 0, s>>>(
                             leaf, Lleaf, near_box, near_stride, m2p, dims[0], dims[1], t.b, (T)scale, phi,
                             down ? *down : none)));
   return cudaGetLastError();

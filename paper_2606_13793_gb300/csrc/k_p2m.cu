@@ -19,7 +19,15 @@ using namespace tree;
 // as many warps fit on an SM to hide the density loads (the second warp's
 // reads of the same cells hit L1).  The parity is warp-uniform and selects a
 // body instantiated for it, so every register index stays compile-time.
-constexpr int kP2mParents = kThreads / 16;  // 2 threads per box, 8 boxes per parent
+//
+// Block size: 256 threads (16 parents) in FP32; 64 (4 parents) in FP64, whose
+// blocks are bound by their SM's narrow DFMA pipe, so that a small grid
+// reaches more SMs (32^3 cells at p = 4: 4 -> 16 blocks; 96^3 at p = 6: 108 ->
+// 432).
+template <typename T>
+constexpr int kP2mThreads = sizeof(T) == 8 ? kP2mThreadsF64 : kThreads;
+template <typename T>
+constexpr int kP2mParents = kP2mThreads<T> / 16;  // 2 threads per box, 8 boxes per parent
 
 // Staged pitch of the folded rows that are written component-major: 10 mod 32
 // values, so that 16 parents' values of one component (read together) lie in
@@ -189,7 +197,7 @@ __device__ __forceinline__ void p2m_body(const Box& B, const T* __restrict__ rho
   if (bad && h == 0) atomicOr(flag, 1);
   // into the block's staged parent rows [parent][coef][child] (rows padded
   // by 8 values so the four parents of a warp fall in different banks)
-  T* dst = Ms + (B.par & (kP2mParents - 1)) * (8 * NC + 8) + B.c;
+  T* dst = Ms + (B.par & (kP2mParents<T> - 1)) * (8 * NC + 8) + B.c;
   int q = 0;
 #pragma unroll
   for (int n = 0; n <= P; ++n)
@@ -220,7 +228,7 @@ __device__ __forceinline__ void p2m_body(const Box& B, const T* __restrict__ rho
           ++r;
         }
     harmonic_fold<P, T>(f);
-    T* dr = Mr + (B.par & (kP2mParents - 1)) * rp + B.c;
+    T* dr = Mr + (B.par & (kP2mParents<T> - 1)) * rp + B.c;
 #pragma unroll
     for (int n = h; n <= P; ++n)
 #pragma unroll
@@ -244,9 +252,9 @@ __device__ __forceinline__ void p2m_block(const T* __restrict__ rho, int nx, int
   constexpr int ROWR = 8 * nred_c(P);  // values per parent row of the harmonic planes
   extern __shared__ __align__(16) unsigned char p2m_smem[];
   T* Ms = reinterpret_cast<T*>(p2m_smem);
-  T* Mr = (harm && (Mhi || Mfold)) ? Ms + kP2mParents * ROWP : nullptr;
+  T* Mr = (harm && (Mhi || Mfold)) ? Ms + kP2mParents<T> * ROWP : nullptr;
   const int rp = harm == 2 ? p2m_fold_pitch<P>() : ROWR + 8;  // staged pitch of the folded rows
-  const long long t = (long long)vb.x * kThreads + threadIdx.x;
+  const long long t = (long long)vb.x * kP2mThreads<T> + threadIdx.x;
   const long long w = t >> 5;
   const Box B = box_of(leaf, (w >> 1) * 32 + (t & 31));
   if (B.par < leaf.npar) {
@@ -256,35 +264,35 @@ __device__ __forceinline__ void p2m_block(const T* __restrict__ rho, int nx, int
       p2m_body<P, T, 0, DIP>(B, rho, nx, ny, b, leaf, Ms, Mr, rp, rho_box, rhi, rlo, flag, dip, ncell);
   }
   __syncthreads();
-  const long long p0 = (long long)vb.x * kP2mParents;
-  const long long np = min((long long)kP2mParents, leaf.npar - p0);
+  const long long p0 = (long long)vb.x * kP2mParents<T>;
+  const long long np = min((long long)kP2mParents<T>, leaf.npar - p0);
   if (np <= 0) return;
   const int count = (int)np * ROW;  // a multiple of 8
   const long long g0 = p0 * ROW;
   if (sizeof(T) == 4) {
     float4* out = reinterpret_cast<float4*>(Mleaf + g0);
-    for (int i = threadIdx.x; i < count / 4; i += kThreads) {
+    for (int i = threadIdx.x; i < count / 4; i += kP2mThreads<T>) {
       const int pr = i / (ROW / 4), wi = i % (ROW / 4);
       out[i] = *reinterpret_cast<const float4*>(Ms + pr * ROWP + wi * 4);
     }
   } else {
-    for (int i = threadIdx.x; i < count; i += kThreads) Mleaf[g0 + i] = Ms[(i / ROW) * ROWP + i % ROW];
+    for (int i = threadIdx.x; i < count; i += kP2mThreads<T>) Mleaf[g0 + i] = Ms[(i / ROW) * ROWP + i % ROW];
   }
   if (Mfold && harm == 2) {  // component-major (CUDA-core harmonic M2L): runs of the block's 16 parents
-    for (int i = threadIdx.x; i < kP2mParents * ROWR; i += kThreads) {
-      const int pr = i % kP2mParents, k = i / kP2mParents;
+    for (int i = threadIdx.x; i < kP2mParents<T> * ROWR; i += kP2mThreads<T>) {
+      const int pr = i % kP2mParents<T>, k = i / kP2mParents<T>;
       if (pr < np) Mfold[(long long)k * leaf.npar + p0 + pr] = Mr[pr * rp + k];
     }
   } else if (Mfold) {  // the folded multipoles as rows, in the level's type (TF32)
     const int pc = (int)np * ROWR;
-    for (int i = threadIdx.x; i < pc; i += kThreads) Mfold[p0 * ROWR + i] = Mr[(i / ROWR) * rp + i % ROWR];
+    for (int i = threadIdx.x; i < pc; i += kP2mThreads<T>) Mfold[p0 * ROWR + i] = Mr[(i / ROWR) * rp + i % ROWR];
   }
   if (Mhi) {  // 8 values -> 16 bytes of hi and 16 bytes of lo
     const int rl = Mr ? ROWR : ROW, sp = Mr ? rp : ROWP;
     const T* src = Mr ? Mr : Ms;
     const int pc = (int)np * rl;
     const long long h0 = p0 * rl;
-    for (int i = threadIdx.x; i < pc / 8; i += kThreads) {
+    for (int i = threadIdx.x; i < pc / 8; i += kP2mThreads<T>) {
       const T* v = src + (i / (rl / 8)) * sp + (i % (rl / 8)) * 8;
       __nv_bfloat16 hh[8], ll[8];
 #pragma unroll
@@ -300,7 +308,7 @@ __device__ __forceinline__ void p2m_block(const T* __restrict__ rho, int nx, int
 }
 
 template <int P, typename T, bool DIP>
-__global__ void __launch_bounds__(kThreads) p2m_kernel(const T* __restrict__ rho, int nx, int ny, int b, Level leaf,
+__global__ void __launch_bounds__(kP2mThreads<T>) p2m_kernel(const T* __restrict__ rho, int nx, int ny, int b, Level leaf,
                                                        T* __restrict__ Mleaf, __nv_bfloat16* __restrict__ Mhi,
                                                        __nv_bfloat16* __restrict__ Mlo, T* __restrict__ rho_box,
                                                        __nv_bfloat16* __restrict__ rhi,
@@ -313,7 +321,7 @@ __global__ void __launch_bounds__(kThreads) p2m_kernel(const T* __restrict__ rho
 
 // The leaf levels of many solves in one launch (batched solves).
 template <int P, typename T>
-__global__ void __launch_bounds__(kThreads) p2m_multi_kernel(const P2mArgs* __restrict__ a,
+__global__ void __launch_bounds__(kP2mThreads<T>) p2m_multi_kernel(const P2mArgs* __restrict__ a,
                                                              const MultiGrid* __restrict__ g, int n) {
   __shared__ P2mArgs x;  // the item's arguments, read by the body from shared memory
   const int i = multi_item(g, n);
@@ -329,8 +337,8 @@ __global__ void __launch_bounds__(kThreads) p2m_multi_kernel(const P2mArgs* __re
 template <int P, typename T>
 cudaError_t p2m_multi_launch(const P2mArgs* args, const MultiGrid* grids, int n, long long blocks, int harm_rows,
                              cudaStream_t s) {
-  constexpr size_t full = (size_t)kP2mParents * (8 * ncoef_c(P) + 8) * sizeof(T);
-  constexpr size_t red0 = (size_t)kP2mParents * (8 * nred_c(P) + 32) * sizeof(T);
+  constexpr size_t full = (size_t)kP2mParents<T> * (8 * ncoef_c(P) + 8) * sizeof(T);
+  constexpr size_t red0 = (size_t)kP2mParents<T> * (8 * nred_c(P) + 32) * sizeof(T);
   constexpr size_t red = full + red0 <= 227 * 1024 ? red0 : 0;
   if (harm_rows && red == 0) return cudaErrorInvalidValue;
   const size_t smem = full + (harm_rows ? red : 0);
@@ -341,7 +349,7 @@ cudaError_t p2m_multi_launch(const P2mArgs* args, const MultiGrid* grids, int n,
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  p2m_multi_kernel<P, T><<<(unsigned)blocks, kThreads, smem, s>>>(args, grids, n);
+  p2m_multi_kernel<P, T><<<(unsigned)blocks, kP2mThreads<T>, smem, s>>>(args, grids, n);
   return cudaGetLastError();
 }
 
@@ -357,7 +365,7 @@ cudaError_t p2m_launch_dip(unsigned blocks, size_t smem, size_t attr_bytes, cuda
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  p2m_kernel<P, T, DIP><<<blocks, kThreads, smem, s>>>(rho, nx, ny, b, leaf, Mleaf, Mhi, Mlo, rho_box, rhi, rlo, flag,
+  p2m_kernel<P, T, DIP><<<blocks, kP2mThreads<T>, smem, s>>>(rho, nx, ny, b, leaf, Mleaf, Mhi, Mlo, rho_box, rhi, rlo, flag,
                                                        harm, Mfold, dip, ncell);
   return cudaGetLastError();
 }
@@ -366,10 +374,10 @@ template <int P, typename T>
 cudaError_t p2m_launch(unsigned blocks, cudaStream_t s, const T* rho, int nx, int ny, int b, Level leaf, T* Mleaf,
                 __nv_bfloat16* Mhi, __nv_bfloat16* Mlo, T* rho_box, __nv_bfloat16* rhi, __nv_bfloat16* rlo, int* flag,
                 int harm, T* Mfold, const T* dip, long long ncell) {
-  constexpr size_t full = (size_t)kP2mParents * (8 * ncoef_c(P) + 8) * sizeof(T);
+  constexpr size_t full = (size_t)kP2mParents<T> * (8 * ncoef_c(P) + 8) * sizeof(T);
   // staged harmonic rows, where they fit beside the full ones (the plan folds
   // nothing at FP64 order 8, which would not)
-  constexpr size_t red0 = (size_t)kP2mParents * (8 * nred_c(P) + 32) * sizeof(T);
+  constexpr size_t red0 = (size_t)kP2mParents<T> * (8 * nred_c(P) + 32) * sizeof(T);
   constexpr size_t red = full + red0 <= 227 * 1024 ? red0 : 0;
   if (harm && (Mhi || Mfold) && red == 0) return cudaErrorInvalidValue;
   const size_t smem = full + ((harm && (Mhi || Mfold)) ? red : 0);
@@ -389,7 +397,7 @@ cudaError_t launch_p2m(const TreeTables& t, const T* rho, const int dims[3], con
   const long long threads = leaf.npar * 16;  // two threads per box
   if (threads == 0) return cudaSuccess;
   cudaError_t e = cudaSuccess;
-  FMM_ORDER_SWITCH(t.p, (e = p2m_launch<PP, T>(grid_threads(threads), s,
+  FMM_ORDER_SWITCH(t.p, (e = p2m_launch<PP, T>((unsigned)((threads + kP2mThreads<T> - 1) / kP2mThreads<T>), s,
                             rho, dims[0], dims[1], t.b, leaf, Mleaf, static_cast<__nv_bfloat16*>(Mhi),
                             static_cast<__nv_bfloat16*>(Mlo), rho_box, static_cast<__nv_bfloat16*>(rho_hi),
                             static_cast<__nv_bfloat16*>(rho_lo), flag, harm, Mfold, dip,
