@@ -329,6 +329,11 @@ fmm_status fmm_plan_autotune(fmm_plan_t plan, void* stream);
  *                              with mult_order < order, for its transposed
  *                              form).
  * All schedules give the same sums up to the order of the FP32 additions.
+ * Until an M2L schedule is selected, the bf16x3 levels whose row tiles (128
+ * rows each) do not fill the GPU run, in plans without the stencil force
+ * (accel 0 or 2), in FP32 on the CUDA cores instead (sums
+ * and differences over mirror pairs, 8 times fewer products), where that is
+ * the faster one; selecting a schedule puts every such level on it.
  * The paper has no counterpart.
  */
 fmm_status fmm_plan_tc_schedule(fmm_plan_t plan, int what, int* prefix, int* available);
@@ -451,7 +456,9 @@ fmm_status fmm_debug_level(fmm_plan_t plan, int what, int level, double* host_ou
 int fmm_plan_leaf_level(fmm_plan_t plan);
 
 /* How the M2L of one level runs: 0 none (levels 0, 1), 1 CUDA cores FP32,
- * 2 CUDA cores FP64, 3 tcgen05 tensor cores; -1 for a bad plan or level. */
+ * 2 CUDA cores FP64, 3 tcgen05 tensor cores (a level too small to fill them
+ * may run FP32 all the same, see fmm_plan_tc_schedule); -1 for a bad plan or
+ * level. */
 int fmm_plan_level_kind(fmm_plan_t plan, int level);
 
 /* 1 when the near field runs on the tensor cores (bf16x3), else 0. */

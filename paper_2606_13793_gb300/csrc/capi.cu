@@ -261,6 +261,10 @@ struct fmm_plan_s {
   bool tp_m2l = false, tp_m2l_t = false, tp_m2p = false, tp_near = false;
   bool span_m2l = false, span_m2l_t = false, span_near = false, span_m2p = false;
   bool use_tp[3] = {true, false, true};
+  // tensor-core levels with a reflection-basis form (Level::rfold_off) run it,
+  // until an M2L schedule is selected; refl_now: in the current (last) solve
+  bool use_refl = true, refl_now = true;
+  bool refl_on(int l) const { return lev[l].rfold_off != 0 && refl_now; }
   // the dedicated near-field kernel of leaf 4 (k_near_tc.cu), used when
   // present unless another schedule is selected
   bool near4 = false, use_near4 = true;
@@ -1710,6 +1714,23 @@ void sym_default(fmm_plan_t P, const NbrGemm& g, fmm_plan_s::SimtChoice* c, bool
   }
 }
 
+// Whether a bf16x3 tensor-core level runs the FP32 reflection basis instead:
+// a wave of row tiles (one per SM, 128 rows each) takes a tile's latency
+// however few there are, 0.195 ms at p = 6 and 0.40 ms at p = 8 (prefix
+// schedule: 32 to 152 tiles 0.197 ms, 256 tiles 0.393, 2048 tiles 2.71 ms),
+// while the reflection basis costs 10.9 (p = 6) or 28 ns a row (16^3 rows 0.064,
+// 32^3 0.36, 64^3 2.86 ms): it wins below ~14000 rows a wave (a full one has
+// 19456).  Both sums are FP32, this one of unsplit operands.  A caller that
+// lowers n_fp64_levels asks for the tensor cores on small levels and gets them.
+// Plans with the stencil force stay on them too: the stencil amplifies what
+// the split operands round (512^3: level 5 alone is 2.5e-5 of the force), and
+// the force keeps to that of earlier releases.
+bool reflect_tc_level(const Level& lv) {
+  const long long tiles = (long long)((lv.np[0] + kTcTileX - 1) / kTcTileX) * ((lv.np[1] + kTcTileY - 1) / kTcTileY) *
+                          lv.np[2];
+  return lv.npar < 14000 * ((tiles + 151) / 152);
+}
+
 fmm_status plan_init(fmm_plan_t P, const int d3[3], double dx, double G, int order, int leaf, const fmm_opts& o,
                      cudaStream_t stream, int dev) {
   cudaStream_t s = stream;
@@ -1778,6 +1799,15 @@ fmm_status plan_init(fmm_plan_t P, const int d3[3], double dx, double G, int ord
       lv.fold_off = off;
       off = align(off + (size_t)lv.npar * 8 * P->nr * 4);
     }
+    if (lv.tc && P->tc_kind == TC_BF16X3 && P->harm && P->harm_cc && o.accel != 1 && o.n_fp64_levels >= 3 &&
+        !(l == P->L && P->m2p) &&
+        reflect_tc_level(lv)) {
+      const size_t red = (size_t)lv.npar * 8 * P->nr * 4;
+      lv.rfold_off = off;
+      off = align(off + red);
+      lv.rred_off = off;
+      off = align(off + red);
+    }
     if (lv.tc && P->tc_kind == TC_BF16X3) {
       const size_t plane = (size_t)lv.npar * 8 * P->plane_nc() * 2;
       lv.hi_off = off;
@@ -1818,6 +1848,7 @@ fmm_status plan_init(fmm_plan_t P, const int d3[3], double dx, double G, int ord
       const size_t one = (size_t)P->lev[l].npar * (size_t)ncol * (size_t)(P->lev[l].f64 ? 8 : 4);
       if (P->split_level(l)) part = std::max(part, 27 * one);
       if (!P->lev[l].tc) want = std::max(want, 27 * one);
+      if (P->lev[l].rfold_off) want = std::max(want, 9 * one);
     }
     // room for the autotuner's neighbour-split candidates (M2L levels and the
     // near field), up to 64 MiB each
@@ -1878,11 +1909,12 @@ fmm_status plan_init(fmm_plan_t P, const int d3[3], double dx, double G, int ord
       (st = P->upload(l2l, &P->d_l2l, s)) || (st = P->upload(one_flag, &P->d_flag, s)))
     return cleanup(st);
   {
-    bool any64 = false, any32 = false, anytc = false;
+    bool any64 = false, any32 = false, anytc = false, anyrf = false;
     for (int l = 2; l <= P->L; ++l) {
       any64 |= P->lev[l].f64 != 0;
       any32 |= (!P->lev[l].f64 && !P->lev[l].tc);
       anytc |= P->lev[l].tc != 0;
+      anyrf |= P->lev[l].rfold_off != 0;
     }
     TaylorTable tt;
     if (P->L >= 2 && !P->static_keep_tables) tt.build(P->mi);
@@ -1909,7 +1941,7 @@ fmm_status plan_init(fmm_plan_t P, const int d3[3], double dx, double G, int ord
       }
       return P->upload(tab, &P->d_sym_tab[slot], s);
     };
-    if (P->harm_cc && (any64 || any32) && (st = put_sym(P->mi, 0))) return cleanup(st);
+    if (P->harm_cc && (any64 || any32 || anyrf) && (st = put_sym(P->mi, 0))) return cleanup(st);
     if (any64) {
       std::vector<double> W;
       m2l_weights<double>(P->mi, tt, W, tk, tw, !P->static_keep_tables, P->harm_cc);
@@ -1931,7 +1963,7 @@ fmm_status plan_init(fmm_plan_t P, const int d3[3], double dx, double G, int ord
     mt.mo = P->p;
     mt.lo = P->mi.mo;
     P->asym = P->mi.mo < P->p && P->L >= 2;
-    if (P->asym && (any64 || any32) && P->harm_cc && (st = put_sym(mt, 1))) return cleanup(st);
+    if (P->asym && (any64 || any32 || anyrf) && P->harm_cc && (st = put_sym(mt, 1))) return cleanup(st);
     if (P->asym && (any64 || any32)) {
       std::vector<int> tk2;
       std::vector<long long> tw2;
@@ -2278,6 +2310,7 @@ fmm_status plan_init(fmm_plan_t P, const int d3[3], double dx, double G, int ord
   P->tcm.err = P->d_flag;
   for (int l = 2; l <= P->L; ++l)
     if (!P->lev[l].tc) zrun_default(m2l_gemm(P, l), P->h_m2l_tile_k, &P->m2l_choice[l], P->lev[l].f64);
+    else if (P->lev[l].rfold_off) sym_default(P, m2l_gemm(P, l), &P->m2l_choice[l], false);
   if (!P->near_tc) zrun_default(near_gemm(P), P->h_near_tile_k, &P->near_choice, P->f64_data());
   // uploads read host vectors that go out of scope here (plans only; the
   // allocation-free solve orders its copies on the caller's stream)
@@ -2406,10 +2439,11 @@ bool sym_level(fmm_plan_t P, int l);
 // Per-level dispatch helpers (a level's expansions are FP64 or FP32).
 fmm_status do_m2m(fmm_plan_t P, const TreeTables& tt, int l, cudaStream_t s) {
   const Level &c = P->lev[l], &q = P->lev[l - 1];
-  const bool planes = q.tc && P->tc_kind == TC_BF16X3;
+  const bool refl = P->refl_on(l - 1);
+  const bool planes = q.tc && P->tc_kind == TC_BF16X3 && !refl;
   void* hi = planes ? P->arena + q.hi_off : nullptr;
   void* lo = planes ? P->arena + q.lo_off : nullptr;
-  void* fold = q.fold_off ? P->arena + q.fold_off : nullptr;
+  void* fold = refl ? P->arena + q.rfold_off : q.fold_off ? P->arena + q.fold_off : nullptr;
   const int harm = sym_level(P, l - 1) ? 2 : (planes && P->harm) || fold ? 1 : 0;  // 2: component-major folds
   cudaError_t e;
   if (c.f64)
@@ -2434,10 +2468,17 @@ bool harmonic_m2l_level(fmm_plan_t P, int l) {
   return ((P->harm && P->lev[l].tc) || P->lev[l].lred_off) && !(l == P->L && P->m2p);
 }
 
+// The compact rows a level's CUDA-core harmonic M2L wrote (NULL: its locals
+// are in the full rows).
+void* red_rows(fmm_plan_t P, int l) {
+  const Level& lv = P->lev[l];
+  return P->refl_on(l) ? P->arena + lv.rred_off : lv.lred_off ? P->arena + lv.lred_off : nullptr;
+}
+
 fmm_status do_l2l(fmm_plan_t P, const TreeTables& tt, int l, cudaStream_t s, int accumulate) {
   const Level &q = P->lev[l - 1], &c = P->lev[l];
   const int harm = accumulate && harmonic_m2l_level(P, l) ? 1 : 0;
-  const void* red = harm && c.lred_off ? P->arena + c.lred_off : nullptr;  // CUDA-core harmonic: compact rows
+  const void* red = harm ? red_rows(P, l) : nullptr;
   cudaError_t e;
   if (l == 2 && c.f64) {
     e = launch_l2l<double, double>(tt, q, nullptr, c, static_cast<double*>(P->Lx(l)), 1, harm,
@@ -2467,7 +2508,7 @@ fmm_status do_l2l(fmm_plan_t P, const TreeTables& tt, int l, cudaStream_t s, int
 bool sym_level(fmm_plan_t P, int l) {
   const Level& lv = P->lev[l];
   const int sh = P->m2l_choice[l].shape;
-  return lv.fold_off && !lv.tc && (lv.f64 || sh == 1 || sh == 2);
+  return P->refl_on(l) || (lv.fold_off && !lv.tc && (lv.f64 || sh == 1 || sh == 2));
 }
 
 // form: the level's own (-1: sym_level), or forced: 0 direct, 1 reflection
@@ -2476,15 +2517,17 @@ NbrGemm m2l_gemm(fmm_plan_t P, int l, int form) {
   const Level& lv = P->lev[l];
   NbrGemm g;
   // harmonic: folded multipoles in, the c <= 1 locals out (compact rows)
-  const int nk = lv.fold_off ? P->nr : P->nc;
-  g.A = lv.fold_off ? static_cast<void*>(P->arena + lv.fold_off) : P->M(l);
+  const bool rf = lv.rfold_off != 0;  // (only reached by a tensor-core level in its reflection-basis form)
+  const int nk = rf || lv.fold_off ? P->nr : P->nc;
+  g.A = rf ? static_cast<void*>(P->arena + lv.rfold_off) : lv.fold_off ? static_cast<void*>(P->arena + lv.fold_off) : P->M(l);
   g.row_len = 8 * nk;
   for (int q = 0; q < 3; ++q) g.grid[q] = lv.np[q];
   const bool tr = P->transposed && P->asym;
   g.W = lv.f64 ? (tr ? P->d_w_m2l_f64_t : P->d_w_m2l_f64) : (tr ? P->d_w_m2l_f32_t : P->d_w_m2l_f32);
   g.tile_k = tr ? P->d_m2l_tile_k_t : P->d_m2l_tile_k;
   g.tile_w = tr ? P->d_m2l_tile_w_t : P->d_m2l_tile_w;
-  g.C = lv.lred_off ? static_cast<void*>(P->arena + lv.lred_off) : P->Lx(l);
+  g.C = rf ? static_cast<void*>(P->arena + lv.rred_off)
+        : lv.lred_off ? static_cast<void*>(P->arena + lv.lred_off) : P->Lx(l);
   g.n_cols = 8 * nk;
   g.ntiles = P->m2l_ntiles;
   g.accumulate = 0;  // M2L writes the level's locals; L2L adds the parent's
@@ -2603,7 +2646,7 @@ fmm_status do_p2l(fmm_plan_t P, cudaStream_t s) {
 
 fmm_status do_m2l(fmm_plan_t P, int l, cudaStream_t s) {
   const Level& lv = P->lev[l];
-  if (lv.tc && tc_prefix(P, TS_M2L)) {
+  if (lv.tc && !P->refl_on(l) && tc_prefix(P, TS_M2L)) {
     TpLaunch& L = (P->transposed && P->asym) ? P->tpl_t : P->tpl;
     L.C = static_cast<float*>(P->Lx(l));
     for (int q = 0; q < 3; ++q) L.grid[q] = lv.np[q];
@@ -2614,7 +2657,7 @@ fmm_status do_m2l(fmm_plan_t P, int l, cudaStream_t s) {
     CUDA_TRY(e);
     return FMM_OK;
   }
-  if (lv.tc) {
+  if (lv.tc && !P->refl_on(l)) {
     TcLaunch L = (P->transposed && P->asym) ? P->tc_t : P->tc;
     L.C = static_cast<float*>(P->Lx(l));
     for (int q = 0; q < 3; ++q) L.grid[q] = lv.np[q];
@@ -2689,6 +2732,7 @@ template <typename T>
 fmm_status run_solve(fmm_plan_t P, const T* rho, T* phi, T* accel, cudaStream_t s, bool adjoint = false) {
   const TreeTables tt = P->tables();
   const int L = P->L;
+  P->refl_now = P->use_refl && !P->inject_timeout;
   T* rho_box = reinterpret_cast<T*>(P->arena + P->rho_box_off);
   T* near_box = reinterpret_cast<T*>(P->arena + P->near_off);
   fmm_status st;
@@ -2706,7 +2750,8 @@ fmm_status run_solve(fmm_plan_t P, const T* rho, T* phi, T* accel, cudaStream_t 
   {
     StageTimer t(P, ST_P2M, s);
     const Level& lf = P->lev[L];
-    const bool mplanes = lf.tc && P->tc_kind == TC_BF16X3;
+    const bool refl = P->refl_on(L);
+    const bool mplanes = lf.tc && P->tc_kind == TC_BF16X3 && !refl;
     const bool near_rows = !adj_g;  // the near field's own inputs (not read by the transposed force's)
     CUDA_TRY(launch_p2m<T>(tt, rho, P->dims, lf, static_cast<T*>(P->M(L)),
                            (P->near_tc || !near_rows) ? nullptr : rho_box,
@@ -2714,7 +2759,10 @@ fmm_status run_solve(fmm_plan_t P, const T* rho, T* phi, T* accel, cudaStream_t 
                            (P->near_tc && near_rows) ? P->arena + P->rho_hi_off : nullptr,
                            (P->near_tc && near_rows) ? P->arena + P->rho_lo_off : nullptr, P->d_flag,
                            sym_level(P, L) ? 2 : ((mplanes && P->harm) || lf.fold_off) ? 1 : 0,
-                           lf.fold_off ? reinterpret_cast<T*>(P->arena + lf.fold_off) : nullptr, s, adj_dip));
+                           refl          ? reinterpret_cast<T*>(P->arena + lf.rfold_off)
+                           : lf.fold_off ? reinterpret_cast<T*>(P->arena + lf.fold_off)
+                                         : nullptr,
+                           s, adj_dip));
   }
   const bool p2l = adjoint && P->m2p;  // leaf level by the transpose of M2P
   if (p2l && P->m2p_comps == 4)  // [w, v] per box, the force columns zero without g
@@ -2738,7 +2786,7 @@ fmm_status run_solve(fmm_plan_t P, const T* rho, T* phi, T* accel, cudaStream_t 
     CUDA_TRY(launch_zero<T>(static_cast<T*>(P->Lx(L)), P->lev[L].bytes / sizeof(T), s));
   }
   bool any_simt = false;
-  for (int l = 2; l <= L; ++l) any_simt |= !P->lev[l].tc;
+  for (int l = 2; l <= L; ++l) any_simt |= !P->lev[l].tc || P->refl_on(l);
   const bool fork = P->side && any_simt;
   cudaStream_t sf = fork ? P->side : s;
   if (fork) {
@@ -2748,7 +2796,7 @@ fmm_status run_solve(fmm_plan_t P, const T* rho, T* phi, T* accel, cudaStream_t 
   {
     int ls[kMaxLevels], n = 0;
     for (int l = 2; l <= L; ++l)
-      if (!P->lev[l].tc && !(p2l && l == L) && !(l == L && P->m2p)) ls[n++] = l;
+      if ((!P->lev[l].tc || P->refl_on(l)) && !(p2l && l == L) && !(l == L && P->m2p)) ls[n++] = l;
     const std::vector<std::vector<int>> groups = row_groups(P, ls, n);
     for (const std::vector<int>& gr : groups) {
       StageTimer t(P, ST_M2L, sf);
@@ -2778,7 +2826,7 @@ fmm_status run_solve(fmm_plan_t P, const T* rho, T* phi, T* accel, cudaStream_t 
   }
   if (fork) CUDA_TRY(cudaEventRecord(P->ev_join, sf));
   for (int l = 2; l <= L; ++l) {
-    if (!P->lev[l].tc || (p2l && l == L)) continue;
+    if (!P->lev[l].tc || P->refl_on(l) || (p2l && l == L)) continue;
     StageTimer t(P, ST_M2L_TC, s);
     if ((st = (l == L && P->m2p) ? do_m2p(P, s) : do_m2l(P, l, s))) return st;
   }
@@ -2838,7 +2886,7 @@ fmm_status run_solve(fmm_plan_t P, const T* rho, T* phi, T* accel, cudaStream_t 
       da.par = P->lev[L - 1];
       da.Lp = static_cast<const T*>(P->Lx(L - 1));
       da.harm = harmonic_m2l_level(P, L) ? 1 : 0;
-      da.Lred = da.harm && P->lev[L].lred_off ? reinterpret_cast<const T*>(P->arena + P->lev[L].lred_off) : nullptr;
+      da.Lred = da.harm ? static_cast<const T*>(red_rows(P, L)) : nullptr;
     }
     CUDA_TRY(launch_leaf_finish<T>(tt, P->lev[L], static_cast<const T*>(P->Lx(L)), adj_g ? rho_box : near_box,
                                    P->b * P->b * P->b * (adj_g ? 1 : P->near_comps),
@@ -3053,7 +3101,7 @@ int fmm_solve_launches(fmm_plan_t P, int with_accel) {
     if (rows_level(P, l) && !(l == L && P->m2p)) n -= 2;  // grouped: counted below (M2L and its reduction)
     if (l == 2 && harmonic_m2l_level(P, 2)) n += 1;  // rebuild of the harmonic level-2 locals
     if (l == 2 && L == 2 && P->m2p) n += 1;          // zero leaf locals (final-stage M2P, no parent far field)
-    if (!P->lev[l].tc && P->m2l_choice[l].dsplit > 1 && !(l == L && P->m2p)) n += 1;  // partial-sum reduction
+    if ((!P->lev[l].tc || P->refl_on(l)) && P->m2l_choice[l].dsplit > 1 && !(l == L && P->m2p)) n += 1;  // partial-sum reduction
   }
   {
     int ls[kMaxLevels], k = 0, nn = 0;
@@ -3143,7 +3191,7 @@ fmm_status fmm_debug_level(fmm_plan_t P, int what, int level, double* host_out, 
     if (e == cudaSuccess) e = cudaMemcpy(full, P->Lx(level), lv.bytes, cudaMemcpyDeviceToDevice);
     const Level& q = P->lev[level - 1];
     const int harm = harmonic_m2l_level(P, level) ? 1 : 0;
-    const void* red = harm && lv.lred_off ? P->arena + lv.lred_off : nullptr;
+    const void* red = harm ? red_rows(P, level) : nullptr;
     if (e == cudaSuccess)
       e = lv.f64 ? launch_l2l<double, double>(P->tables(), q, static_cast<const double*>(P->Lx(level - 1)), lv,
                                               static_cast<double*>(full), 1, harm, static_cast<const double*>(red), 0)
@@ -3955,6 +4003,12 @@ fmm_status tune_tc(fmm_plan_t P, int what, cudaStream_t s) {
   char key[160];
   std::snprintf(key, sizeof key, "tc%d/%d,%d,%d/%d/%d/%d/%d/%d", what, g[0], g[1], g[2], P->p, P->b, P->tc_kind,
                 P->harm ? 1 : 0, P->near_comps);
+  struct Refl {  // the timed launches are the tensor-core schedules' own
+    fmm_plan_t P;
+    bool was;
+    ~Refl() { P->refl_now = was; }
+  } refl{P, P->refl_now};
+  if (what == TS_M2L) P->refl_now = false;
   // candidate c: 0 span, 1 prefix, 2 the dedicated near-field kernel
   auto select = [&](int c) {
     P->use_tp[what] = c == 1;
@@ -4068,6 +4122,7 @@ extern "C" fmm_status fmm_plan_set_tc_schedule(fmm_plan_t P, int what, int prefi
   if (what == TS_M2L && P->asym && !(prefix ? P->tp_m2l_t : P->span_m2l_t))
     return fail(FMM_ERR_ARG, "the transposed M2L has no %s schedule", prefix ? "prefix" : "span");
   P->use_tp[what] = prefix != 0;
+  if (what == TS_M2L) P->use_refl = P->refl_now = false;  // every tensor-core level on that schedule
   if (what == TS_NEAR) P->use_near4 = false;
   return FMM_OK;
 }

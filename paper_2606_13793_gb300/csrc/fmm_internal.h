@@ -58,6 +58,9 @@ struct Level {
   // M2L's c <= 1 locals (rows of 8 (p+1)^2 values), in the level's type; TF32
   // levels: folded rows (0: none)
   size_t fold_off, lred_off;
+  // tensor-core bf16x3 level whose row tiles do not fill the GPU: the same two
+  // arrays of its reflection-basis form (0: none)
+  size_t rfold_off = 0, rred_off = 0;
 };
 
 // One item of a multi-item launch (multi.cuh): its grid of blocks and the
