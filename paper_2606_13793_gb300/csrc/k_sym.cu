@@ -123,6 +123,34 @@ __device__ __forceinline__ void sy_step(const double (&v)[HV], int uo, int lo, d
   }
 }
 
+// v[z] = (uu + fx lu) + fy (ul + fx ll): one (x, y) mirror pair of a halo
+// column, z in 16-byte pieces.
+template <int HV>
+__device__ __forceinline__ void sy_column(float (&v)[HV], const float* uu, const float* lu, const float* ul,
+                                          const float* ll, float fx, float fy) {
+  static_assert(HV % 4 == 0, "whole 16-byte pieces");
+  const unsigned long long fx2 = sy_pack(fx, fx), fy2 = sy_pack(fy, fy);
+#pragma unroll
+  for (int z = 0; z < HV; z += 4) {
+    const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(uu + z), b = *reinterpret_cast<const ulonglong2*>(lu + z);
+    const ulonglong2 c = *reinterpret_cast<const ulonglong2*>(ul + z), d = *reinterpret_cast<const ulonglong2*>(ll + z);
+    const float2 p = sy_unpack(sy_fma2(fy2, sy_fma2(fx2, d.x, c.x), sy_fma2(fx2, b.x, a.x)));
+    const float2 q = sy_unpack(sy_fma2(fy2, sy_fma2(fx2, d.y, c.y), sy_fma2(fx2, b.y, a.y)));
+    v[z] = p.x, v[z + 1] = p.y, v[z + 2] = q.x, v[z + 3] = q.y;
+  }
+}
+template <int HV>
+__device__ __forceinline__ void sy_column(double (&v)[HV], const double* uu, const double* lu, const double* ul,
+                                          const double* ll, double fx, double fy) {
+#pragma unroll
+  for (int z = 0; z < HV; z += 2) {
+    const double2 a = *reinterpret_cast<const double2*>(uu + z), b = *reinterpret_cast<const double2*>(lu + z);
+    const double2 c = *reinterpret_cast<const double2*>(ul + z), d = *reinterpret_cast<const double2*>(ll + z);
+    v[z] = fma(fy, fma(fx, d.x, c.x), fma(fx, b.x, a.x));
+    v[z + 1] = fma(fy, fma(fx, d.y, c.y), fma(fx, b.y, a.y));
+  }
+}
+
 template <typename T>
 __device__ __forceinline__ void cp_async_elt(T* dst, const T* src, bool ok) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
@@ -161,21 +189,31 @@ __device__ __forceinline__ void sy_unfold(T (&v)[8], int p) {
 
 // ------------------------------------------------------------ M2L, z-run --
 
-// Halo of one component's child values: (8 + 2) x (4 + 2) x (RZ + 2) parents,
-// stored [jz][cx][jy][bx] with a row pitch of 12 so that a warp's 8 x 4 lanes
-// (x stride 1, y stride 24) hit 32 banks.
-constexpr int kMlPitch = 12;
-constexpr int kMlX = 12 * kMlPitch;  // stride of the child's x bit
-constexpr int kMlZ = 2 * kMlX;       // stride of jz
-constexpr int kMlStages = 3;
-template <int RZ>
-constexpr int sy_ml_raw() {
-  return (2 * (RZ + 2)) * kMlZ;
+// A halo column's values lie along z, so a lane reads its z-run in 16-byte
+// pieces; the pitch of a column keeps the 8 lanes of a quarter warp (adjacent
+// columns) in different banks: a multiple of 16 bytes, 12 or 20 mod 32 words
+// (or 4 or 28).
+template <typename T>
+constexpr int sy_pitch(int hv) {
+  constexpr int V = 16 / (int)sizeof(T);  // values per 16 bytes
+  int p = (hv + V - 1) / V * V;
+  while ((p / V) % 2 == 0) p += V;  // an odd number of pieces
+  return p;
 }
+
+// Halo of one component's child values: (8 + 2) x (4 + 2) x (RZ + 2) parents,
+// stored [cx][jy][bx][jz].
+constexpr int kMlStages = 3;
+template <typename T, int RZ>
+struct MlHalo {
+  static constexpr int pz = sy_pitch<T>(2 * (RZ + 2));
+  static constexpr int y = 10 * pz, x = 12 * y;  // strides of jy and of the child's x bit
+  static constexpr int size = 2 * x;
+};
 constexpr int kMlW = 9 * 4 * 3 * 8 * 2;  // weights of one component: 9 (x, y) pairs, 8 columns
 template <typename T, int RZ>
 constexpr size_t sym_m2l_smem() {
-  return sizeof(T) * (size_t)kMlStages * (sy_ml_raw<RZ>() + kMlW);
+  return sizeof(T) * (size_t)kMlStages * (MlHalo<T, RZ>::size + kMlW);
 }
 
 template <typename T, int RZ, int NL>
@@ -184,15 +222,12 @@ __device__ __forceinline__ void sy_ml_component(const T* raw, const T* W, int xy
   constexpr int HV = 2 * (RZ + 2);
   for (int j = nxy - 1; j >= 0; --j) {  // far pairs first
     const int xy = xy0 + j, kx = xy % 3, ky = xy / 3;
-    const int xu = ((3 + kx) & 1) * kMlX + xl + ((3 + kx) >> 1), xlo = ((2 - kx) & 1) * kMlX + xl + ((2 - kx) >> 1);
-    const int yu = (2 * yl + 3 + ky) * kMlPitch, ylo = (2 * yl + 2 - ky) * kMlPitch;
-    const T *puu = raw + xu + yu, *plu = raw + xlo + yu, *pul = raw + xu + ylo, *pll = raw + xlo + ylo;
+    using H = MlHalo<T, RZ>;
+    const int xu = ((3 + kx) & 1) * H::x + (xl + ((3 + kx) >> 1)) * H::pz;
+    const int xlo = ((2 - kx) & 1) * H::x + (xl + ((2 - kx) >> 1)) * H::pz;
+    const int yu = (2 * yl + 3 + ky) * H::y, ylo = (2 * yl + 2 - ky) * H::y;
     T v[HV];
-#pragma unroll
-    for (int z = 0; z < HV; ++z) {
-      const T a = fma(fx, plu[z * kMlZ], puu[z * kMlZ]), b = fma(fx, pll[z * kMlZ], pul[z * kMlZ]);
-      v[z] = fma(fy, b, a);
-    }
+    sy_column<HV>(v, raw + xu + yu, raw + xlo + yu, raw + xu + ylo, raw + xlo + ylo, fx, fy);
     const T* w = W + j * (4 * 3 * NL * 2);
 #pragma unroll
     for (int kz = 2; kz >= 0; --kz) {
@@ -206,7 +241,8 @@ template <typename T, int RZ>
 __device__ __forceinline__ void sym_m2l_body(const NbrGemm& g, const VBlock& vb) {
   extern __shared__ __align__(16) unsigned char sy_smem[];
   T* sm = reinterpret_cast<T*>(sy_smem);
-  constexpr int kRaw = sy_ml_raw<RZ>(), kStage = kRaw + kMlW;
+  using H = MlHalo<T, RZ>;
+  constexpr int kRaw = H::size, kStage = kRaw + kMlW;
   constexpr int kPos = (RZ + 2) * 60, kNp = (kPos + kSyThreads - 1) / kSyThreads;
   const SymTab& st = *g.st;
   const int u = (int)vb.y;
@@ -227,7 +263,7 @@ __device__ __forceinline__ void sym_m2l_body(const NbrGemm& g, const VBlock& vb)
     const int e = t + i * kSyThreads;
     const int bx = e % 10, by = (e / 10) % 6, bz = e / 60;
     const int x = ox + bx - 1, y = oy + by - 1, z = oz + bz - 1;
-    soff[i] = e < kPos ? bz * 2 * kMlZ + by * 2 * kMlPitch + bx : -1;
+    soff[i] = e < kPos ? by * 2 * H::y + bx * H::pz + bz * 2 : -1;
     goff[i] = (x >= 0 && y >= 0 && z >= 0 && x < g.grid[0] && y < g.grid[1] && z < g.grid[2])
                   ? (z * g.grid[1] + y) * g.grid[0] + x
                   : -1;
@@ -241,7 +277,7 @@ __device__ __forceinline__ void sym_m2l_body(const NbrGemm& g, const VBlock& vb)
       const T* Aa = A + (long long)a * 8 * g.lda;
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
-        T* d = stg + (c >> 2) * kMlZ + ((c >> 1) & 1) * kMlPitch + (c & 1) * kMlX;
+        T* d = stg + (c >> 2) + ((c >> 1) & 1) * H::y + (c & 1) * H::x;
 #pragma unroll
         for (int e = 0; e < kNp; ++e)
           if (soff[e] >= 0) cp_async_elt(d + soff[e], Aa + (goff[e] < 0 ? 0 : goff[e]), goff[e] >= 0);
@@ -320,30 +356,32 @@ __device__ __forceinline__ void sym_m2l_body(const NbrGemm& g, const VBlock& vb)
 }
 
 template <typename T, int RZ>
-__global__ void __launch_bounds__(kSyThreads, sizeof(T) == 4 ? 2 : 1) sym_m2l_kernel(NbrGemm g) {
+__global__ void __launch_bounds__(kSyThreads, sizeof(T) == 4 ? (RZ <= 4 ? 3 : 2) : 1) sym_m2l_kernel(NbrGemm g) {
   sym_m2l_body<T, RZ>(g, native_vblock());
 }
 
 // ----------------------------------------------------- near field, leaf 4 --
 
 // Halo of the density: (8 + 2) x (4 + 2) x (RZ + 2) boxes, stored
-// [jz][cx][jy][bx]: a warp's lanes (x stride 1, y stride 40) hit 32 banks.
-constexpr int kNfY = 10, kNfX = 24 * kNfY, kNfZ = 4 * kNfX;
+// [cx][jy][bx][jz] like the M2L's.
+template <typename T, int RZ>
+struct NfHalo {
+  static constexpr int pz = sy_pitch<T>(4 * (RZ + 2));
+  static constexpr int y = 10 * pz, x = 24 * y;
+  static constexpr int size = 4 * x;
+};
 constexpr int kNfW = 36 * 4 * 6 * 8 * 2;
-template <int RZ>
-constexpr int sy_nf_raw() {
-  return 4 * (RZ + 2) * kNfZ;
-}
 template <typename T>
 constexpr bool kNfSmemW = sizeof(T) == 4;  // FP64: the weights stay in L1 / L2 (the DFMA pipe is the limit)
 template <typename T, int RZ>
 constexpr size_t sym_near4_smem() {
-  return sizeof(T) * ((size_t)sy_nf_raw<RZ>() + (kNfSmemW<T> ? kNfW : 0));
+  return sizeof(T) * ((size_t)NfHalo<T, RZ>::size + (kNfSmemW<T> ? kNfW : 0));
 }
 
 template <typename T, int RZ>
 __device__ __forceinline__ void sym_near4_body(const NbrGemm& g, const VBlock& vb) {
   extern __shared__ __align__(16) unsigned char sy_smem[];
+  using H = NfHalo<T, RZ>;
   T* raw = reinterpret_cast<T*>(sy_smem);
   if (vb.y) return;  // the launch has one block row per 32 columns; this form computes all 64 in one
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -355,7 +393,7 @@ __device__ __forceinline__ void sym_near4_body(const NbrGemm& g, const VBlock& v
   const T* A = static_cast<const T*>(g.A);
   const T* W = static_cast<const T*>(g.Ws);
   if constexpr (kNfSmemW<T>) {
-    T* Wsm = raw + sy_nf_raw<RZ>();
+    T* Wsm = raw + H::size;
     const char* src = reinterpret_cast<const char*>(W + xy0 * 384);
     for (int i = t * 16; i < nxy * 384 * (int)sizeof(T); i += kSyThreads * 16)
       cp_async16(reinterpret_cast<char*>(Wsm) + i, src + i);
@@ -374,7 +412,7 @@ __device__ __forceinline__ void sym_near4_body(const NbrGemm& g, const VBlock& v
       const bool in = x >= 0 && y >= 0 && z >= 0 && x < g.grid[0] && y < g.grid[1] && z < g.grid[2];
       const uint4* src =
           reinterpret_cast<const uint4*>(A + (in ? (((long long)z * g.grid[1] + y) * g.grid[0] + x) * 64 : 0));
-      T* dst = raw + bz * 4 * kNfZ + by * 4 * kNfY + bx;
+      T* dst = raw + by * 4 * H::y + bx * H::pz + bz * 4;
 #pragma unroll
       for (int q0 = 0; q0 < PB; q0 += 8) {
         uint4 v[8];
@@ -386,7 +424,7 @@ __device__ __forceinline__ void sym_near4_body(const NbrGemm& g, const VBlock& v
 #pragma unroll
           for (int i = 0; i < VN; ++i) {
             const int cell = (q0 + q) * VN + i;  // x fastest
-            dst[(cell >> 4) * kNfZ + (cell & 3) * kNfX + ((cell >> 2) & 3) * kNfY] = pv[i];
+            dst[(cell >> 4) + (cell & 3) * H::x + ((cell >> 2) & 3) * H::y] = pv[i];
           }
         }
       }
@@ -400,15 +438,11 @@ __device__ __forceinline__ void sym_near4_body(const NbrGemm& g, const VBlock& v
   SyAcc<T> acc[RZ][8];
   for (int j = nxy - 1; j >= 0; --j) {  // far pairs (small weights) first
     const int xy = xy0 + j, kx = xy % 6, ky = xy / 6;
-    const int xu = ((2 + kx) & 3) * kNfX + xl + 1 + ((2 + kx) >> 2), xlo = ((5 - kx) & 3) * kNfX + xl + ((5 - kx) >> 2);
-    const int yu = (4 * yl + 6 + ky) * kNfY, ylo = (4 * yl + 5 - ky) * kNfY;
-    const T *puu = raw + xu + yu, *plu = raw + xlo + yu, *pul = raw + xu + ylo, *pll = raw + xlo + ylo;
+    const int xu = ((2 + kx) & 3) * H::x + (xl + 1 + ((2 + kx) >> 2)) * H::pz;
+    const int xlo = ((5 - kx) & 3) * H::x + (xl + ((5 - kx) >> 2)) * H::pz;
+    const int yu = (4 * yl + 6 + ky) * H::y, ylo = (4 * yl + 5 - ky) * H::y;
     T v[HV];
-#pragma unroll
-    for (int z = 0; z < HV; ++z) {
-      const T a = fma(fx, plu[z * kNfZ], puu[z * kNfZ]), b = fma(fx, pll[z * kNfZ], pul[z * kNfZ]);
-      v[z] = fma(fy, b, a);
-    }
+    sy_column<HV>(v, raw + xu + yu, raw + xlo + yu, raw + xu + ylo, raw + xlo + ylo, fx, fy);
     const T* w = W + j * 384 + warp * 96;
 #pragma unroll
     for (int kz = 5; kz >= 0; --kz) sy_step<RZ, 8, 8, 4, HV>(v, 6 + kz, 5 - kz, T(1), w + kz * 16, acc);
@@ -741,7 +775,7 @@ __global__ void __launch_bounds__(kSyTinyThreads)
 
 // Items of one launch: blocks [first, first + gridDim.x) of the step.
 template <typename T, int RZ>
-__global__ void __launch_bounds__(kSyThreads, sizeof(T) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(kSyThreads, sizeof(T) == 4 ? (RZ <= 4 ? 3 : 2) : 1)
     sym_m2l_multi_kernel(const NbrGemm* __restrict__ gs, const MultiGrid* __restrict__ grids, int n, long long first) {
   __shared__ NbrGemm g;
   const long long b = (long long)blockIdx.x + first;
