@@ -3320,6 +3320,8 @@ struct MultiStep {
   // MK_GEMM: items and blocks of each kind, in this order (one launch each):
   // reflection-basis M2L, reflection-basis leaf-4 near field, direct form
   int kn[3] = {0, 0, 0};
+  int ny[3] = {0, 0, 0};  // the kind's common gy (column tiles), 0 if its items differ
+  int nx[3] = {0, 0, 0};  // and gx (the tiny form's column tiles)
   long long kb[3] = {0, 0, 0};
 };
 }  // namespace
@@ -3533,6 +3535,9 @@ void build_fused(fmm_batch_t B, const void* const* rho, void* const* phi, void* 
       for (int k = 0; k < 3; ++k)
         for (const std::array<unsigned, 3>& x : g[sh][k]) {
           const long long nb = (long long)x[0] * x[1] * x[2];
+          if (nb > 0) st.ny[k] = st.kn[k] == 0 || st.ny[k] == (int)x[1] ? (int)x[1] : 0;
+          if (x[2] != 1) st.ny[k] = 0;
+          if (nb > 0) st.nx[k] = st.kn[k] == 0 || st.nx[k] == (int)x[0] ? (int)x[0] : 0;
           st.kn[k] += nb > 0;
           st.kb[k] += nb;
         }
@@ -3649,23 +3654,29 @@ fmm_status run_fused(fmm_batch_t B, cudaStream_t s) {
       case MK_GEMM: {
         const NbrGemm* gs = static_cast<const NbrGemm*>(a);
         const int zs = st.shape == 5 ? 2 : st.shape == 4 ? 3 : st.shape - 1;
+        // The direct items first: their few long blocks then run beside the other
+        // shapes' launches (after the near field, whose CTAs take an SM each,
+        // they ran alone: the 16-field contractions 1.83 ms).
+        {
+          const NbrGemm* ds = gs + st.kn[0] + st.kn[1];
+          const MultiGrid* dg = g + st.kn[0] + st.kn[1];
+          const int n = st.kn[2];
+          const long long nb = st.kb[2], first = st.kb[0] + st.kb[1];
+          if (st.shape == 4)
+            e = launch_nbr_gemm_tiny_multi<T>(ds, dg, n, nb, ls, first, st.nx[2]);
+          else if (st.shape == 0)
+            e = launch_nbr_gemm_simt_multi<T>(ds, dg, n, nb, ls);
+          else if (st.shape == 3)
+            e = launch_nbr_gemm_col_multi<T>(ds, dg, n, nb, ls);
+          else
+            e = launch_nbr_gemm_zrun_multi<T>(zs, ds, dg, n, nb, ls, first, st.ny[2]);
+        }
         for (int k = 0; k < 2 && e == cudaSuccess; ++k) {  // reflection-basis items: M2L, near field
           e = launch_nbr_gemm_sym_multi<T>(zs, k == 0 ? kSymM2l : kSymNear4, gs, g, st.kn[k], st.kb[k],
-                                           k == 0 ? 0 : st.kb[0], ls);
+                                           k == 0 ? 0 : st.kb[0], st.ny[k], ls);
           gs += st.kn[k];
           g += st.kn[k];
         }
-        if (e != cudaSuccess) break;
-        const int n = st.kn[2];  // direct form
-        const long long nb = st.kb[2], first = st.kb[0] + st.kb[1];
-        if (st.shape == 4)
-          e = launch_nbr_gemm_tiny_multi<T>(gs, g, n, nb, ls, first);
-        else if (st.shape == 0)
-          e = launch_nbr_gemm_simt_multi<T>(gs, g, n, nb, ls);
-        else if (st.shape == 3)
-          e = launch_nbr_gemm_col_multi<T>(gs, g, n, nb, ls);
-        else
-          e = launch_nbr_gemm_zrun_multi<T>(zs, gs, g, n, nb, ls, first);
         break;
       }
       case MK_L2L:

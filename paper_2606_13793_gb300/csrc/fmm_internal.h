@@ -145,9 +145,11 @@ cudaError_t launch_nbr_gemm_sym_rows(const NbrGemm* gs, int n, cudaStream_t s);
 // Multi-item forms over the items of one kind: blocks [first, first + blocks)
 // of the step's block ranges.  shape as launch_nbr_gemm_zrun_multi, or 3: the
 // tiny-grid form (at most 64 rows, one block per 32 columns; kSymM2l only).
+// ny: the items' common number of column tiles (tile-major block order,
+// multi.cuh), 0 if they differ.
 template <typename T>
 cudaError_t launch_nbr_gemm_sym_multi(int shape, int kind, const NbrGemm* gs, const MultiGrid* grids, int n,
-                                      long long blocks, long long first, cudaStream_t s);
+                                      long long blocks, long long first, int ny, cudaStream_t s);
 
 template <typename T>
 cudaError_t launch_nbr_gemm_simt(const NbrGemm& g, cudaStream_t s);
@@ -174,15 +176,16 @@ cudaError_t launch_nbr_gemm_col_multi(const NbrGemm* gs, const MultiGrid* grids,
 // shape here: 0 / 1 as launch_nbr_gemm_zrun, 2 = a z run of 6 rows (FP32; 3 in FP64)
 template <typename T>
 cudaError_t launch_nbr_gemm_zrun_multi(int shape, const NbrGemm* gs, const MultiGrid* grids, int n, long long blocks,
-                                       cudaStream_t s, long long first = 0);
+                                       cudaStream_t s, long long first = 0, int ny = 0);
 template <typename T>
 void nbr_gemm_simt_col_grid(const NbrGemm& g, unsigned out[3]);
 // Grids of at most 64 rows (nbr_gemm_tiny_fits): one block per column tile
-// (an item's grid is ntiles x 1 x 1), in-grid neighbours only.
+// (an item's grid is ntiles x 1 x 1), in-grid neighbours only.  nx: the items'
+// common ntiles, 0 if they differ.
 bool nbr_gemm_tiny_fits(const NbrGemm& g);
 template <typename T>
 cudaError_t launch_nbr_gemm_tiny_multi(const NbrGemm* gs, const MultiGrid* grids, int n, long long blocks,
-                                       cudaStream_t s, long long first = 0);
+                                       cudaStream_t s, long long first = 0, int nx = 0);
 template <typename T>
 void nbr_gemm_zrun_grid(const NbrGemm& g, int shape, unsigned out[3]);
 // C (+)= sum over nparts partial arrays of count values, in part order.

@@ -226,14 +226,43 @@ __global__ void __launch_bounds__(128) nbr_gemm_col_multi_kernel(const NbrGemm* 
 // summing over the in-grid neighbours only.  The level's useful
 // multiply-adds are few; the general tiles would spend most of theirs on
 // padded rows and out-of-grid neighbours, and their staged reduction chunks
-// (two barriers each) would set a long latency for little work.  No shared
-// memory: the rows and weights of such a level stay in L1 / L2.
+// (two barriers each) would set a long latency for little work.  The level's
+// rows (the tile's prefix of them) sit in shared memory where they fit: read
+// from L1 by every thread, four rows a warp, they made the blocks
+// wavefront-bound (565 us for the 416 blocks of 16 fields at order 6).
 // The reduction is split into kTinyKS parts over as many groups of 256
 // threads, added in part order at the end: the blocks are latency-bound, and
 // this divides their length.
 constexpr int kTinyRows = 64;
 constexpr int kTinyKS = 4;
 constexpr int kTinyThreads = 256 * kTinyKS;  // per part: 32 row pairs x 8 column groups of 4
+constexpr size_t kTinySmem = 170 * 1024;     // rows: 64 x (648 + 1) floats (order 8, harmonic) fit
+
+// acc += a_r[k] w[k][0..3] for the two rows, k in order.
+template <typename T>
+__device__ __forceinline__ void tiny_steps(const T* a0p, const T* a1p, bool v0, bool v1, const T* w, int k0, int k1,
+                                           T (&acc)[2][4]) {
+#pragma unroll 4
+  for (int k = k0; k < k1; ++k) {
+    const T* wk = w + (long long)k * kNTile;
+    T w0, w1, w2, w3;
+    if constexpr (sizeof(T) == 4) {
+      const float4 q = __ldg(reinterpret_cast<const float4*>(wk));
+      w0 = q.x, w1 = q.y, w2 = q.z, w3 = q.w;
+    } else {
+      w0 = __ldg(wk), w1 = __ldg(wk + 1), w2 = __ldg(wk + 2), w3 = __ldg(wk + 3);
+    }
+    const T a0 = v0 ? a0p[k] : T(0), a1 = v1 ? a1p[k] : T(0);
+    acc[0][0] = fma(a0, w0, acc[0][0]);
+    acc[0][1] = fma(a0, w1, acc[0][1]);
+    acc[0][2] = fma(a0, w2, acc[0][2]);
+    acc[0][3] = fma(a0, w3, acc[0][3]);
+    acc[1][0] = fma(a1, w0, acc[1][0]);
+    acc[1][1] = fma(a1, w1, acc[1][1]);
+    acc[1][2] = fma(a1, w2, acc[1][2]);
+    acc[1][3] = fma(a1, w3, acc[1][3]);
+  }
+}
 
 template <typename T>
 __device__ __forceinline__ void nbr_gemm_tiny_body(const NbrGemm& g, const VBlock vb) {
@@ -247,6 +276,18 @@ __device__ __forceinline__ void nbr_gemm_tiny_body(const NbrGemm& g, const VBloc
   const int k0 = kp * Kq, k1 = min(Kt, k0 + Kq);
   const T* W0 = static_cast<const T*>(g.W) + g.tile_w[tile] + cq * 4;
   const T* A = static_cast<const T*>(g.A);
+  extern __shared__ __align__(16) unsigned char tiny_smem[];
+  T* As = reinterpret_cast<T*>(tiny_smem);
+  // an odd pitch: the four rows of a warp in different banks
+  const int pitch = Kt | 1;
+  const bool staged = (size_t)R * pitch * sizeof(T) <= kTinySmem;
+  if (staged) {
+    for (int e = threadIdx.x; e < R * Kt; e += kTinyThreads) {
+      const int r = e / Kt, k = e - r * Kt;
+      As[r * pitch + k] = __ldg(A + (long long)r * g.row_len + k);
+    }
+    __syncthreads();
+  }
   T acc[2][4];
   int rx[2], ry[2], rz[2];
   bool live[2];
@@ -265,28 +306,19 @@ __device__ __forceinline__ void nbr_gemm_tiny_body(const NbrGemm& g, const VBloc
     if (d == 13 && g.skip_center) continue;  // the centre block is zero
     const int dx = d % 3 - 1, dy = (d / 3) % 3 - 1, dz = d / 9 - 1;
     bool v[2];
-    const T* ap[2];
+    int nr[2];
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       const int x = rx[i] + dx, y = ry[i] + dy, z = rz[i] + dz;
       v[i] = live[i] && x >= 0 && y >= 0 && z >= 0 && x < g.grid[0] && y < g.grid[1] && z < g.grid[2];
-      ap[i] = A + (v[i] ? ((long long)(z * g.grid[1] + y) * g.grid[0] + x) * g.row_len : 0);
+      nr[i] = v[i] ? (z * g.grid[1] + y) * g.grid[0] + x : 0;
     }
     if (!v[0] && !v[1]) continue;
     const T* w = W0 + (long long)d * Kt * kNTile;
-    for (int k = k0; k < k1; ++k) {
-      const T* wk = w + (long long)k * kNTile;
-      const T w0 = __ldg(wk), w1 = __ldg(wk + 1), w2 = __ldg(wk + 2), w3 = __ldg(wk + 3);
-      const T a0 = v[0] ? __ldg(ap[0] + k) : T(0), a1 = v[1] ? __ldg(ap[1] + k) : T(0);
-      acc[0][0] = fma(a0, w0, acc[0][0]);
-      acc[0][1] = fma(a0, w1, acc[0][1]);
-      acc[0][2] = fma(a0, w2, acc[0][2]);
-      acc[0][3] = fma(a0, w3, acc[0][3]);
-      acc[1][0] = fma(a1, w0, acc[1][0]);
-      acc[1][1] = fma(a1, w1, acc[1][1]);
-      acc[1][2] = fma(a1, w2, acc[1][2]);
-      acc[1][3] = fma(a1, w3, acc[1][3]);
-    }
+    if (staged)
+      tiny_steps<T>(As + nr[0] * pitch, As + nr[1] * pitch, v[0], v[1], w, k0, k1, acc);
+    else
+      tiny_steps<T>(A + (long long)nr[0] * g.row_len, A + (long long)nr[1] * g.row_len, v[0], v[1], w, k0, k1, acc);
   }
   if (kTinyKS > 1) {  // parts 1 .. KS-1 hand their sums to part 0, which adds them in order
     if (kp > 0) {
@@ -321,13 +353,18 @@ __device__ __forceinline__ void nbr_gemm_tiny_body(const NbrGemm& g, const VBloc
 template <typename T>
 __global__ void __launch_bounds__(kTinyThreads) nbr_gemm_tiny_multi_kernel(const NbrGemm* __restrict__ gs,
                                                                            const MultiGrid* __restrict__ grids,
-                                                                           int n, long long first) {
+                                                                           int n, long long first, int nx) {
   __shared__ NbrGemm g;  // the item's description, read by the body from shared memory
   const long long b = (long long)blockIdx.x + first;
-  const int i = multi_item_at(grids, n, b);
+  int i = multi_item_at(grids, n, b);
+  VBlock vb = multi_vblock_at(grids[i], b);
+  if (nx > 0) {  // items of nx tiles each: the long first tiles of all of them first
+    i = (int)(blockIdx.x % n);
+    vb.x = blockIdx.x / n;
+  }
   if (threadIdx.x == 0) g = gs[i];
   __syncthreads();
-  nbr_gemm_tiny_body<T>(g, multi_vblock_at(grids[i], b));
+  nbr_gemm_tiny_body<T>(g, vb);
 }
 
 // C (+)= sum over the neighbour-group partials, in group order.
@@ -411,10 +448,17 @@ cudaError_t launch_nbr_gemm_col_multi(const NbrGemm* gs, const MultiGrid* grids,
 
 template <typename T>
 cudaError_t launch_nbr_gemm_tiny_multi(const NbrGemm* gs, const MultiGrid* grids, int n, long long blocks,
-                                       cudaStream_t s, long long first) {
+                                       cudaStream_t s, long long first, int nx) {
   if (n <= 0 || blocks <= 0) return cudaSuccess;
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  nbr_gemm_tiny_multi_kernel<T><<<(unsigned)blocks, kTinyThreads, 0, s>>>(gs, grids, n, first);
+  static bool attr = false;
+  if (!attr) {
+    const cudaError_t e = cudaFuncSetAttribute(nbr_gemm_tiny_multi_kernel<T>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTinySmem);
+    if (e != cudaSuccess) return e;
+    attr = true;
+  }
+  nbr_gemm_tiny_multi_kernel<T><<<(unsigned)blocks, kTinyThreads, kTinySmem, s>>>(gs, grids, n, first, nx);
   return cudaGetLastError();
 }
 
@@ -440,9 +484,9 @@ template cudaError_t launch_nbr_gemm_simt_multi<double>(const NbrGemm*, const Mu
 template cudaError_t launch_nbr_gemm_col_multi<float>(const NbrGemm*, const MultiGrid*, int, long long, cudaStream_t);
 template cudaError_t launch_nbr_gemm_col_multi<double>(const NbrGemm*, const MultiGrid*, int, long long, cudaStream_t);
 template cudaError_t launch_nbr_gemm_tiny_multi<float>(const NbrGemm*, const MultiGrid*, int, long long, cudaStream_t,
-                                                       long long);
+                                                       long long, int);
 template cudaError_t launch_nbr_gemm_tiny_multi<double>(const NbrGemm*, const MultiGrid*, int, long long, cudaStream_t,
-                                                        long long);
+                                                        long long, int);
 template void nbr_gemm_simt_col_grid<float>(const NbrGemm&, unsigned[3]);
 template void nbr_gemm_simt_col_grid<double>(const NbrGemm&, unsigned[3]);
 template cudaError_t launch_nbr_gemm_simt<float>(const NbrGemm&, cudaStream_t);

@@ -241,13 +241,17 @@ __global__ void __launch_bounds__(kZrThreads, 4) nbr_gemm_zrun_multi_kernel(cons
 // against 18 per 48).  Every output adds the same products in the same order
 // as the wide form: the results are its, bit for bit.
 template <int RZ>
-__device__ __forceinline__ void zrun_narrow_body(const NbrGemm& g, const VBlock& vb, int cg) {
+constexpr int narrow_smem() {  // floats
+  return 27 * kZrKC * 8 + kZrKC * ZrHalo<RZ>::stride;
+}
+template <int RZ>
+__device__ __forceinline__ void zrun_narrow_body(const NbrGemm& g, const VBlock& vb, int cg, float* sm) {
   using H = ZrHalo<RZ>;
   constexpr int HR = RZ / 2;
   constexpr int kA = (H::rows * 2 + kZrThreads - 1) / kZrThreads;  // float4 of A per thread and stage
   constexpr int kW = (27 * kZrKC * 2 + kZrThreads - 1) / kZrThreads;
-  __shared__ __align__(16) float As[kZrKC * H::stride];
-  __shared__ __align__(16) float Ws[27 * kZrKC * 8];
+  float* Ws = sm;                   // [27 neighbours][kZrKC][8]
+  float* As = sm + 27 * kZrKC * 8;  // [kZrKC][H::stride]
   const int t = threadIdx.x;
   const int xr = t & 7, yr = (t >> 3) & 3, zh = (t >> 5) & 1, cq = t >> 6;
   const int ntx = (g.grid[0] + kZrBX - 1) / kZrBX, nty = (g.grid[1] + kZrBY - 1) / kZrBY;
@@ -345,30 +349,41 @@ __device__ __forceinline__ void zrun_narrow_body(const NbrGemm& g, const VBlock&
 template <int RZ>
 __global__ void __launch_bounds__(kZrThreads) zrun_narrow_multi_kernel(const NbrGemm* __restrict__ gs,
                                                                        const MultiGrid* __restrict__ grids, int n,
-                                                                       long long first) {
+                                                                       long long first, int ny) {
   __shared__ NbrGemm g;
-  const long long b = (long long)(blockIdx.x >> 2) + first;
-  const int it = multi_item_at(grids, n, b);
+  VBlock vb;
+  const int it = multi_tile_major(grids, n, first, gridDim.x >> 2, ny, blockIdx.x >> 2, &vb);
   if (threadIdx.x == 0) g = gs[it];
   __syncthreads();
-  zrun_narrow_body<RZ>(g, multi_vblock_at(grids[it], b), blockIdx.x & 3);
+  __shared__ __align__(16) float sm[narrow_smem<RZ>()];
+  zrun_narrow_body<RZ>(g, vb, blockIdx.x & 3, sm);
 }
 
 // A few contractions by value (blocks of item i: [grids[i].start, ...)).
 struct ZrunGroup {
   NbrGemm g[kZrunGroupMax];
   MultiGrid grids[kZrunGroupMax];
-  int n;
+  int rz[kZrunGroupMax];  // z-run of the item's tiles: 2, 4, 6 or 8
+  int n, ny;
 };
+// The shortest z-run that holds the grid's z extent (the sums do not depend on it).
+int narrow_rz(const NbrGemm& g) { return g.grid[2] <= 2 ? 2 : g.grid[2] <= 4 ? 4 : g.grid[2] <= 6 ? 6 : 8; }
 __global__ void __launch_bounds__(kZrThreads) zrun_narrow_group_kernel(const __grid_constant__ ZrunGroup G) {
-  const long long b = blockIdx.x >> 2;
-  const int it = multi_item_at(G.grids, G.n, b);
-  zrun_narrow_body<8>(G.g[it], multi_vblock_at(G.grids[it], b), blockIdx.x & 3);
+  VBlock vb;
+  const int it = multi_tile_major(G.grids, G.n, 0, gridDim.x >> 2, G.ny, blockIdx.x >> 2, &vb);
+  const int cg = blockIdx.x & 3;
+  __shared__ __align__(16) float sm[narrow_smem<8>()];
+  switch (G.rz[it]) {
+    case 2: zrun_narrow_body<2>(G.g[it], vb, cg, sm); break;
+    case 4: zrun_narrow_body<4>(G.g[it], vb, cg, sm); break;
+    case 6: zrun_narrow_body<6>(G.g[it], vb, cg, sm); break;
+    default: zrun_narrow_body<8>(G.g[it], vb, cg, sm); break;
+  }
 }
 
 template <typename T, int RZ>
 cudaError_t launch_rz_multi(const NbrGemm* gs, const MultiGrid* grids, int n, long long blocks, cudaStream_t s,
-                            long long first) {
+                            long long first, int ny) {
   constexpr size_t smem = zrun_smem_bytes<T, RZ>();
   static bool attr = false;
   if (!attr) {
@@ -381,7 +396,7 @@ cudaError_t launch_rz_multi(const NbrGemm* gs, const MultiGrid* grids, int n, lo
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   if constexpr (sizeof(T) == 4 && RZ % 2 == 0) {
     if (blocks < kZrunNarrowBlocks) {  // under two waves of four CTAs per SM
-      zrun_narrow_multi_kernel<RZ><<<(unsigned)(4 * blocks), kZrThreads, 0, s>>>(gs, grids, n, first);
+      zrun_narrow_multi_kernel<RZ><<<(unsigned)(4 * blocks), kZrThreads, 0, s>>>(gs, grids, n, first, ny);
       return cudaGetLastError();
     }
   }
@@ -450,10 +465,10 @@ void nbr_gemm_zrun_grid(const NbrGemm& g, int shape, unsigned out[3]) {
 
 template <typename T>
 cudaError_t launch_nbr_gemm_zrun_multi(int shape, const NbrGemm* gs, const MultiGrid* grids, int n, long long blocks,
-                                       cudaStream_t s, long long first) {
-  return shape == 0   ? launch_rz_multi<T, zrun_rz<T>(0)>(gs, grids, n, blocks, s, first)
-         : shape == 1 ? launch_rz_multi<T, zrun_rz<T>(1)>(gs, grids, n, blocks, s, first)
-                      : launch_rz_multi<T, zrun_rz<T>(2)>(gs, grids, n, blocks, s, first);
+                                       cudaStream_t s, long long first, int ny) {
+  return shape == 0   ? launch_rz_multi<T, zrun_rz<T>(0)>(gs, grids, n, blocks, s, first, ny)
+         : shape == 1 ? launch_rz_multi<T, zrun_rz<T>(1)>(gs, grids, n, blocks, s, first, ny)
+                      : launch_rz_multi<T, zrun_rz<T>(2)>(gs, grids, n, blocks, s, first, ny);
 }
 
 cudaError_t launch_nbr_gemm_zrun_group(const NbrGemm* gs, int n, cudaStream_t s) {
@@ -461,19 +476,23 @@ cudaError_t launch_nbr_gemm_zrun_group(const NbrGemm* gs, int n, cudaStream_t s)
   ZrunGroup G{};
   long long blocks = 0;
   for (int i = 0; i < n; ++i) {
-    unsigned gr[3];
-    nbr_gemm_zrun_grid<float>(gs[i], 0, gr);
-    const long long nb = (long long)gr[0] * gr[1] * gr[2];
-    if (gs[i].dsplit != 1) return cudaErrorInvalidValue;
+    if (gs[i].dsplit != 1 || gs[i].ntiles != gs[0].ntiles) return cudaErrorInvalidValue;
+    const int rz = narrow_rz(gs[i]);
+    const long long tiles = (long long)((gs[i].grid[0] + kZrBX - 1) / kZrBX) * ((gs[i].grid[1] + kZrBY - 1) / kZrBY) *
+                            ((gs[i].grid[2] + rz - 1) / rz);
+    const long long nb = tiles * gs[i].ntiles;
     if (nb <= 0) continue;
+    if (nb > 0x1fffffffLL) return cudaErrorInvalidConfiguration;
     G.g[G.n] = gs[i];
-    G.grids[G.n].gx = gr[0];
-    G.grids[G.n].gy = gr[1];
-    G.grids[G.n].gz = gr[2];
+    G.rz[G.n] = rz;
+    G.grids[G.n].gx = (unsigned)tiles;
+    G.grids[G.n].gy = (unsigned)gs[i].ntiles;
+    G.grids[G.n].gz = 1;
     G.grids[G.n++].start = blocks;
     blocks += nb;
   }
   if (G.n == 0) return cudaSuccess;
+  G.ny = gs[0].ntiles;
   if (blocks > 0x1fffffffLL) return cudaErrorInvalidConfiguration;
   zrun_narrow_group_kernel<<<(unsigned)(4 * blocks), kZrThreads, 0, s>>>(G);
   return cudaGetLastError();
@@ -482,9 +501,9 @@ cudaError_t launch_nbr_gemm_zrun_group(const NbrGemm* gs, int n, cudaStream_t s)
 template void nbr_gemm_zrun_grid<float>(const NbrGemm&, int, unsigned[3]);
 template void nbr_gemm_zrun_grid<double>(const NbrGemm&, int, unsigned[3]);
 template cudaError_t launch_nbr_gemm_zrun_multi<float>(int, const NbrGemm*, const MultiGrid*, int, long long,
-                                                       cudaStream_t, long long);
+                                                       cudaStream_t, long long, int);
 template cudaError_t launch_nbr_gemm_zrun_multi<double>(int, const NbrGemm*, const MultiGrid*, int, long long,
-                                                        cudaStream_t, long long);
+                                                        cudaStream_t, long long, int);
 template cudaError_t launch_nbr_gemm_zrun<float>(const NbrGemm&, int, cudaStream_t);
 template cudaError_t launch_nbr_gemm_zrun<double>(const NbrGemm&, int, cudaStream_t);
 

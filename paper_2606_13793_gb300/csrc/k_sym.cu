@@ -776,13 +776,14 @@ __global__ void __launch_bounds__(kSyTinyThreads)
 // Items of one launch: blocks [first, first + gridDim.x) of the step.
 template <typename T, int RZ>
 __global__ void __launch_bounds__(kSyThreads, sizeof(T) == 4 ? (RZ <= 4 ? 3 : 2) : 1)
-    sym_m2l_multi_kernel(const NbrGemm* __restrict__ gs, const MultiGrid* __restrict__ grids, int n, long long first) {
+    sym_m2l_multi_kernel(const NbrGemm* __restrict__ gs, const MultiGrid* __restrict__ grids, int n, long long first,
+                         int ny) {
   __shared__ NbrGemm g;
-  const long long b = (long long)blockIdx.x + first;
-  const int i = multi_item_at(grids, n, b);
+  VBlock vb;
+  const int i = multi_tile_major(grids, n, first, gridDim.x, ny, blockIdx.x, &vb);
   if (threadIdx.x == 0) g = gs[i];
   __syncthreads();
-  sym_m2l_body<T, RZ>(g, multi_vblock_at(grids[i], b));
+  sym_m2l_body<T, RZ>(g, vb);
 }
 template <typename T, int RZ>
 __global__ void __launch_bounds__(kSyThreads, 1)
@@ -858,7 +859,7 @@ cudaError_t launch_rows_form(const NbrGemm* gs, int n, cudaStream_t s) {
 
 template <typename T, int RZ>
 cudaError_t launch_multi_form(int kind, const NbrGemm* gs, const MultiGrid* grids, int n, long long blocks,
-                              long long first, cudaStream_t s) {
+                              long long first, int ny, cudaStream_t s) {
   if (kind == kSymNear4) {
     static bool done = false;
     if (cudaError_t e = opt_in(sym_near4_multi_kernel<T, RZ>, sym_near4_smem<T, RZ>(), &done)) return e;
@@ -866,7 +867,7 @@ cudaError_t launch_multi_form(int kind, const NbrGemm* gs, const MultiGrid* grid
   } else {
     static bool done = false;
     if (cudaError_t e = opt_in(sym_m2l_multi_kernel<T, RZ>, sym_m2l_smem<T, RZ>(), &done)) return e;
-    sym_m2l_multi_kernel<T, RZ><<<(unsigned)blocks, kSyThreads, sym_m2l_smem<T, RZ>(), s>>>(gs, grids, n, first);
+    sym_m2l_multi_kernel<T, RZ><<<(unsigned)blocks, kSyThreads, sym_m2l_smem<T, RZ>(), s>>>(gs, grids, n, first, ny);
   }
   return cudaGetLastError();
 }
@@ -904,7 +905,7 @@ cudaError_t launch_nbr_gemm_sym(const NbrGemm& g, cudaStream_t s) {
 
 template <typename T>
 cudaError_t launch_nbr_gemm_sym_multi(int shape, int kind, const NbrGemm* gs, const MultiGrid* grids, int n,
-                                      long long blocks, long long first, cudaStream_t s) {
+                                      long long blocks, long long first, int ny, cudaStream_t s) {
   constexpr bool f = sizeof(T) == 4;
   if (n <= 0 || blocks <= 0) return cudaSuccess;
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
@@ -915,16 +916,16 @@ cudaError_t launch_nbr_gemm_sym_multi(int shape, int kind, const NbrGemm* gs, co
     sym_tiny_multi_kernel<T><<<(unsigned)blocks, kSyTinyThreads, sym_tiny_smem<T>(), s>>>(gs, grids, n, first);
     return cudaGetLastError();
   }
-  return shape == 0   ? launch_multi_form<T, f ? 8 : 4>(kind, gs, grids, n, blocks, first, s)
-         : shape == 1 ? launch_multi_form<T, f ? 4 : 2>(kind, gs, grids, n, blocks, first, s)
-                      : launch_multi_form<T, f ? 6 : 3>(kind, gs, grids, n, blocks, first, s);
+  return shape == 0   ? launch_multi_form<T, f ? 8 : 4>(kind, gs, grids, n, blocks, first, ny, s)
+         : shape == 1 ? launch_multi_form<T, f ? 4 : 2>(kind, gs, grids, n, blocks, first, ny, s)
+                      : launch_multi_form<T, f ? 6 : 3>(kind, gs, grids, n, blocks, first, ny, s);
 }
 
 template cudaError_t launch_nbr_gemm_sym<float>(const NbrGemm&, cudaStream_t);
 template cudaError_t launch_nbr_gemm_sym<double>(const NbrGemm&, cudaStream_t);
 template cudaError_t launch_nbr_gemm_sym_multi<float>(int, int, const NbrGemm*, const MultiGrid*, int, long long,
-                                                      long long, cudaStream_t);
+                                                      long long, int, cudaStream_t);
 template cudaError_t launch_nbr_gemm_sym_multi<double>(int, int, const NbrGemm*, const MultiGrid*, int, long long,
-                                                       long long, cudaStream_t);
+                                                       long long, int, cudaStream_t);
 
 }  // namespace fmmgb

@@ -45,6 +45,27 @@ __host__ __device__ __forceinline__ VBlock multi_vblock_at(const MultiGrid& g, l
   return v;
 }
 
+// Tile-major order of a launch whose items all have gy = ny column tiles (gz =
+// 1): block p runs column tile p / (blocks / ny) of every item before the next
+// tile.  M2L column tiles shrink from the first to the last by up to (p + 1)^2
+// in length, so the long ones of all items start first.  ny = 0: the item
+// order.  Returns the item and its block.
+__host__ __device__ __forceinline__ int multi_tile_major(const MultiGrid* __restrict__ g, int n, long long first,
+                                                         long long blocks, int ny, long long p, VBlock* vb) {
+  if (ny <= 1) {
+    const int i = multi_item_at(g, n, first + p);
+    *vb = multi_vblock_at(g[i], first + p);
+    return i;
+  }
+  const long long per = blocks / ny, r = p % per;
+  const int i = multi_item_at(g, n, first + r * ny);
+  vb->gx = g[i].gx, vb->gy = g[i].gy, vb->gz = g[i].gz;
+  vb->x = (unsigned)(r - (g[i].start - first) / ny);
+  vb->y = (unsigned)(p / per);
+  vb->z = 0;
+  return i;
+}
+
 __device__ __forceinline__ int multi_item(const MultiGrid* __restrict__ g, int n) {
   return multi_item_at(g, n, (long long)blockIdx.x);
 }
