@@ -174,6 +174,10 @@ struct fmm_plan_s {
   void* d_sym_wq[2] = {nullptr, nullptr};
   void* d_sym_near = nullptr;
   int sym_q_len[2] = {0, 0};
+  SymTab* d_sym_near2_tab = nullptr;  // leaf-2 near field (weights in d_sym_near)
+  SymTab* d_sym_m2p_tab = nullptr;    // final-stage M2P off the tensor cores, leaf 2 and 4
+  void* d_sym_m2p = nullptr;
+  size_t m2p_fold_off = 0;  // its folded leaf multipoles, component-major
   // near field
   void* d_w_near = nullptr;
   int* d_near_tile_k = nullptr;
@@ -501,6 +505,8 @@ struct SymHost {
   SymTab tab{};
   std::vector<double> Ws, Wq;
 };
+void sym_fold6(std::vector<double>& w, int par);
+double sym_at6(const std::vector<double>& w, int k, int sg);
 void sym_m2l_weights(const MultiIndex& mi, const TaylorTable& tt, SymHost& H, bool fill) {
   const std::vector<int> red = harmonic_components(mi);
   SymTab& T = H.tab;
@@ -537,7 +543,7 @@ void sym_m2l_weights(const MultiIndex& mi, const TaylorTable& tt, SymHost& H, bo
   H.Ws.assign((size_t)off, 0.0);
   H.Wq.assign((size_t)27 * ql, 0.0);
   if (!fill) return;
-  std::vector<double> w(216), x(216);
+  std::vector<double> w(216);
   for (int a = 0; a < nk; ++a)
     for (int b = 0; b < nk; ++b) {
       if (a >= T.kb[b]) continue;
@@ -550,20 +556,7 @@ void sym_m2l_weights(const MultiIndex& mi, const TaylorTable& tt, SymHost& H, bo
         const int cheb = std::max(std::abs(u[0]), std::max(std::abs(u[1]), std::abs(u[2])));
         w[i] = cheb < 2 ? 0.0 : mult * (-tt.at(u)[g]);
       }
-      // per axis: position j + 2 in 0 .. 5 -> 2 k + (0: sum, 1: difference)
-      const int str[3] = {1, 6, 36};
-      for (int q = 0; q < 3; ++q) {
-        const double f = (T.par[a] >> q) & 1 ? -1.0 : 1.0;
-        for (int i = 0; i < 216; ++i) {
-          if ((i / str[q]) % 6) continue;
-          for (int k = 0; k < 3; ++k) {
-            const double up = w[i + (3 + k) * str[q]], lo = w[i + (2 - k) * str[q]];
-            x[i + 2 * k * str[q]] = up + f * lo;
-            x[i + (2 * k + 1) * str[q]] = up - f * lo;
-          }
-        }
-        w.swap(x);
-      }
+      sym_fold6(w, T.par[a]);
       const int un = b / 8, n = b % 8;
       const int nl = a < T.n8[un] ? 8 : a < T.n4[un] ? 4 : 1;
       const long long wo = T.w_off[un] + 216LL * (a < T.n8[un] ? 8 * a
@@ -571,9 +564,8 @@ void sym_m2l_weights(const MultiIndex& mi, const TaylorTable& tt, SymHost& H, bo
                                                                  : 8 * T.n8[un] + 4 * (T.n4[un] - T.n8[un]) + a - T.n4[un]);
       for (int k = 0; k < 27; ++k)
         for (int sg = 0; sg < 8; ++sg) {
-          const int kx = k % 3, ky = (k / 3) % 3, kz = k / 9;
-          const double v = w[(2 * kx + (sg & 1)) + 6 * (2 * ky + ((sg >> 1) & 1)) + 36 * (2 * kz + (sg >> 2))];
-          H.Ws[(size_t)(wo + ((((ky * 3 + kx) * 4 + (sg & 3)) * 3 + kz) * nl + n) * 2 + (sg >> 2))] = v;
+          const double v = sym_at6(w, k, sg);
+          H.Ws[(size_t)(wo + ((((k % 9) * 4 + (sg & 3)) * 3 + k / 9) * nl + n) * 2 + (sg >> 2))] = v;
           H.Wq[(size_t)k * ql + T.q_off[a] + b * 8 + sg] = v;
         }
     }
@@ -1589,6 +1581,86 @@ void near_weights(int b, int comps, std::vector<T>& W, std::vector<int>& tile_k,
 
 // M2M: Mt_alpha(P) += C(alpha,beta) 2^-|alpha| (+-1/2)^(alpha-beta) Mt_beta(C);
 // L2L: Lt_beta(C) += C(gamma,beta) 2^(-1-|gamma|) (+-1/2)^(gamma-beta) Lt_gamma(P).
+// The reflection basis of 6^3 weights to an upper target from the source
+// positions -2 .. 3 per axis (x fastest): per axis position pairs (1 + k, -k)
+// -> 2 k + (0: sum, 1: difference), with the source component's parity.
+void sym_fold6(std::vector<double>& w, int par) {
+  std::vector<double> x(216);
+  const int str[3] = {1, 6, 36};
+  for (int q = 0; q < 3; ++q) {
+    const double f = (par >> q) & 1 ? -1.0 : 1.0;
+    for (int i = 0; i < 216; ++i) {
+      if ((i / str[q]) % 6) continue;
+      for (int k = 0; k < 3; ++k) {
+        const double up = w[i + (3 + k) * str[q]], lo = w[i + (2 - k) * str[q]];
+        x[i + 2 * k * str[q]] = up + f * lo;
+        x[i + (2 * k + 1) * str[q]] = up - f * lo;
+      }
+    }
+    w.swap(x);
+  }
+}
+double sym_at6(const std::vector<double>& w, int k, int sg) {  // triple k, signs sg
+  const int kx = k % 3, ky = (k / 3) % 3, kz = k / 9;
+  return w[(2 * kx + (sg & 1)) + 6 * (2 * ky + ((sg >> 1) & 1)) + 36 * (2 * kz + (sg >> 2))];
+}
+
+// The leaf-2 near field as one component over the box's 8 cells.
+void sym_near2_weights(SymHost& H) {
+  H.tab = SymTab{};
+  H.tab.nk = H.tab.nunits = 1;
+  H.tab.n1[0] = 1;
+  H.tab.kb[0] = 1;
+  H.Ws.assign(216, 0.0);
+  std::vector<double> w(216);
+  for (int i = 0; i < 216; ++i) {
+    const double u0 = 1 - (i % 6 - 2), u1 = 1 - ((i / 6) % 6 - 2), u2 = 1 - (i / 36 - 2);
+    const double r = std::sqrt(u0 * u0 + u1 * u1 + u2 * u2);
+    w[i] = -0.125 / (r > 0.0 ? r : 1.0);
+  }
+  sym_fold6(w, 0);
+  for (int k = 0; k < 27; ++k)
+    for (int sg = 0; sg < 8; ++sg) H.Ws[(size_t)((((k % 9) * 4 + (sg & 3)) * 3 + k / 9) * 2 + (sg >> 2))] = sym_at6(w, k, sg);
+}
+
+// The final-stage M2P on the harmonic components to the multipole limit:
+// columns are the b^3 cells of the upper child (1, 1, 1).
+void sym_m2p_weights(const MultiIndex& mi, const M2pTable& tab, int b, SymHost& H) {
+  const std::vector<int> red = harmonic_components(mi);
+  SymTab& T = H.tab;
+  T = SymTab{};
+  const int b3 = b * b * b, K = (mi.mo + 1) * (mi.mo + 1);
+  T.nk = K;
+  T.nunits = b3 / 8;
+  for (int a = 0; a < K; ++a)
+    T.par[a] = (unsigned char)((mi.a[red[a]] & 1) | (mi.b[red[a]] & 1) << 1 | (mi.c[red[a]] & 1) << 2);
+  H.Ws.assign((size_t)T.nunits * K * 216 * 8, 0.0);
+  for (int u = 0; u < T.nunits; ++u) {
+    T.n8[u] = T.n4[u] = T.n1[u] = K;
+    T.w_off[u] = (long long)u * K * 216 * 8;
+  }
+  std::vector<double> w(216);
+  for (int a = 0; a < K; ++a)
+    for (int cell = 0; cell < b3; ++cell) {
+      for (int i = 0; i < 216; ++i) {
+        const int j[3] = {i % 6 - 2, (i / 6) % 6 - 2, i / 36 - 2};
+        int d = 0, cs = 0, str = 1;
+        for (int q = 0; q < 3; ++q) {
+          const int dq = j[q] < 0 ? -1 : j[q] > 1 ? 1 : 0;
+          d += (dq + 1) * str;
+          cs |= (j[q] - 2 * dq) << q;
+          str *= 3;
+        }
+        w[i] = 0.125 * m2p_entry(mi, tab, d, red[a] * 8 + cs, 7 * b3 + cell);
+      }
+      sym_fold6(w, T.par[a]);
+      for (int k = 0; k < 27; ++k)
+        for (int sg = 0; sg < 8; ++sg)
+          H.Ws[(size_t)(T.w_off[cell / 8] + (long long)a * 216 * 8 +
+                        ((((k % 9) * 4 + (sg & 3)) * 3 + k / 9) * 8 + cell % 8) * 2 + (sg >> 2))] = sym_at6(w, k, sg);
+    }
+}
+
 // Reflection-basis weights of the leaf-4 near field (k_sym.cu): source
 // position j in -4 .. 7 and upper targets 2, 3 per axis; mirror pairs
 // (2 + k, 1 - k).  [36 (x, y) pairs][4 signs][6 z pairs][8 targets][2].
@@ -1672,6 +1744,7 @@ namespace {
 // for plans, the static array for the allocation-free solve).  On failure
 // the caller releases P.
 bool sym_level(fmm_plan_t P, int l);
+bool near2_sym(fmm_plan_t P);
 NbrGemm m2l_gemm(fmm_plan_t P, int l, int form = -1);
 NbrGemm near_gemm(fmm_plan_t P);
 
@@ -1826,6 +1899,13 @@ fmm_status plan_init(fmm_plan_t P, const int d3[3], double dx, double G, int ord
     P->m2p_off = off;
     off = align(off + (size_t)P->lev[P->L].npar * 8 * (size_t)(P->b * P->b * P->b) * P->m2p_comps * P->esize());
   }
+  // the CUDA-core M2P in the reflection basis: folded leaf multipoles (P2M
+  // stages them, so only where that fits shared memory)
+  const bool m2p_sym = P->m2p && !P->lev[P->L].tc && o.accel != 2 && (leaf == 2 || leaf == 4) && P->harm_cc;
+  if (m2p_sym) {
+    P->m2p_fold_off = off;
+    off = align(off + (size_t)P->lev[P->L].npar * 8 * P->nr * (P->lev[P->L].f64 ? 8 : 4));
+  }
   P->work_off = off;
   off = align(off + cells_bytes);
   if (P->near_comps == 4) {
@@ -1872,7 +1952,12 @@ fmm_status plan_init(fmm_plan_t P, const int d3[3], double dx, double G, int ord
       c->shape = 3;
       return;
     }
-    if (g.sym == kSymNear4 || (g.sym == kSymM2l || P->harm_cc) && g.skip_center) {
+    if (P->d_sym_near2_tab && !g.skip_center) {  // leaf-2 near field: short z-runs, plenty of tiles
+      c->shape = 2;
+      c->dsplit = 1;
+      return;
+    }
+    if (g.sym == kSymNear4 || (P->harm_cc && g.skip_center)) {
       sym_default(P, g, c, f64);
       return;
     }
@@ -2089,9 +2174,17 @@ fmm_status plan_init(fmm_plan_t P, const int d3[3], double dx, double G, int ord
     }
     // (the static array: where it leaves room, the two small tables below included)
     const bool room = !P->static_base || P->static_used + 36 * 384 * P->esize() + 4096 <= P->static_cap;
-    if (P->b == 4 && P->near_comps == 1 && !P->near_tc && room) {
+    if ((P->b == 4 || (P->b == 2 && !P->static_base)) && P->near_comps == 1 && !P->near_tc && room) {
       std::vector<double> W;
-      sym_near4_weights(W);
+      if (P->b == 4) {
+        sym_near4_weights(W);
+      } else {
+        SymHost H;
+        sym_near2_weights(H);
+        W = H.Ws;
+        std::vector<SymTab> tab(1, H.tab);
+        if ((st = P->upload(tab, &P->d_sym_near2_tab, s))) return cleanup(st);
+      }
       if (P->f64_data()) {
         double* d = nullptr;
         if ((st = P->upload(W, &d, s))) return cleanup(st);
@@ -2186,7 +2279,22 @@ fmm_status plan_init(fmm_plan_t P, const int d3[3], double dx, double G, int ord
         P->m2p_tc = P->span_m2p = true;
       }
     }
-    if (!P->m2p_tc) {
+    if (P->m2p_fold_off) {
+      SymHost H;
+      sym_m2p_weights(P->mi, tab, P->b, H);
+      std::vector<SymTab> st1(1, H.tab);
+      if ((st = P->upload(st1, &P->d_sym_m2p_tab, s))) return cleanup(st);
+      if (lf.f64) {
+        double* d = nullptr;
+        if ((st = P->upload(H.Ws, &d, s))) return cleanup(st);
+        P->d_sym_m2p = d;
+      } else {
+        const std::vector<float> wf(H.Ws.begin(), H.Ws.end());
+        float* d = nullptr;
+        if ((st = P->upload(wf, &d, s))) return cleanup(st);
+        P->d_sym_m2p = d;
+      }
+    } else if (!P->m2p_tc) {
       const int ncol = 8 * mc * P->b * P->b * P->b;
       auto entry = [&](int d, int k, int n) { return m2p_entry(P->mi, tab, d, k, n, mc); };
       std::vector<int> tk;
@@ -2546,6 +2654,12 @@ NbrGemm m2l_gemm(fmm_plan_t P, int l, int form) {
   return g;
 }
 
+// Whether the leaf-2 near field runs in the reflection basis (its density is
+// then cell-major): the z-run shapes of plans off the tensor cores.
+bool near2_sym(fmm_plan_t P) {
+  return P->d_sym_near2_tab && (P->near_choice.shape == 1 || P->near_choice.shape == 2);
+}
+
 NbrGemm near_gemm(fmm_plan_t P) {
   NbrGemm g;
   g.A = P->arena + P->rho_box_off;
@@ -2560,7 +2674,12 @@ NbrGemm near_gemm(fmm_plan_t P) {
   g.accumulate = 0;
   g.shape = P->near_choice.shape;
   g.dsplit = P->near_choice.dsplit;
-  if (P->d_sym_near) {
+  if (near2_sym(P)) {
+    g.sym = kSymM2l;
+    g.st = P->d_sym_near2_tab;
+    g.Ws = P->d_sym_near;
+    g.lda = P->lev[P->L].nbox;
+  } else if (P->d_sym_near && P->b == 4) {
     g.sym = kSymNear4;
     g.Ws = P->d_sym_near;
   }
@@ -2605,6 +2724,32 @@ fmm_status do_m2p(fmm_plan_t P, cudaStream_t s) {
     return FMM_OK;
   }
   NbrGemm g;
+  if (P->m2p_fold_off) {  // reflection basis
+    g.A = P->arena + P->m2p_fold_off;
+    g.row_len = 8 * P->nr;
+    for (int q = 0; q < 3; ++q) g.grid[q] = lf.np[q];
+    g.W = nullptr;
+    g.tile_k = nullptr;
+    g.tile_w = nullptr;
+    g.C = P->arena + P->m2p_off;
+    g.n_cols = 8 * P->b * P->b * P->b;
+    g.ntiles = 0;
+    g.accumulate = 0;
+    g.dsplit = 1;
+    g.partial = nullptr;
+    g.skip_center = 1;
+    g.sym = kSymM2p;
+    g.b = P->b;
+    g.st = P->d_sym_m2p_tab;
+    g.Ws = P->d_sym_m2p;
+    g.lda = lf.npar;
+    // the long z-run where it gives every SM two blocks (32^3 parents, one unit: 62 us in 128 blocks)
+    const int rz = lf.f64 ? 4 : 8;
+    g.shape = (long long)((lf.np[0] + 7) / 8) * ((lf.np[1] + 3) / 4) * ((lf.np[2] + rz - 1) / rz) *
+                          ((g.n_cols / 8 + 7) / 8) >= 304 ? 1 : 2;
+    CUDA_TRY(lf.f64 ? launch_nbr_gemm<double>(g, s) : launch_nbr_gemm<float>(g, s));
+    return FMM_OK;
+  }
   g.A = P->M(P->L);
   g.row_len = 8 * P->nc;
   for (int q = 0; q < 3; ++q) g.grid[q] = lf.np[q];
@@ -2758,11 +2903,12 @@ fmm_status run_solve(fmm_plan_t P, const T* rho, T* phi, T* accel, cudaStream_t 
                            mplanes ? P->arena + lf.hi_off : nullptr, mplanes ? P->arena + lf.lo_off : nullptr,
                            (P->near_tc && near_rows) ? P->arena + P->rho_hi_off : nullptr,
                            (P->near_tc && near_rows) ? P->arena + P->rho_lo_off : nullptr, P->d_flag,
-                           sym_level(P, L) ? 2 : ((mplanes && P->harm) || lf.fold_off) ? 1 : 0,
-                           refl          ? reinterpret_cast<T*>(P->arena + lf.rfold_off)
-                           : lf.fold_off ? reinterpret_cast<T*>(P->arena + lf.fold_off)
-                                         : nullptr,
-                           s, adj_dip));
+                           sym_level(P, L) || P->m2p_fold_off ? 2 : ((mplanes && P->harm) || lf.fold_off) ? 1 : 0,
+                           refl              ? reinterpret_cast<T*>(P->arena + lf.rfold_off)
+                           : lf.fold_off     ? reinterpret_cast<T*>(P->arena + lf.fold_off)
+                           : P->m2p_fold_off ? reinterpret_cast<T*>(P->arena + P->m2p_fold_off)
+                                             : nullptr,
+                           s, adj_dip, near2_sym(P) ? 1 : 0));
   }
   const bool p2l = adjoint && P->m2p;  // leaf level by the transpose of M2P
   if (p2l && P->m2p_comps == 4)  // [w, v] per box, the force columns zero without g
@@ -3519,7 +3665,9 @@ void build_fused(fmm_batch_t B, const void* const* rho, void* const* phi, void* 
     };
     for (fmm_plan_t P : B->plans) {
       for (int l = 2; l <= P->L; ++l) add(m2l_gemm(P, l, reflect(P, l) ? 1 : 0), P->h_m2l_tile_k);
-      add(near_gemm(P), P->h_near_tile_k);
+      NbrGemm ng = near_gemm(P);
+      if (ng.sym == kSymM2l) ng.sym = kSymNone;  // leaf 2: the batch's P2M writes box rows
+      add(ng, P->h_near_tile_k);
     }
     for (int sh : {1, 5, 0, 2, 3, 4}) {  // the tiny-grid launch last
       std::vector<NbrGemm> all;

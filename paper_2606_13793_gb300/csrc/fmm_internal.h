@@ -86,7 +86,10 @@ struct SymTab {
   int q_len;                      // values of one triple
   unsigned char par[kSymMaxK];    // bit q: odd along axis q
 };
-enum SymKind { kSymNone = 0, kSymM2l = 1, kSymNear4 = 2 };
+// kSymM2l: also the near field of leaf-2 boxes (one component, cells as
+// children).  kSymM2p: the final-stage M2P; its columns are the cells of the
+// parent's upper children, unit u holds cells 8 u .. 8 u + 7 (x fastest).
+enum SymKind { kSymNone = 0, kSymM2l = 1, kSymNear4 = 2, kSymM2p = 3 };
 
 // Neighbour-contraction ("implicit GEMM") description for the SIMT kernel:
 //   C[row][n] (+)= sum_{d in 27 neighbours} sum_{k < K(tile(n))} A[row + d][k] * W_d[k][n]
@@ -113,6 +116,7 @@ struct NbrGemm {
   // reflection-basis form (k_sym.cu), SymKind.  kSymM2l: A is component-major,
   // [8 alpha + child][lda rows]; kSymNear4: A as above
   int sym = 0;
+  int b = 0;  // kSymM2p: cells per leaf-box side
   const SymTab* st = nullptr;  // device
   const void* Ws = nullptr;
   const void* Wq = nullptr;
@@ -210,12 +214,13 @@ struct TreeTables {
 // Mfold (nullable, with harm): the folded components in the level's type,
 // rows of 8 (p+1)^2 values (TF32 levels) or, with harm = 2, component-major
 // [8 r + child][parent] (the CUDA-core harmonic M2L, k_sym.cu).
+// rho_soa = 1: rho_box is cell-major, [b^3][boxes] (leaf 2, reflection basis).
 // dip (nullable): dipole sources [3][cells], weights v_q adding v_q d/de_q (e^alpha)
 // (box units) per cell -- the transpose of the analytic force's L2P gradient.
 template <typename T>
 cudaError_t launch_p2m(const TreeTables& t, const T* rho, const int dims[3], const Level& leaf, T* Mleaf, T* rho_box,
                        void* Mhi, void* Mlo, void* rho_hi, void* rho_lo, int* flag, int harm, T* Mfold,
-                       cudaStream_t s, const T* dip = nullptr);
+                       cudaStream_t s, const T* dip = nullptr, int rho_soa = 0);
 // M2M into the parent level; Mhi/Mlo (bf16 planes of the parent, harmonic
 // components when harm = 1) when non-NULL.
 template <typename Tc, typename Tp>

@@ -404,7 +404,8 @@ cudaError_t launch_nbr_gemm_col(const NbrGemm& g, cudaStream_t s) {
 
 template <typename T>
 cudaError_t launch_nbr_gemm(const NbrGemm& g, cudaStream_t s) {
-  if (g.sym == kSymM2l || (g.sym == kSymNear4 && (g.shape == 1 || g.shape == 2))) return launch_nbr_gemm_sym<T>(g, s);
+  if (g.sym == kSymM2l || g.sym == kSymM2p || (g.sym == kSymNear4 && (g.shape == 1 || g.shape == 2)))
+    return launch_nbr_gemm_sym<T>(g, s);
   if (g.shape == 3) return launch_nbr_gemm_col<T>(g, s);
   return g.shape == 0 ? launch_nbr_gemm_simt<T>(g, s) : launch_nbr_gemm_zrun<T>(g, g.shape - 1, s);
 }

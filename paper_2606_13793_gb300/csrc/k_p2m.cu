@@ -52,7 +52,7 @@ __device__ __forceinline__ void p2m_body(const Box& B, const T* __restrict__ rho
                                          const Level& leaf, T* __restrict__ Ms, T* __restrict__ Mr, int rp,
                                          T* __restrict__ rho_box, __nv_bfloat16* __restrict__ rhi,
                                          __nv_bfloat16* __restrict__ rlo, int* __restrict__ flag,
-                                         const T* __restrict__ dip, long long ncell) {
+                                         const T* __restrict__ dip, long long ncell, int rho_soa) {
   constexpr int NC = ncoef_c(P);
   constexpr int NH = ncoef_parity<P>(h);
   T acc[NH > 0 ? NH : 1];  // this thread's coefficients, in canonical order restricted to parity h of c
@@ -185,7 +185,7 @@ __device__ __forceinline__ void p2m_body(const Box& B, const T* __restrict__ rho
             if (DIP)
               for (int q = 0; q < 3; ++q) vrow[q * b * b + j * b + i] = dip[q * ncell + c0 + i];
             if (h == 0) {
-              if (rho_box) rho_box[e0 + i] = m;
+              if (rho_box) rho_box[rho_soa ? (e0 + i - box * b3) * (ncell / b3) + box : e0 + i] = m;
               if (rhi) store_split(rhi, rlo, (size_t)(e0 + i), m);
             }
           }
@@ -245,7 +245,7 @@ __device__ __forceinline__ void p2m_block(const T* __restrict__ rho, int nx, int
                                           __nv_bfloat16* __restrict__ Mlo, T* __restrict__ rho_box,
                                           __nv_bfloat16* __restrict__ rhi, __nv_bfloat16* __restrict__ rlo,
                                           int* __restrict__ flag, int harm, T* __restrict__ Mfold,
-                                          const T* __restrict__ dip, long long ncell, const VBlock& vb) {
+                                          const T* __restrict__ dip, long long ncell, const VBlock& vb, int rho_soa) {
   constexpr int NC = ncoef_c(P);
   constexpr int ROW = 8 * NC;     // values per parent row
   constexpr int ROWP = ROW + 8;   // staged row pitch
@@ -259,9 +259,9 @@ __device__ __forceinline__ void p2m_block(const T* __restrict__ rho, int nx, int
   const Box B = box_of(leaf, (w >> 1) * 32 + (t & 31));
   if (B.par < leaf.npar) {
     if (w & 1)
-      p2m_body<P, T, 1, DIP>(B, rho, nx, ny, b, leaf, Ms, Mr, rp, rho_box, rhi, rlo, flag, dip, ncell);
+      p2m_body<P, T, 1, DIP>(B, rho, nx, ny, b, leaf, Ms, Mr, rp, rho_box, rhi, rlo, flag, dip, ncell, rho_soa);
     else
-      p2m_body<P, T, 0, DIP>(B, rho, nx, ny, b, leaf, Ms, Mr, rp, rho_box, rhi, rlo, flag, dip, ncell);
+      p2m_body<P, T, 0, DIP>(B, rho, nx, ny, b, leaf, Ms, Mr, rp, rho_box, rhi, rlo, flag, dip, ncell, rho_soa);
   }
   __syncthreads();
   const long long p0 = (long long)vb.x * kP2mParents<T>;
@@ -314,9 +314,9 @@ __global__ void __launch_bounds__(kP2mThreads<T>) p2m_kernel(const T* __restrict
                                                        __nv_bfloat16* __restrict__ rhi,
                                                        __nv_bfloat16* __restrict__ rlo, int* __restrict__ flag,
                                                        int harm, T* __restrict__ Mfold, const T* __restrict__ dip,
-                                                       long long ncell) {
+                                                       long long ncell, int rho_soa) {
   p2m_block<P, T, DIP>(rho, nx, ny, b, leaf, Mleaf, Mhi, Mlo, rho_box, rhi, rlo, flag, harm, Mfold, dip, ncell,
-                       native_vblock());
+                       native_vblock(), rho_soa);
 }
 
 // The leaf levels of many solves in one launch (batched solves).
@@ -331,7 +331,7 @@ __global__ void __launch_bounds__(kP2mThreads<T>) p2m_multi_kernel(const P2mArgs
                          static_cast<__nv_bfloat16*>(x.Mhi), static_cast<__nv_bfloat16*>(x.Mlo),
                          static_cast<T*>(x.rho_box), static_cast<__nv_bfloat16*>(x.rho_hi),
                          static_cast<__nv_bfloat16*>(x.rho_lo), x.flag, x.harm, static_cast<T*>(x.Mfold), nullptr,
-                         x.ncell, multi_vblock(g[i]));
+                         x.ncell, multi_vblock(g[i]), 0);
 }
 
 template <int P, typename T>
@@ -357,7 +357,7 @@ template <int P, typename T, bool DIP>
 cudaError_t p2m_launch_dip(unsigned blocks, size_t smem, size_t attr_bytes, cudaStream_t s, const T* rho, int nx,
                            int ny, int b, Level leaf, T* Mleaf, __nv_bfloat16* Mhi, __nv_bfloat16* Mlo, T* rho_box,
                            __nv_bfloat16* rhi, __nv_bfloat16* rlo, int* flag, int harm, T* Mfold, const T* dip,
-                           long long ncell) {
+                           long long ncell, int rho_soa) {
   static bool attr = false;
   if (!attr && attr_bytes > 48 * 1024) {
     const cudaError_t e =
@@ -366,14 +366,14 @@ cudaError_t p2m_launch_dip(unsigned blocks, size_t smem, size_t attr_bytes, cuda
     attr = true;
   }
   p2m_kernel<P, T, DIP><<<blocks, kP2mThreads<T>, smem, s>>>(rho, nx, ny, b, leaf, Mleaf, Mhi, Mlo, rho_box, rhi, rlo, flag,
-                                                       harm, Mfold, dip, ncell);
+                                                       harm, Mfold, dip, ncell, rho_soa);
   return cudaGetLastError();
 }
 
 template <int P, typename T>
 cudaError_t p2m_launch(unsigned blocks, cudaStream_t s, const T* rho, int nx, int ny, int b, Level leaf, T* Mleaf,
                 __nv_bfloat16* Mhi, __nv_bfloat16* Mlo, T* rho_box, __nv_bfloat16* rhi, __nv_bfloat16* rlo, int* flag,
-                int harm, T* Mfold, const T* dip, long long ncell) {
+                int harm, T* Mfold, const T* dip, long long ncell, int rho_soa) {
   constexpr size_t full = (size_t)kP2mParents<T> * (8 * ncoef_c(P) + 8) * sizeof(T);
   // staged harmonic rows, where they fit beside the full ones (the plan folds
   // nothing at FP64 order 8, which would not)
@@ -383,9 +383,9 @@ cudaError_t p2m_launch(unsigned blocks, cudaStream_t s, const T* rho, int nx, in
   const size_t smem = full + ((harm && (Mhi || Mfold)) ? red : 0);
   if (dip)
     return p2m_launch_dip<P, T, true>(blocks, smem, full + red, s, rho, nx, ny, b, leaf, Mleaf, Mhi, Mlo, rho_box, rhi,
-                                      rlo, flag, harm, Mfold, dip, ncell);
+                                      rlo, flag, harm, Mfold, dip, ncell, rho_soa);
   return p2m_launch_dip<P, T, false>(blocks, smem, full + red, s, rho, nx, ny, b, leaf, Mleaf, Mhi, Mlo, rho_box, rhi,
-                                     rlo, flag, harm, Mfold, nullptr, ncell);
+                                     rlo, flag, harm, Mfold, nullptr, ncell, rho_soa);
 }
 
 }  // namespace
@@ -393,7 +393,7 @@ cudaError_t p2m_launch(unsigned blocks, cudaStream_t s, const T* rho, int nx, in
 template <typename T>
 cudaError_t launch_p2m(const TreeTables& t, const T* rho, const int dims[3], const Level& leaf, T* Mleaf, T* rho_box,
                        void* Mhi, void* Mlo, void* rho_hi, void* rho_lo, int* flag, int harm, T* Mfold,
-                       cudaStream_t s, const T* dip) {
+                       cudaStream_t s, const T* dip, int rho_soa) {
   const long long threads = leaf.npar * 16;  // two threads per box
   if (threads == 0) return cudaSuccess;
   cudaError_t e = cudaSuccess;
@@ -401,7 +401,7 @@ cudaError_t launch_p2m(const TreeTables& t, const T* rho, const int dims[3], con
                             rho, dims[0], dims[1], t.b, leaf, Mleaf, static_cast<__nv_bfloat16*>(Mhi),
                             static_cast<__nv_bfloat16*>(Mlo), rho_box, static_cast<__nv_bfloat16*>(rho_hi),
                             static_cast<__nv_bfloat16*>(rho_lo), flag, harm, Mfold, dip,
-                            (long long)dims[0] * dims[1] * dims[2])));
+                            (long long)dims[0] * dims[1] * dims[2], rho_soa)));
   return e;
 }
 
@@ -419,8 +419,8 @@ template cudaError_t launch_p2m_multi<double>(int, const P2mArgs*, const MultiGr
                                               cudaStream_t);
 
 template cudaError_t launch_p2m<float>(const TreeTables&, const float*, const int*, const Level&, float*, float*,
-                                       void*, void*, void*, void*, int*, int, float*, cudaStream_t, const float*);
+                                       void*, void*, void*, void*, int*, int, float*, cudaStream_t, const float*, int);
 template cudaError_t launch_p2m<double>(const TreeTables&, const double*, const int*, const Level&, double*, double*,
-                                        void*, void*, void*, void*, int*, int, double*, cudaStream_t, const double*);
+                                        void*, void*, void*, void*, int*, int, double*, cudaStream_t, const double*, int);
 
 }  // namespace fmmgb

@@ -1,7 +1,7 @@
 // Neighbour contractions on the CUDA cores in the reflection basis.
 //
-// The M2L of a level (Sec. 2.3, eq. M2L) and the near field of leaf-4 boxes
-// (eq. direct) are the contraction of k_gemm_simt.cu,
+// The M2L of a level (Sec. 2.3, eq. M2L), the final-stage M2P (Sec. 4) and the
+// near field of leaf-2 and leaf-4 boxes (eq. direct) are the contraction of k_gemm_simt.cu,
 //   C[P][n] = sum_{d in 27 neighbours} sum_k A[P + d][k] W_d[k][n],
 // and their weights are those of an even kernel: reflecting an axis about the
 // target row's centre maps source position j (a child box, or a cell) to
@@ -13,7 +13,8 @@
 // per axis, the operator falls into 8 blocks (one per choice of the three
 // signs) of 1/8 of the rows and 1/8 of the columns: 8 times fewer products,
 // exactly, for ~3 additions per source value.  (M = 2: children of a parent,
-// components alpha; M = 4: cells of a leaf box, no components.)
+// components alpha, or the cells of a leaf-2 box; M = 4: cells of a leaf-4
+// box.  The M2P's targets are the 2 b cells of a parent per axis.)
 //
 // What bounds it: shared-memory reads and FMAs, about equally.  A source
 // value takes 4 reads per (x, y) mirror pair and a weight serves the RZ rows
@@ -320,7 +321,7 @@ __device__ __forceinline__ void sym_m2l_body(const NbrGemm& g, const VBlock& vb)
   const bool add = g.dsplit <= 1 && g.accumulate;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    if (u * 8 + h * 4 >= st.nk) break;
+    if (u * 8 + h * 4 >= g.n_cols / 8) break;
     __syncthreads();  // the stages (first pass) or the previous pass's values are free
 #pragma unroll
     for (int r = 0; r < RZ; ++r)
@@ -332,8 +333,8 @@ __device__ __forceinline__ void sym_m2l_body(const NbrGemm& g, const VBlock& vb)
     __syncthreads();
     const int be = u * 8 + h * 4 + warp;  // this warp's column
     const int x = ox + xl, y = oy + yl;
-    if (be < st.nk && x < g.grid[0] && y < g.grid[1]) {
-      const int p = st.par[be];
+    if (be < g.n_cols / 8 && x < g.grid[0] && y < g.grid[1]) {
+      const int p = g.sym == kSymM2p ? 0 : st.par[be];
 #pragma unroll
       for (int r = 0; r < RZ; ++r) {
         const int z = oz + r;
@@ -342,6 +343,17 @@ __device__ __forceinline__ void sym_m2l_body(const NbrGemm& g, const VBlock& vb)
 #pragma unroll
         for (int s = 0; s < 8; ++s) v[s] = sm[((s * RZ + r) * 4 + warp) * 32 + lane];
         sy_unfold(v, p);
+        if (g.sym == kSymM2p) {  // cell `be` of the upper child, mirrored into the lower ones
+          const int b = g.b, ox = be % b, oy = (be / b) % b, oz = be / (b * b);
+          T* o = C + (((long long)z * g.grid[1] + y) * g.grid[0] + x) * g.n_cols;
+#pragma unroll
+          for (int c = 0; c < 8; ++c) {
+            const int cx = (c & 1) ? ox : b - 1 - ox, cy = (c & 2) ? oy : b - 1 - oy, cz = (c & 4) ? oz : b - 1 - oz;
+            T* oc = o + c * (b * b * b) + (cz * b + cy) * b + cx;
+            *oc = add ? *oc + v[c] : v[c];
+          }
+          continue;
+        }
         T* o = C + (((long long)z * g.grid[1] + y) * g.grid[0] + x) * g.n_cols + be * 8;
         if (add) {
 #pragma unroll

@@ -131,10 +131,84 @@ bool near_case() {
   return err <= 1e-13;
 }
 
+bool near2_case() {
+  SymHost H;
+  sym_near2_weights(H);
+  std::mt19937 rng(8);
+  std::uniform_real_distribution<double> U(0, 1);
+  std::vector<double> A(216);
+  for (double& v : A) v = U(rng);
+  double L[8] = {}, err = 0;
+  for (int k = 0; k < 27; ++k)
+    for (int s = 0; s < 8; ++s)
+      L[s] += block_value(A, 2, k, s, 0) * H.Ws[(((k % 9) * 4 + (s & 3)) * 3 + k / 9) * 2 + (s >> 2)];
+  const int par[3] = {0, 0, 0};
+  for (int c = 0; c < 8; ++c) {
+    double ref = 0;
+    for (int d = 0; d < 27; ++d)
+      for (int sc = 0; sc < 8; ++sc) {
+        const int D[3] = {d % 3 - 1, (d / 3) % 3 - 1, d / 9 - 1};
+        int idx = 0, str = 1;
+        for (int q = 0; q < 3; ++q) idx += str * (2 + 2 * D[q] + ((sc >> q) & 1)), str *= 6;
+        ref += A[idx] * near_entry(2, D, sc, c);
+      }
+    err = std::max(err, std::fabs(unfold(L, c, par) / ref - 1));
+  }
+  std::printf("reflection near leaf 2: err %.1e\n", err);
+  return err <= 1e-13 && H.tab.n1[0] == 1 && H.tab.n8[0] == 0;
+}
+
+bool m2p_case(int p, int b, int mo) {
+  MultiIndex mi;
+  mi.init(p);
+  if (mo >= 0) mi.mo = mo;
+  M2pTable tab;
+  tab.build(mi, b);
+  SymHost H;
+  sym_m2p_weights(mi, tab, b, H);
+  const SymTab& T = H.tab;
+  const std::vector<int> red = harmonic_components(mi);
+  const int b3 = b * b * b;
+  std::mt19937 rng(30 + p);
+  std::uniform_real_distribution<double> U(-1, 1);
+  std::vector<std::vector<double>> A(T.nk, std::vector<double>(216));
+  for (auto& a : A)
+    for (double& v : a) v = U(rng);
+  double err = 0;
+  for (int cell = 0; cell < b3; ++cell) {
+    double L[8] = {};
+    for (int a = 0; a < T.nk; ++a)
+      for (int k = 0; k < 27; ++k)
+        for (int s = 0; s < 8; ++s)
+          L[s] += block_value(A[a], 2, k, s, T.par[a]) *
+                  H.Ws[T.w_off[cell / 8] + (long long)a * 216 * 8 +
+                       ((((k % 9) * 4 + (s & 3)) * 3 + k / 9) * 8 + cell % 8) * 2 + (s >> 2)];
+    const int par[3] = {0, 0, 0}, o[3] = {cell % b, (cell / b) % b, cell / (b * b)};
+    for (int c = 0; c < 8; ++c) {
+      int t[3];
+      for (int q = 0; q < 3; ++q) t[q] = (c >> q) & 1 ? o[q] : b - 1 - o[q];
+      double ref = 0, sabs = 0;
+      for (int a = 0; a < T.nk; ++a)
+        for (int d = 0; d < 27; ++d)
+          for (int cs = 0; cs < 8; ++cs) {
+            const int D[3] = {d % 3 - 1, (d / 3) % 3 - 1, d / 9 - 1};
+            int idx = 0, str = 1;
+            for (int q = 0; q < 3; ++q) idx += str * (2 + 2 * D[q] + ((cs >> q) & 1)), str *= 6;
+            const double v = A[a][idx] * m2p_entry(mi, tab, d, red[a] * 8 + cs, c * b3 + (t[2] * b + t[1]) * b + t[0]);
+            ref += v;
+            sabs += std::fabs(v);
+          }
+      err = std::max(err, std::fabs(unfold(L, c, par) - ref) / sabs);
+    }
+  }
+  std::printf("reflection M2P p=%d b=%d mo=%d: err/sum|terms| %.1e\n", p, b, mi.mo, err);
+  return err <= 1e-13;
+}
+
 }  // namespace
 
 int main() {
-  bool ok = near_case();
+  bool ok = near_case() && near2_case() && m2p_case(3, 2, 2) && m2p_case(4, 4, -1) && m2p_case(6, 2, -1);
   for (int p = 2; p <= 8; ++p) ok &= m2l_case(p, -1, -1);
   ok &= m2l_case(3, 2, -1) && m2l_case(3, -1, 2) && m2l_case(6, 4, -1) && m2l_case(6, -1, 4) && m2l_case(4, 0, -1);
   return ok ? 0 : 1;

@@ -38,7 +38,7 @@ def test_reflection_weights_equal_the_direct_contraction(tmp_path):
     r = subprocess.run([exe], capture_output=True, text=True, timeout=300)
     print(r.stdout)
     assert r.returncode == 0, r.stdout + r.stderr
-    assert r.stdout.count("reflection m2l") == 12
+    assert r.stdout.count("reflection m2l") == 12 and r.stdout.count("reflection M2P") == 3
 
 
 def _rel(a, b):
@@ -75,6 +75,27 @@ def test_reflection_forms_match_oracle(orc, prec, shape, p):
                     pass  # the split scratch does not hold this variant
         err = _rel(_solve(plan, rho), ref)
         assert err <= TOL[prec], (variant, err)
+        plan.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("shape,p,leaf,mo", [((16, 16, 16), 3, 2, 2), ((18, 34, 66), 4, 2, None),
+                                             ((36, 20, 68), 4, 4, 3), ((130, 10, 22), 2, 2, None)])
+def test_reflection_m2p_and_leaf2_near_field_match_oracle(orc, prec, shape, p, leaf, mo):
+    import paper_2606_13793_gb300 as fmm
+
+    rho = inputs.plummer(shape, seed=p).astype(np.float64)
+    ref = orc.fmm_orders(rho, leaf, p, p if mo is None else mo, p, "m2p")
+    for near in (None, (1, 1), (2, 3), (0, 1)):
+        plan = fmm.FMMPlan(shape, p, leaf, prec, final_stage="m2p", mult_order=mo)
+        if near:
+            try:
+                plan.set_tuning(-1, *near)
+            except fmm.FMMError:
+                pass  # the split scratch does not hold this variant
+        err = _rel(_solve(plan, rho), ref)
+        assert err <= TOL[prec], (near, err)
         plan.close()
 
 
