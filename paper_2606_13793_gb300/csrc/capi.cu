@@ -1967,7 +1967,8 @@ fmm_status plan_init(fmm_plan_t P, const int d3[3], double dx, double G, int ord
     // partial sums fit the scratch
     const long long blocks = (long long)((g.grid[0] + 7) / 8) * ((g.grid[1] + 3) / 4) * ((g.grid[2] + 7) / 8) * g.ntiles;
     const size_t part3 = (size_t)3 * g.grid[0] * g.grid[1] * g.grid[2] * (size_t)g.n_cols * (f64 ? 8 : 4);
-    if (blocks < 4 * 152 && part3 <= P->part_cap) c->dsplit = 3;
+    const size_t cap = g.skip_center ? P->part_cap : P->near_part_cap;  // an M2L level's scratch, the near field's
+    if (blocks < 4 * 152 && part3 <= cap) c->dsplit = 3;
   };
   P->arena_bytes = off;
 
