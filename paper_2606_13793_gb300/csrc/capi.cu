@@ -229,6 +229,9 @@ struct fmm_plan_s {
   cudaStream_t last_stream = nullptr;
   // side stream of the concurrent far field (CUDA-core M2L levels), fork/join events
   cudaStream_t side = nullptr;
+  // levels that share no scratch: the unsplit CUDA-core levels, and the
+  // tensor-core levels above the finest one
+  cudaStream_t side2 = nullptr;
   int near_comps = 1;  // near-field columns per cell: potential, + 3 force components (analytic accel)
   // final-stage M2P (the paper's own final stage): leaf interaction list at the cell centres
   bool m2p = false, m2p_tc = false;
@@ -275,7 +278,7 @@ struct fmm_plan_s {
   NearTcLaunch ntl{};
   bool inject_timeout = false;  // test hook (fmm_plan_debug_timeout): the next prefix launch starves its first stage
   TpLaunch tpl{}, tpl_t{}, tpm{}, tpn{};
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_join2 = nullptr;
   // timing
   bool timing = false;
   std::vector<cudaEvent_t> ev_pool;
@@ -360,9 +363,11 @@ struct fmm_plan_s {
     ev_pool.clear();
     if (ev_fork) cudaEventDestroy(ev_fork);
     if (ev_join) cudaEventDestroy(ev_join);
+    if (ev_join2) cudaEventDestroy(ev_join2);
     if (side) cudaStreamDestroy(side);
-    ev_fork = ev_join = nullptr;
-    side = nullptr;
+    if (side2) cudaStreamDestroy(side2);
+    ev_fork = ev_join = ev_join2 = nullptr;
+    side = side2 = nullptr;
     for (void* d : allocs) cudaFree(d);
     allocs.clear();
     for (void* d : {d_io_rho, d_io_phi, d_io_acc, d_io_rho1, d_io_phi1, d_io_acc1})
@@ -2498,6 +2503,8 @@ fmm_status fmm_plan(const fmm_grid* grid, int order, int leaf, const fmm_opts* o
   fmm_status st = plan_init(P, d3, grid->dx, grid->G, order, leaf, o, static_cast<cudaStream_t>(stream), dev);
   if (st == FMM_OK &&
       (cudaStreamCreateWithPriority(&P->side, cudaStreamNonBlocking, side_priority()) != cudaSuccess ||
+       cudaStreamCreateWithFlags(&P->side2, cudaStreamNonBlocking) != cudaSuccess ||
+       cudaEventCreateWithFlags(&P->ev_join2, cudaEventDisableTiming) != cudaSuccess ||
        cudaEventCreateWithFlags(&P->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
        cudaEventCreateWithFlags(&P->ev_join, cudaEventDisableTiming) != cudaSuccess))
     st = fail(FMM_ERR_CUDA, "stream or event creation failed");
@@ -2932,14 +2939,30 @@ fmm_status run_solve(fmm_plan_t P, const T* rho, T* phi, T* accel, cudaStream_t 
     StageTimer t(P, ST_L2L, s);
     CUDA_TRY(launch_zero<T>(static_cast<T*>(P->Lx(L)), P->lev[L].bytes / sizeof(T), s));
   }
-  bool any_simt = false;
-  for (int l = 2; l <= L; ++l) any_simt |= !P->lev[l].tc || P->refl_on(l);
-  const bool fork = P->side && any_simt;
-  cudaStream_t sf = fork ? P->side : s;
-  if (fork) {
-    CUDA_TRY(cudaEventRecord(P->ev_fork, s));
-    CUDA_TRY(cudaStreamWaitEvent(sf, P->ev_fork, 0));
+  // Which levels go where: `s` the finest tensor-core level and the near field;
+  // side2 the other tensor-core levels (few row tiles: their waves then fill
+  // the finest level's last one instead of running alone, 0.2 ms each) and the
+  // unsplit CUDA-core levels beside them, finest first; side the rest (what
+  // uses the split scratch one after another; every level of the CUDA-core
+  // precisions, whose kernels fill the GPU by themselves: 256^3 FP32 0.99 ms
+  // so, 1.01 ms over two streams).
+  bool any_simt = false, any2 = false;
+  int tc_first = -1;
+  auto level2 = [&](int l) {  // CUDA-core level without partial sums, in a plan with tensor-core work
+    return P->tc_kind >= 0 && !rows_level(P, l) && !narrow_level(P, l) && P->m2l_choice[l].dsplit == 1;
+  };
+  for (int l = L; l >= 2; --l) {
+    const bool cc = !P->lev[l].tc || P->refl_on(l);
+    any_simt |= cc;
+    if (p2l && l == L) continue;
+    if (!cc && tc_first < 0) tc_first = l;
+    any2 |= cc ? !(l == L && P->m2p) && level2(l) : l != tc_first;
   }
+  const bool fork = P->side && any_simt, fork2 = P->side2 && any2;
+  cudaStream_t sf = fork ? P->side : s, s2 = fork2 ? P->side2 : s;
+  if (fork || fork2) CUDA_TRY(cudaEventRecord(P->ev_fork, s));
+  if (fork) CUDA_TRY(cudaStreamWaitEvent(sf, P->ev_fork, 0));
+  if (fork2) CUDA_TRY(cudaStreamWaitEvent(s2, P->ev_fork, 0));
   {
     int ls[kMaxLevels], n = 0;
     for (int l = 2; l <= L; ++l)
@@ -2958,9 +2981,14 @@ fmm_status run_solve(fmm_plan_t P, const T* rho, T* phi, T* accel, cudaStream_t 
       CUDA_TRY(launch_nbr_gemm_zrun_group(ng, nn, sf));
     }
     for (int i = 0, k = 0; i < n; ++i) {
-      if (rows_level(P, ls[i]) || (narrow_level(P, ls[i]) && k++ < nn)) continue;
+      if (rows_level(P, ls[i]) || (narrow_level(P, ls[i]) && k++ < nn) || (fork2 && level2(ls[i]))) continue;
       StageTimer t(P, ST_M2L, sf);
       if ((st = do_m2l(P, ls[i], sf))) return st;
+    }
+    for (int i = n - 1; fork2 && i >= 0; --i) {
+      if (!level2(ls[i])) continue;
+      StageTimer t(P, ST_M2L, s2);
+      if ((st = do_m2l(P, ls[i], s2))) return st;
     }
     if (P->m2p && !p2l && !P->lev[L].tc) {
       StageTimer t(P, ST_M2L, sf);
@@ -2972,11 +3000,14 @@ fmm_status run_solve(fmm_plan_t P, const T* rho, T* phi, T* accel, cudaStream_t 
     if ((st = do_p2l(P, sf))) return st;
   }
   if (fork) CUDA_TRY(cudaEventRecord(P->ev_join, sf));
-  for (int l = 2; l <= L; ++l) {
-    if (!P->lev[l].tc || P->refl_on(l) || (p2l && l == L)) continue;
-    StageTimer t(P, ST_M2L_TC, s);
-    if ((st = (l == L && P->m2p) ? do_m2p(P, s) : do_m2l(P, l, s))) return st;
-  }
+  for (int k = 0; k < 2; ++k)  // the finest level first: the others' CTAs queue behind it
+    for (int l = 2; l <= L; ++l) {
+      if (!P->lev[l].tc || P->refl_on(l) || (p2l && l == L) || (l == tc_first) != (k == 0)) continue;
+      cudaStream_t st2 = l == tc_first ? s : s2;
+      StageTimer t(P, ST_M2L_TC, st2);
+      if ((st = (l == L && P->m2p) ? do_m2p(P, st2) : do_m2l(P, l, st2))) return st;
+    }
+  if (fork2) CUDA_TRY(cudaEventRecord(P->ev_join2, s2));
   // near field over the 27 neighbour leaf boxes
   if (adj_g) {  // the transposed near field of the potential and the force, one output column
     StageTimer t(P, ST_NEAR, s);
@@ -3004,6 +3035,7 @@ fmm_status run_solve(fmm_plan_t P, const T* rho, T* phi, T* accel, cudaStream_t 
     CUDA_TRY(launch_nbr_gemm<T>(near_gemm(P), s));
   }
   if (fork) CUDA_TRY(cudaStreamWaitEvent(s, P->ev_join, 0));
+  if (fork2) CUDA_TRY(cudaStreamWaitEvent(s, P->ev_join2, 0));
   if (L >= 2 && harmonic_m2l_level(P, 2)) {  // level 2 locals are its M2L alone: rebuild
     StageTimer t(P, ST_L2L, s);
     if ((st = do_l2l(P, tt, 2, s, 1))) return st;
