@@ -135,6 +135,31 @@ def algorithmic_counts(dims, leaf, p):
     return {"m2l_flop": m2l_flop, "near_flop": near_flop}
 
 
+def mirror_products(leaf, fp64, harmonic, variant, near=False, accel_columns=False):
+    """Share of the pairwise products a CUDA-core contraction multiplies: an
+    eighth where it runs in the basis of sums and differences over mirror pairs
+    (harmonic M2L and M2P in FP64 or on the z-run tiles, shapes 1 and 2; the
+    near field of leaf 2 and 4 on those tiles, without force columns)."""
+    zrun = variant is not None and variant[0] in (1, 2)
+    if near:
+        return 1 / 8 if zrun and leaf in (2, 4) and not accel_columns else 1
+    return 1 / 8 if harmonic and (fp64 or zrun) else 1
+
+
+def batch_products(sizes, leaf, p, fp64):
+    """Flops of one fused batch step's contractions as multiplied: the leaf
+    level (every level in FP64) and the near field of leaf 4 an eighth of the
+    pairwise products, the other FP32 levels all of them."""
+    total = 0
+    for s in sizes:
+        lev = hierarchy((s, s, s), leaf)
+        for l in range(2, len(lev)):
+            total += m2l_flop_level((s, s, s), leaf, p, l, p >= 2) * \
+                mirror_products(leaf, fp64, p >= 2, (1, 1) if l == len(lev) - 1 else (0, 1))
+        total += algorithmic_counts((s, s, s), leaf, p)["near_flop"] * mirror_products(leaf, fp64, False, (1, 1), near=True)
+    return total
+
+
 def batch_contraction_flops(sizes, leaf, p):
     """Algorithmic flops of one batch step's contractions: every M2L level of
     every cubic field (the CUDA-core contraction on the (p+1)^2 harmonic
@@ -148,13 +173,13 @@ def batch_contraction_flops(sizes, leaf, p):
     return total
 
 
-def batch_roofline(sizes, leaf, p, precision, ms_per_step, peaks):
-    """Roofline of the fused batch's contraction launches (the z-run and the
-    tiny-grid multi-field launches, 92% of the launch list), timed as the
-    whole step: a lower bound on their rate, against the CUDA-core FMA peak
-    of the precision (FP32 from the unit counts and the maximum clock, FP64
-    nominal)."""
-    flop = batch_contraction_flops(sizes, leaf, p)
+def batch_roofline(sizes, leaf, p, precision, ms_per_step, peaks, flop=None):
+    """Roofline of the fused batch's contraction launches (most of the launch
+    list), timed as the whole step: a lower bound on their rate, against the
+    CUDA-core FMA peak of the precision (FP32 from the unit counts and the
+    maximum clock, FP64 nominal).  flop: products counted (default: every
+    pairwise product of the method)."""
+    flop = batch_contraction_flops(sizes, leaf, p) if flop is None else flop
     if precision == "fp64":
         peak, note = 1.25, "FP64 1.25 TFLOP/s (nominal)"
     else:
@@ -162,7 +187,7 @@ def batch_roofline(sizes, leaf, p, precision, ms_per_step, peaks):
         note = "FP32 FFMA 152 SMs x 128 lanes x 2 x max clock"
     ach = flop / (ms_per_step / 1e3) / 1e12
     return {"bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak, "traffic": None,
-            "kernel": "nbr_gemm_zrun_multi + nbr_gemm_tiny_multi (contraction launches)",
+            "kernel": "contraction launches (reflection basis, direct z-run and tiny grids)",
             "peak_source": "derived: " + note, "flop_per_step": flop,
             "timing": "whole batch step (a lower bound on the contraction launches' rate)"}
 
@@ -525,7 +550,10 @@ def main():
         hl = harmonic if k == "tensor" else harmonic_cc
         f = m2p_flop_leaf((n, n, n), b, p, hl) if (l == L and args.final_stage == "m2p") else \
             m2l_flop_level((n, n, n), b, p, l, hl)
-        flop_by["m2l_tc" if k == "tensor" else "m2l"] += f
+        # products the CUDA cores multiply, so that a fraction of their rate means what it says
+        m2p = l == L and args.final_stage == "m2p"
+        cut = 1 if k == "tensor" or (m2p and b not in (2, 4)) else mirror_products(b, k == "fp64", hl, tuning.get(str(l)))
+        flop_by["m2l_tc" if k == "tensor" else "m2l"] += f * cut
     simt64 = any(k == "fp64" for k in kinds.values())
     bf16_peak = peaks["bf16_tflops_sustained"]
     fp32_peak = 152 * 128 * 2 * peaks.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
@@ -538,7 +566,9 @@ def main():
         "near_field_tc": (counts["near_flop"], 3, "tensor", bf16_peak, "bf16 sustained (measured)"),
         "m2l": (flop_by["m2l"], 1, "alu", 1.25 if simt64 else fp32_peak,
                 "FP64 1.25 TFLOP/s (nominal)" if simt64 else "FP32 FFMA 152 SMs x 128 lanes x 2 x max clock"),
-        "near_field": (counts["near_flop"], 1, "alu", fp32_peak, "FP32 FFMA 152 SMs x 128 lanes x 2 x max clock"),
+        "near_field": (counts["near_flop"] * mirror_products(b, simt64, False, tuning.get("near"), True,
+                                                             args.accel == "analytic"),
+                       1, "alu", fp32_peak, "FP32 FFMA 152 SMs x 128 lanes x 2 x max clock"),
     }
     per_kernel = {}
     for k, (flop, passes, bound, peak_val, note) in kern.items():
@@ -713,7 +743,8 @@ def batch_main(args, fmm, inputs, torch, dist, rank, world):
                                cells * args.steps * world / (seq_ms / 1e3) / 1e6,
                            "l2": "inputs larger than L2 (all fields together)",
                            "parallelism": f"replicas x{world}"},
-                "roofline": (batch_roofline(sizes, b, p, prec, ms / args.steps, measured_peaks()[0])
+                "roofline": (batch_roofline(sizes, b, p, prec, ms / args.steps, measured_peaks()[0],
+                                            batch_products(sizes, b, p, prec == "fp64"))
                              if batch.fused == 1 else None),
                 "cpu_baseline": None, "e2e": e2e,
                 "gpu_launches": batch.launches(True) * args.steps, "clocks": clk.summary()}

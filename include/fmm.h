@@ -297,6 +297,12 @@ fmm_status fmm_solve_static(const fmm_grid* grid, int order, int leaf, const voi
  *                         it; shapes 1 and 2 are not used there), and the
  *                         number of blocks sharing the 27 neighbours of a row
  *                         tile (shapes 0, 3: 1 or 27; shapes 1, 2: 1, 3 or 9).
+ *                         Shapes 1 and 2 of harmonic M2L levels and of the
+ *                         near field of leaf 2 and 4, and shapes 0 and 3 of
+ *                         harmonic FP64 levels, run the contraction in the
+ *                         basis of sums and differences over mirror pairs
+ *                         (the same operator, an eighth of the products)
+ *                         with the same row tiles.
  *   fmm_plan_set_tuning : sets it; FMM_ERR_ARG if the variant does not apply
  *                         (level on the tensor cores, reduction lengths not a
  *                         multiple of 8, split scratch too small).
@@ -403,8 +409,8 @@ fmm_status fmm_batch_destroy(fmm_batch_t batch);
 fmm_status fmm_batch_set_fused(fmm_batch_t batch, int enable);
 int fmm_batch_is_fused(fmm_batch_t batch);
 /* Kernel launches one fmm_batch_solve graph holds: the fused form's step
- * count when the plans qualify for it (and it is enabled), else the sum over
- * the plans. */
+ * count when the plans qualify for it (and it is enabled; a contraction step
+ * holds up to three kernels), else the sum over the plans. */
 int fmm_batch_launches(fmm_batch_t batch, int with_accel);
 
 /* fmm_check -- synchronises the plan's last stream and reports device-side
@@ -424,7 +430,8 @@ int fmm_solve_launches(fmm_plan_t plan, int with_accel);
  *   fmm_timing_enable : 1 starts recording (and clears totals), 0 stops.
  *                       Creates its event pool here, not during solves.
  *   fmm_timing_read   : synchronises, then writes for each stage i < nstages
- *                       the summed milliseconds ms[i] and launch count
+ *                       the milliseconds ms[i] covered by its launches (those
+ *                       that run side by side count once) and the launch count
  *                       launches[i] since the last enable/read, and clears them.
  * Stages (index: name): see fmm_timing_stage_name().  Errors: FMM_ERR_ARG
  * (NULL plan or arrays), FMM_ERR_CUDA (event creation or timing failure).

@@ -3327,14 +3327,31 @@ fmm_status fmm_timing_read(fmm_plan_t P, double* ms, int* launches, int nstages)
   if (!ms || !launches || nstages <= 0) return fail(FMM_ERR_ARG, "bad output arrays");
   CUDA_TRY(cudaDeviceSynchronize());
   for (int i = 0; i < nstages; ++i) ms[i] = 0.0, launches[i] = 0;
+  // Launches of a stage on two streams may overlap: the union of their spans.
+  // A span is kept from the first event of a run of overlapping launches.
+  struct Span {
+    cudaEvent_t from = nullptr;
+    float lo = 0.f, hi = 0.f;  // against `from`
+  };
+  std::vector<Span> open((size_t)nstages);
   for (const auto& r : P->recs) {
-    float t = 0.f;
-    CUDA_TRY(cudaEventElapsedTime(&t, r.a, r.b));
-    if (r.stage < nstages) {
-      ms[r.stage] += t;
-      launches[r.stage] += 1;
+    if (r.stage >= nstages) continue;
+    Span& sp = open[(size_t)r.stage];
+    launches[r.stage] += 1;
+    float a = 0.f, b = 0.f;
+    if (sp.from) {
+      CUDA_TRY(cudaEventElapsedTime(&a, sp.from, r.a));
+      CUDA_TRY(cudaEventElapsedTime(&b, sp.from, r.b));
+      if (a <= sp.hi && b >= sp.lo) {
+        sp.lo = std::min(sp.lo, a), sp.hi = std::max(sp.hi, b);
+        continue;
+      }
+      ms[r.stage] += sp.hi - sp.lo;
     }
+    sp.from = r.a, sp.lo = 0.f;
+    CUDA_TRY(cudaEventElapsedTime(&sp.hi, r.a, r.b));
   }
+  for (int i = 0; i < nstages; ++i) ms[i] += open[(size_t)i].hi - open[(size_t)i].lo;
   P->recs.clear();
   P->ev_used = 0;
   return FMM_OK;
