@@ -137,9 +137,6 @@ cudaError_t launch_nbr_gemm_zrun_group(const NbrGemm* gs, int n, cudaStream_t s)
 // for the partial sums; the sums of the simt kernel, bit for bit.
 constexpr int kRowsGroupMax = 8;
 cudaError_t launch_nbr_gemm_rows(const NbrGemm* gs, int n, cudaStream_t s);
-// Whether that kernel takes this contraction (dsplit 27, reduction lengths
-// and column counts multiples of 8).
-bool nbr_gemm_rows_fits(const NbrGemm& g, const int* tile_k_host, int ntiles);
 
 // The reflection-basis row form (shapes 0 and 3) over up to kSymGroupMax levels of one plan in
 // one launch, same shape and split, each with its own scratch for the partial sums.

@@ -10,19 +10,23 @@
 //
 // These levels (8, 64, 512 rows) are bound by latency: a chain of up to
 // 8 (p+1)^2 multiply-adds per output, and a kernel each.  So: one launch for
-// all of a plan's coarse levels; one warp per (64 rows x 32 columns,
-// neighbour), independent of the others (no block barrier), its operands by
-// double-buffered 16-byte cp.async in chunks of 32 values of k; an 8 x 8
-// register tile per lane (16 floats read for 64 multiply-adds, the ratio at
-// which shared memory and the FMA pipe run level), cut to the live rows of
-// the block; the longest column tiles first.
+// all of a plan's coarse levels; one warp per (32 rows x 32 columns,
+// neighbour), a CTA of its own, so that the long column tiles, first in the
+// grid, spread over all SMs; its operands by double-buffered 16-byte cp.async
+// in chunks of 32 values of k; a 4 x 8 register tile per lane, cut to the
+// live rows of the block.  Levels 2-4 at p = 6, launch by launch: 540 us as
+// three 4 x 4 x 4 launches, 56 us as one with 64 rows and four warps a CTA;
+// whole 64^3 solve 112 us so, 116 us with one warp a CTA, 107 us with 32 rows
+// and four, 105 us with 32 rows and one (12 warps an SM instead of 8, and the
+// longest chain of multiply-adds halved).
 #include "fmm_internal.h"
 
 namespace fmmgb {
 namespace {
 
-constexpr int kRwWarps = 4;    // independent warps per CTA
-constexpr int kRwRows = 64;    // rows per warp
+constexpr int kRwWarps = 1;    // independent warps per CTA
+constexpr int kRwRows = 32;    // rows per warp
+constexpr int kRwTR = kRwRows / 8;  // rows per lane
 constexpr int kRwKC = 32;      // reduction values per stage
 constexpr int kRwPitch = kRwKC + 4;
 constexpr int kRwStage = kRwRows * kRwPitch + kRwKC * kNTile;  // floats
@@ -54,7 +58,7 @@ __device__ __forceinline__ unsigned long long rw_splat(float a) {
 // One stage: rows rg + 8 i (i < TR), columns 8 cg .. 8 cg + 7, k ascending.
 template <int TR>
 __device__ __forceinline__ void rw_stage(const float* As, const float* Ws, int kn, int rg, int cg,
-                                         unsigned long long (&acc)[8][4]) {
+                                         unsigned long long (&acc)[kRwTR][4]) {
   for (int k0 = 0; k0 < kn; k0 += 4) {
     float4 a[TR];
 #pragma unroll
@@ -123,9 +127,9 @@ __global__ void __launch_bounds__(32 * kRwWarps) nbr_gemm_rows_kernel(const __gr
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   const int rg = lane & 7, cg = lane >> 3;
-  unsigned long long acc[8][4];
+  unsigned long long acc[kRwTR][4];
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
+  for (int i = 0; i < kRwTR; ++i)
 #pragma unroll
     for (int c = 0; c < 4; ++c) acc[i][c] = 0ull;
   load(0, st);
@@ -136,10 +140,10 @@ __global__ void __launch_bounds__(32 * kRwWarps) nbr_gemm_rows_kernel(const __gr
     const float* As = st + b * kRwStage;
     const float* Ws = As + kRwRows * kRwPitch;
     const int kn = min(kRwKC, K - kc);
-    if (live > 32)
-      rw_stage<8>(As, Ws, kn, rg, cg, acc);
-    else if (live > 16)
-      rw_stage<4>(As, Ws, kn, rg, cg, acc);
+    if (live > 8 * (kRwTR / 2))
+      rw_stage<kRwTR>(As, Ws, kn, rg, cg, acc);
+    else if (kRwTR > 4 && live > 16)
+      rw_stage<kRwTR < 4 ? kRwTR : 4>(As, Ws, kn, rg, cg, acc);
     else if (live > 8)
       rw_stage<2>(As, Ws, kn, rg, cg, acc);
     else
@@ -150,7 +154,7 @@ __global__ void __launch_bounds__(32 * kRwWarps) nbr_gemm_rows_kernel(const __gr
   if (col >= g.n_cols) return;  // a multiple of 8
   float* P = static_cast<float*>(g.partial) + (long long)d * rows * g.n_cols;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
+  for (int i = 0; i < kRwTR; ++i) {
     const int r = r0 + rg + 8 * i;
     if (r >= rows) break;
     ulonglong2* o = reinterpret_cast<ulonglong2*>(P + (long long)r * g.n_cols + col);
@@ -181,13 +185,6 @@ __global__ void __launch_bounds__(kRwRed) nbr_rows_reduce_kernel(const __grid_co
 }
 
 }  // namespace
-
-bool nbr_gemm_rows_fits(const NbrGemm& g, const int* tile_k_host, int ntiles) {
-  if (g.row_len % 8 != 0 || g.n_cols % 8 != 0 || g.dsplit != 27) return false;
-  for (int i = 0; i < ntiles; ++i)
-    if (tile_k_host[i] % 8 != 0) return false;
-  return true;
-}
 
 cudaError_t launch_nbr_gemm_rows(const NbrGemm* gs, int n, cudaStream_t s) {
   if (n < 1 || n > kRowsGroupMax) return cudaErrorInvalidValue;
