@@ -1757,14 +1757,17 @@ NbrGemm near_gemm(fmm_plan_t P);
 // 32^3 .. 256^3 cells (FP32 p = 6, FP64 p = 4, 6):
 //  * M2L levels of at most 512 rows: the row forms, split 27 ways (one launch
 //    for all of them; FP64 in the reflection basis, 8 rows a block);
-//  * other M2L levels: the long z-run from 100 tiles on (64^3 rows 2.9 ms
-//    against 3.4 ms with the short one, 32^3 0.51 against 0.56 ms, 24^3 0.32
-//    against 0.23 ms), else the short one split until 304 blocks (two per SM)
+//  * other M2L levels: the long z-run from 100 tiles on (whole solves: 256^3,
+//    32^3 rows, 0.998 ms against 1.015 ms with the short one; 192^3, 24^3
+//    rows, 0.665 against 0.614 ms), else the short one split until 304 blocks (two per SM)
 //    run; FP64
 //    until the first unit's blocks, half of all work, fill the SMs twice
 //    (12^3 rows: 9 ways 1.25 ms, 3 ways 1.38 ms);
-//  * near field: the long z-run from 100 tiles on (32^3 boxes 46 us, short 55),
-//    else the short one, FP32 split until 32 blocks run (16^3 boxes: 31 us
+//  * near field: the long z-run from 100 tiles on (FP32 leaf 4: from 1000 on,
+//    its blocks share the SMs with the M2L's and the short ones pack better;
+//    whole solves with the short and the long one: 128^3 0.283 and 0.295 ms,
+//    192^3 0.572 and 0.616, 256^3 1.008 and 0.999), else
+//    the short one, FP32 split until 32 blocks run (16^3 boxes: 31 us
 //    unsplit, 57 us in three beside the M2L), FP64 until every SM has one.
 void sym_default(fmm_plan_t P, const NbrGemm& g, fmm_plan_s::SimtChoice* c, bool f64) {
   const long long rows = (long long)g.grid[0] * g.grid[1] * g.grid[2];
@@ -1778,7 +1781,7 @@ void sym_default(fmm_plan_t P, const NbrGemm& g, fmm_plan_s::SimtChoice* c, bool
     return d;
   };
   if (!g.skip_center) {  // the near field
-    c->shape = tiles(f64 ? 4 : 8) >= 100 ? 1 : 2;
+    c->shape = tiles(f64 ? 4 : 8) >= (f64 || P->b != 4 ? 100 : 1000) ? 1 : 2;
     c->dsplit = c->shape == 1 ? 1 : split(tiles(f64 ? 2 : 4), f64 ? 152 : 32, P->near_part_cap);
   } else if (c->dsplit == 27 && rows <= 512 && 27 * one <= P->part_cap) {
     c->shape = f64 ? 3 : 0;
@@ -1796,9 +1799,9 @@ void sym_default(fmm_plan_t P, const NbrGemm& g, fmm_plan_s::SimtChoice* c, bool
 // a wave of row tiles (one per SM, 128 rows each) takes a tile's latency
 // however few there are, 0.195 ms at p = 6 and 0.40 ms at p = 8 (prefix
 // schedule: 32 to 152 tiles 0.197 ms, 256 tiles 0.393, 2048 tiles 2.71 ms),
-// while the reflection basis costs 10.9 (p = 6) or 28 ns a row (16^3 rows 0.064,
-// 32^3 0.36, 64^3 2.86 ms): it wins below ~14000 rows a wave (a full one has
-// 19456).  Both sums are FP32, this one of unsplit operands.  A caller that
+// while the reflection basis costs about 10 (p = 6) or 28 ns a row (p = 6: 16^3
+// rows 0.064, 32^3 0.34, 64^3 2.25 ms): it wins below ~14000 rows a wave at
+// p = 8; a full one has 19456, for which the two are close at p = 6.  Both sums are FP32, this one of unsplit operands.  A caller that
 // lowers n_fp64_levels asks for the tensor cores on small levels and gets them.
 // Plans with the stencil force stay on them too: the stencil amplifies what
 // the split operands round (512^3: level 5 alone is 2.5e-5 of the force), and

@@ -27,7 +27,7 @@
 //    signs of z in the two halves of a packed pair, so that the weights (one
 //    pair per column) need no splat.  The four warps exchange their blocks
 //    through shared memory at the end.  Against the direct z-run tiles of
-//    k_gemm_zrun.cu (GB300): FP32 p = 6, 32^3 rows (256^3 cells) 1.48 -> 0.36
+//    k_gemm_zrun.cu (GB300): FP32 p = 6, 32^3 rows (256^3 cells) 1.48 -> 0.33
 //    ms, its near field 1.11 -> 0.28 ms; FP64 p = 6, 12^3 rows 7.6 -> 1.1 ms,
 //    24^3 boxes 2.9 -> 0.63 ms.  Of the issue slots ~45% are used: 8 warps an
 //    SM, the 128 accumulator registers a thread (RZ = 8, N = 8) allow no more,
