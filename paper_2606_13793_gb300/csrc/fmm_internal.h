@@ -94,7 +94,11 @@ enum SymKind { kSymNone = 0, kSymM2l = 1, kSymNear4 = 2, kSymM2p = 3 };
 // Neighbour-contraction ("implicit GEMM") description for the SIMT kernel:
 //   C[row][n] (+)= sum_{d in 27 neighbours} sum_{k < K(tile(n))} A[row + d][k] * W_d[k][n]
 // rows live on a 3-D grid; a neighbour outside the grid contributes zero.
-struct NbrGemm {
+// The kernels of the direct form (k_gemm_simt.cu, k_gemm_zrun.cu) take this part
+// alone: with the reflection basis' fields in their parameters they compile to
+// other registers (the long FP32 z-run on a leaf-8 near field with force columns,
+// 12^3 boxes: 3.98 ms, 3.90 ms without).
+struct DirectGemm {
   const void* A;       // [rows][row_len]
   int row_len;
   int grid[3];         // row grid extents
@@ -113,6 +117,9 @@ struct NbrGemm {
   int max_blocks = 0;  // shape 0: at most this many CTAs, each looping over work items (0: one per item)
   int skip_center = 0; // 1: W_d of the centre neighbour (d = 13) is all zero (the M2L: a parent's
                        // children are each other's near neighbours), and the kernels skip it
+};
+static_assert(sizeof(DirectGemm) == 96, "the fields of the direct form only");
+struct NbrGemm : DirectGemm {
   // reflection-basis form (k_sym.cu), SymKind.  kSymM2l: A is component-major,
   // [8 alpha + child][lda rows]; kSymNear4: A as above
   int sym = 0;

@@ -35,7 +35,7 @@ template <typename T>
 constexpr int kChunkOf = sizeof(T) == 8 ? kKChunk / 2 : kKChunk;
 
 template <typename T>
-__device__ __forceinline__ void nbr_gemm_simt_body(const NbrGemm& g, const VBlock vb) {
+__device__ __forceinline__ void nbr_gemm_simt_body(const DirectGemm& g, const VBlock vb) {
   constexpr int KC = kChunkOf<T>;
   __shared__ T As[KC][kRows + kPad];
   __shared__ T Bs[KC][kNTile];
@@ -123,14 +123,14 @@ __device__ __forceinline__ void nbr_gemm_simt_body(const NbrGemm& g, const VBloc
 }
 
 template <typename T>
-__global__ void __launch_bounds__(64) nbr_gemm_simt_kernel(NbrGemm g) {
+__global__ void __launch_bounds__(64) nbr_gemm_simt_kernel(DirectGemm g) {
   nbr_gemm_simt_body<T>(g, native_vblock());
 }
 
 template <typename T>
 __global__ void __launch_bounds__(64) nbr_gemm_simt_multi_kernel(const NbrGemm* __restrict__ gs,
                                                                  const MultiGrid* __restrict__ grids, int n) {
-  __shared__ NbrGemm g;  // the item's description, read by the body from shared memory
+  __shared__ DirectGemm g;  // the item's description, read by the body from shared memory
   const int i = multi_item(grids, n);
   if (threadIdx.x == 0) g = gs[i];
   __syncthreads();
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(64) nbr_gemm_simt_multi_kernel(const NbrGemm* 
 constexpr int kColRows = 4;  // rows per warp
 
 template <typename T>
-__device__ __forceinline__ void nbr_gemm_col_body(const NbrGemm& g, const VBlock vb) {
+__device__ __forceinline__ void nbr_gemm_col_body(const DirectGemm& g, const VBlock vb) {
   constexpr int R = kColRows;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long rows = (long long)g.grid[0] * g.grid[1] * g.grid[2];
@@ -207,14 +207,14 @@ __device__ __forceinline__ void nbr_gemm_col_body(const NbrGemm& g, const VBlock
 }
 
 template <typename T>
-__global__ void __launch_bounds__(128) nbr_gemm_col_kernel(NbrGemm g) {
+__global__ void __launch_bounds__(128) nbr_gemm_col_kernel(DirectGemm g) {
   nbr_gemm_col_body<T>(g, native_vblock());
 }
 
 template <typename T>
 __global__ void __launch_bounds__(128) nbr_gemm_col_multi_kernel(const NbrGemm* __restrict__ gs,
                                                                  const MultiGrid* __restrict__ grids, int n) {
-  __shared__ NbrGemm g;  // the item's description, read by the body from shared memory
+  __shared__ DirectGemm g;  // the item's description, read by the body from shared memory
   const int i = multi_item(grids, n);
   if (threadIdx.x == 0) g = gs[i];
   __syncthreads();
@@ -265,7 +265,7 @@ __device__ __forceinline__ void tiny_steps(const T* a0p, const T* a1p, bool v0, 
 }
 
 template <typename T>
-__device__ __forceinline__ void nbr_gemm_tiny_body(const NbrGemm& g, const VBlock vb) {
+__device__ __forceinline__ void nbr_gemm_tiny_body(const DirectGemm& g, const VBlock vb) {
   __shared__ T part[(kTinyKS > 1 ? kTinyKS - 1 : 1) * 256 * 8];
   const int tile = vb.x;
   const int kp = threadIdx.x >> 8, tl = threadIdx.x & 255;  // reduction part, thread in the part
@@ -354,7 +354,7 @@ template <typename T>
 __global__ void __launch_bounds__(kTinyThreads) nbr_gemm_tiny_multi_kernel(const NbrGemm* __restrict__ gs,
                                                                            const MultiGrid* __restrict__ grids,
                                                                            int n, long long first, int nx) {
-  __shared__ NbrGemm g;  // the item's description, read by the body from shared memory
+  __shared__ DirectGemm g;  // the item's description, read by the body from shared memory
   const long long b = (long long)blockIdx.x + first;
   int i = multi_item_at(grids, n, b);
   VBlock vb = multi_vblock_at(grids[i], b);

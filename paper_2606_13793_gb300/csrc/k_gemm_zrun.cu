@@ -77,7 +77,7 @@ constexpr size_t zrun_smem_bytes() {
 }
 
 template <typename T, int RZ>
-__device__ __forceinline__ void nbr_gemm_zrun_body(const NbrGemm& g, const VBlock vb) {
+__device__ __forceinline__ void nbr_gemm_zrun_body(const DirectGemm& g, const VBlock vb) {
   using H = ZrHalo<RZ>;
   using V = typename Vec<T>::type;
   constexpr int VN = Vec<T>::n;
@@ -215,7 +215,7 @@ __device__ __forceinline__ void nbr_gemm_zrun_body(const NbrGemm& g, const VBloc
 }
 
 template <typename T, int RZ>
-__global__ void __launch_bounds__(kZrThreads, 4) nbr_gemm_zrun_kernel(NbrGemm g) {
+__global__ void __launch_bounds__(kZrThreads, 4) nbr_gemm_zrun_kernel(DirectGemm g) {
   nbr_gemm_zrun_body<T, RZ>(g, native_vblock());
 }
 
@@ -223,7 +223,7 @@ template <typename T, int RZ>
 __global__ void __launch_bounds__(kZrThreads, 4) nbr_gemm_zrun_multi_kernel(const NbrGemm* __restrict__ gs,
                                                                          const MultiGrid* __restrict__ grids, int n,
                                                                          long long first) {
-  __shared__ NbrGemm g;  // the item's description, read by the body from shared memory
+  __shared__ DirectGemm g;  // the item's description, read by the body from shared memory
   const long long b = (long long)blockIdx.x + first;
   const int i = multi_item_at(grids, n, b);
   if (threadIdx.x == 0) g = gs[i];
@@ -245,7 +245,7 @@ constexpr int narrow_smem() {  // floats
   return 27 * kZrKC * 8 + kZrKC * ZrHalo<RZ>::stride;
 }
 template <int RZ>
-__device__ __forceinline__ void zrun_narrow_body(const NbrGemm& g, const VBlock& vb, int cg, float* sm) {
+__device__ __forceinline__ void zrun_narrow_body(const DirectGemm& g, const VBlock& vb, int cg, float* sm) {
   using H = ZrHalo<RZ>;
   constexpr int HR = RZ / 2;
   constexpr int kA = (H::rows * 2 + kZrThreads - 1) / kZrThreads;  // float4 of A per thread and stage
@@ -350,7 +350,7 @@ template <int RZ>
 __global__ void __launch_bounds__(kZrThreads) zrun_narrow_multi_kernel(const NbrGemm* __restrict__ gs,
                                                                        const MultiGrid* __restrict__ grids, int n,
                                                                        long long first, int ny) {
-  __shared__ NbrGemm g;
+  __shared__ DirectGemm g;
   VBlock vb;
   const int it = multi_tile_major(grids, n, first, gridDim.x >> 2, ny, blockIdx.x >> 2, &vb);
   if (threadIdx.x == 0) g = gs[it];
