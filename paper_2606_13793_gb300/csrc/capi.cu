@@ -2880,6 +2880,26 @@ fmm_status do_m2l_rows(fmm_plan_t P, const std::vector<int>& ls, cudaStream_t s)
   return FMM_OK;
 }
 
+// Stream of the CUDA-core levels beside the near field (and of the final
+// stage): `side`, whose higher priority starts their few blocks first.  A
+// leaf-8 near field off the tensor cores runs for milliseconds in direct tiles,
+// four register-full CTAs an SM; levels that started first spread its CTAs
+// unevenly, and its last wave then piles up on a few SMs.  There the levels (20
+// us of work) go on `side2`, at the near field's own priority (FP32, order 4):
+// 96^3 with force columns 5.32 -> 4.54 ms, 160^3 4.46 -> 3.58 ms.  With the
+// final-stage M2P, itself as long, they keep `side` (adjoint at 208 x 216 x 136,
+// order 3: 14.0 ms, 21.3 ms on `side2`), and a split near field runs behind it
+// (near_behind).
+cudaStream_t levels_stream(fmm_plan_t P, bool adj_g) {
+  return !P->near_tc && P->b == 8 && !P->m2p && !adj_g ? P->side2 : P->side;
+}
+// Whether the near field runs on the levels' stream, after the final stage: a
+// split leaf-8 one, whose blocks and the direct M2P's (as long) only hold each
+// other up (FP64, 56 x 48 x 40, order 6: 29.9 ms so, 42.1 ms side by side).
+bool near_behind(fmm_plan_t P, bool adj_g) {
+  return !P->near_tc && P->b == 8 && P->m2p && P->near_choice.dsplit > 1 && !adj_g;
+}
+
 // adjoint = true (fmm_solve_adjoint): the same chain on the adjoint source,
 // except that with the final-stage M2P the leaf level runs its transpose
 // (P2L into the leaf locals, then L2L adds the parents' and L2P evaluates);
@@ -2962,7 +2982,7 @@ fmm_status run_solve(fmm_plan_t P, const T* rho, T* phi, T* accel, cudaStream_t 
     any2 |= cc ? !(l == L && P->m2p) && level2(l) : l != tc_first;
   }
   const bool fork = P->side && any_simt, fork2 = P->side2 && any2;
-  cudaStream_t sf = fork ? P->side : s, s2 = fork2 ? P->side2 : s;
+  cudaStream_t sf = fork ? levels_stream(P, adj_g != nullptr) : s, s2 = fork2 ? P->side2 : s;
   if (fork || fork2) CUDA_TRY(cudaEventRecord(P->ev_fork, s));
   if (fork) CUDA_TRY(cudaStreamWaitEvent(sf, P->ev_fork, 0));
   if (fork2) CUDA_TRY(cudaStreamWaitEvent(s2, P->ev_fork, 0));
@@ -3002,6 +3022,11 @@ fmm_status run_solve(fmm_plan_t P, const T* rho, T* phi, T* accel, cudaStream_t 
     StageTimer t(P, ST_M2L, sf);
     if ((st = do_p2l(P, sf))) return st;
   }
+  const bool behind = fork && near_behind(P, adj_g != nullptr);
+  if (behind) {
+    StageTimer t(P, ST_NEAR, sf);
+    CUDA_TRY(launch_nbr_gemm<T>(near_gemm(P), sf));
+  }
   if (fork) CUDA_TRY(cudaEventRecord(P->ev_join, sf));
   for (int k = 0; k < 2; ++k)  // the finest level first: the others' CTAs queue behind it
     for (int l = 2; l <= L; ++l) {
@@ -3033,7 +3058,7 @@ fmm_status run_solve(fmm_plan_t P, const T* rho, T* phi, T* accel, cudaStream_t 
   } else if (P->near_tc) {
     StageTimer t(P, ST_NEAR_TC, s);
     if ((st = do_near_tc(P, s))) return st;
-  } else {
+  } else if (!behind) {
     StageTimer t(P, ST_NEAR, s);
     CUDA_TRY(launch_nbr_gemm<T>(near_gemm(P), s));
   }

@@ -20,11 +20,55 @@ void direct_gemm() {
   expect(reinterpret_cast<const char*>(&d) == reinterpret_cast<const char*>(&g), "its fields come first");
 }
 
+// A plan's layout without device memory, with placeholder side streams.
+struct Dry {
+  fmm_plan_t P;
+  Dry(int nx, int ny, int nz, int order, int leaf, const fmm_opts& o) : P(new fmm_plan_s) {
+    P->static_base = reinterpret_cast<unsigned char*>((uintptr_t)1 << 40);
+    P->static_cap = (size_t)1 << 39;
+    P->static_keep_tables = P->dry = true;
+    const int d3[3] = {nx, ny, nz};
+    expect(plan_init(P, d3, 1.0, 1.0, order, leaf, o, nullptr, 0) == FMM_OK, fmm_last_error());
+  }
+  ~Dry() { delete P; }
+};
+fmm_opts opts(int precision, int accel, int final_stage = 0) {
+  fmm_opts o;
+  fmm_default_opts(&o);
+  o.precision = precision;
+  o.accel = accel;
+  o.final_stage = final_stage;
+  return o;
+}
+
+// The levels beside a leaf-8 near field off the tensor cores run at its own
+// priority; with the final-stage M2P on the high-priority stream, a split near
+// field behind it; other leaves as ever.
+void leaf8_streams() {
+  cudaStream_t hi = reinterpret_cast<cudaStream_t>(16), lo = reinterpret_cast<cudaStream_t>(32);
+  for (int leaf : {2, 4, 8})
+    for (int prec : {FMM_FP32, FMM_FP64})
+      for (int m2p : {0, 1}) {
+        Dry d(leaf * 12, leaf * 12, leaf * 12, 4, leaf, opts(prec, 1, m2p));
+        d.P->side = hi, d.P->side2 = lo;
+        const bool flat = leaf == 8 && !m2p;
+        expect(levels_stream(d.P, false) == (flat ? lo : hi), "levels' stream of a forward solve");
+        expect(levels_stream(d.P, true) == hi, "levels' stream of the transposed force");
+        for (int split : {1, 3}) {
+          d.P->near_choice.dsplit = split;
+          expect(near_behind(d.P, false) == (leaf == 8 && m2p && split > 1), "near field behind the final stage");
+          expect(!near_behind(d.P, true), "the transposed force's near field is unsplit");
+        }
+        d.P->side = d.P->side2 = nullptr;
+      }
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
   const std::string what = argc > 1 ? argv[1] : "";
   if (what == "direct_gemm") direct_gemm();
+  else if (what == "leaf8_streams") leaf8_streams();
   else expect(false, "unknown check");
   return failures ? 1 : 0;
 }

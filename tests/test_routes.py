@@ -29,7 +29,7 @@ def host_routes(tmp_path_factory):
     return exe
 
 
-CHECKS = ["direct_gemm"]
+CHECKS = ["direct_gemm", "leaf8_streams"]
 
 
 @pytest.mark.parametrize("check", CHECKS)
