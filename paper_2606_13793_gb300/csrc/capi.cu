@@ -3547,6 +3547,7 @@ struct MultiStep {
   int ny[3] = {0, 0, 0};  // the kind's common gy (column tiles), 0 if its items differ
   int nx[3] = {0, 0, 0};  // and gx (the tiny form's column tiles)
   long long kb[3] = {0, 0, 0};
+  bool wide = false;  // the direct z-run items in the wide form whatever their number
 };
 }  // namespace
 
@@ -3672,10 +3673,20 @@ void build_fused(fmm_batch_t B, const void* const* rho, void* const* phi, void* 
   // which the 5-point force amplifies (a change of it shows as 2.2e-5 to
   // 3.7e-5 of the force, against 5e-6 for the leaf level's): the force would
   // differ from earlier releases' by more than their FP32 solves of one field
-  // agree in.
+  // agree in.  FP32 fields of leaf 8 keep the direct form at the leaf level too:
+  // its blocks fill the gaps of the long direct near field, whose launch a
+  // second form would have to wait for (below).
   auto reflect = [&](fmm_plan_t P, int l) {
-    return P->lev[l].fold_off != 0 && !P->lev[l].tc && (P->f64_data() || l == P->L);
+    return P->lev[l].fold_off != 0 && !P->lev[l].tc && (P->f64_data() || (l == P->L && P->b != 8));
   };
+  // With leaf-8 fields every direct item goes in one wide z-run launch: the
+  // narrow form's four CTAs an SM leave no room for the tiny-grid blocks beside
+  // them, which then run alone (FP32, order 4, 40, 96, 64, 40, 96, 96, 32, 64:
+  // 3.33 ms wide with the leaf level's M2L direct, 4.18 ms narrow with it in the
+  // reflection basis; order 8, 56, 32, 88, 96, 88, 32, 48: 3.37 and 4.43 ms).
+  bool wide = false;
+  for (fmm_plan_t P : B->plans) wide |= P->b == 8;
+
   {  // P2M (and the near field's box-major density)
     std::vector<P2mArgs> a;
     std::vector<std::array<unsigned, 3>> g;
@@ -3758,6 +3769,7 @@ void build_fused(fmm_batch_t B, const void* const* rho, void* const* phi, void* 
       add_step(B, MK_GEMM, sh, 0, 0, all, ag);
       if (B->steps.size() == before) continue;
       MultiStep& st = B->steps.back();
+      st.wide = wide;
       for (int k = 0; k < 3; ++k)
         for (const std::array<unsigned, 3>& x : g[sh][k]) {
           const long long nb = (long long)x[0] * x[1] * x[2];
@@ -3895,7 +3907,7 @@ fmm_status run_fused(fmm_batch_t B, cudaStream_t s) {
           else if (st.shape == 3)
             e = launch_nbr_gemm_col_multi<T>(ds, dg, n, nb, ls);
           else
-            e = launch_nbr_gemm_zrun_multi<T>(zs, ds, dg, n, nb, ls, first, st.ny[2]);
+            e = launch_nbr_gemm_zrun_multi<T>(zs, ds, dg, n, nb, ls, first, st.ny[2], st.wide);
         }
         for (int k = 0; k < 2 && e == cudaSuccess; ++k) {  // reflection-basis items: M2L, near field
           e = launch_nbr_gemm_sym_multi<T>(zs, k == 0 ? kSymM2l : kSymNear4, gs, g, st.kn[k], st.kb[k],

@@ -181,10 +181,11 @@ cudaError_t launch_nbr_gemm_simt_multi(const NbrGemm* gs, const MultiGrid* grids
 template <typename T>
 cudaError_t launch_nbr_gemm_col_multi(const NbrGemm* gs, const MultiGrid* grids, int n, long long blocks,
                                       cudaStream_t s);
-// shape here: 0 / 1 as launch_nbr_gemm_zrun, 2 = a z run of 6 rows (FP32; 3 in FP64)
+// shape here: 0 / 1 as launch_nbr_gemm_zrun, 2 = a z run of 6 rows (FP32; 3 in FP64).
+// wide: never the narrow form (which launches under kZrunNarrowBlocks blocks take)
 template <typename T>
 cudaError_t launch_nbr_gemm_zrun_multi(int shape, const NbrGemm* gs, const MultiGrid* grids, int n, long long blocks,
-                                       cudaStream_t s, long long first = 0, int ny = 0);
+                                       cudaStream_t s, long long first = 0, int ny = 0, bool wide = false);
 template <typename T>
 void nbr_gemm_simt_col_grid(const NbrGemm& g, unsigned out[3]);
 // Grids of at most 64 rows (nbr_gemm_tiny_fits): one block per column tile

@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(kZrThreads) zrun_narrow_group_kernel(const __g
 
 template <typename T, int RZ>
 cudaError_t launch_rz_multi(const NbrGemm* gs, const MultiGrid* grids, int n, long long blocks, cudaStream_t s,
-                            long long first, int ny) {
+                            long long first, int ny, bool wide) {
   constexpr size_t smem = zrun_smem_bytes<T, RZ>();
   static bool attr = false;
   if (!attr) {
@@ -395,7 +395,7 @@ cudaError_t launch_rz_multi(const NbrGemm* gs, const MultiGrid* grids, int n, lo
   if (n <= 0 || blocks <= 0) return cudaSuccess;
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   if constexpr (sizeof(T) == 4 && RZ % 2 == 0) {
-    if (blocks < kZrunNarrowBlocks) {  // under two waves of four CTAs per SM
+    if (!wide && blocks < kZrunNarrowBlocks) {  // under two waves of four CTAs per SM
       zrun_narrow_multi_kernel<RZ><<<(unsigned)(4 * blocks), kZrThreads, 0, s>>>(gs, grids, n, first, ny);
       return cudaGetLastError();
     }
@@ -465,10 +465,10 @@ void nbr_gemm_zrun_grid(const NbrGemm& g, int shape, unsigned out[3]) {
 
 template <typename T>
 cudaError_t launch_nbr_gemm_zrun_multi(int shape, const NbrGemm* gs, const MultiGrid* grids, int n, long long blocks,
-                                       cudaStream_t s, long long first, int ny) {
-  return shape == 0   ? launch_rz_multi<T, zrun_rz<T>(0)>(gs, grids, n, blocks, s, first, ny)
-         : shape == 1 ? launch_rz_multi<T, zrun_rz<T>(1)>(gs, grids, n, blocks, s, first, ny)
-                      : launch_rz_multi<T, zrun_rz<T>(2)>(gs, grids, n, blocks, s, first, ny);
+                                       cudaStream_t s, long long first, int ny, bool wide) {
+  return shape == 0   ? launch_rz_multi<T, zrun_rz<T>(0)>(gs, grids, n, blocks, s, first, ny, wide)
+         : shape == 1 ? launch_rz_multi<T, zrun_rz<T>(1)>(gs, grids, n, blocks, s, first, ny, wide)
+                      : launch_rz_multi<T, zrun_rz<T>(2)>(gs, grids, n, blocks, s, first, ny, wide);
 }
 
 cudaError_t launch_nbr_gemm_zrun_group(const NbrGemm* gs, int n, cudaStream_t s) {
@@ -501,9 +501,9 @@ cudaError_t launch_nbr_gemm_zrun_group(const NbrGemm* gs, int n, cudaStream_t s)
 template void nbr_gemm_zrun_grid<float>(const NbrGemm&, int, unsigned[3]);
 template void nbr_gemm_zrun_grid<double>(const NbrGemm&, int, unsigned[3]);
 template cudaError_t launch_nbr_gemm_zrun_multi<float>(int, const NbrGemm*, const MultiGrid*, int, long long,
-                                                       cudaStream_t, long long, int);
+                                                       cudaStream_t, long long, int, bool);
 template cudaError_t launch_nbr_gemm_zrun_multi<double>(int, const NbrGemm*, const MultiGrid*, int, long long,
-                                                        cudaStream_t, long long, int);
+                                                        cudaStream_t, long long, int, bool);
 template cudaError_t launch_nbr_gemm_zrun<float>(const NbrGemm&, int, cudaStream_t);
 template cudaError_t launch_nbr_gemm_zrun<double>(const NbrGemm&, int, cudaStream_t);
 

@@ -63,12 +63,34 @@ void leaf8_streams() {
       }
 }
 
+// Fused FP32 batches: with leaf-8 fields one wide direct launch per tile shape
+// (their leaf level included); other leaves run it in the reflection basis.
+void leaf8_batch() {
+  for (std::array<int, 2> leaf : {std::array<int, 2>{4, 4}, {8, 8}, {4, 8}, {2, 2}}) {
+    Dry a(leaf[0] * 8, leaf[0] * 12, leaf[0] * 12, 4, leaf[0], opts(FMM_FP32, 1));
+    Dry b(leaf[1] * 12, leaf[1] * 10, leaf[1] * 24, 4, leaf[1], opts(FMM_FP32, 1));
+    fmm_batch_s B;
+    B.plans = {a.P, b.P};
+    build_fused<float>(&B, nullptr, nullptr, nullptr, true);
+    int sym = 0, gemm = 0;
+    for (const MultiStep& st : B.steps) {
+      if (st.kind != MK_GEMM) continue;
+      ++gemm;
+      sym += st.kn[0] + st.kn[1];
+      expect(st.wide == (leaf[0] == 8 || leaf[1] == 8), "wide form with leaf-8 fields");
+    }
+    const int want = (leaf[0] == 4 ? 2 : leaf[0] == 2 ? 1 : 0) + (leaf[1] == 4 ? 2 : leaf[1] == 2 ? 1 : 0);
+    expect(gemm > 0 && sym == want, "reflection-basis items (leaf level, near field of leaf 4)");
+  }
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
   const std::string what = argc > 1 ? argv[1] : "";
   if (what == "direct_gemm") direct_gemm();
   else if (what == "leaf8_streams") leaf8_streams();
+  else if (what == "leaf8_batch") leaf8_batch();
   else expect(false, "unknown check");
   return failures ? 1 : 0;
 }
