@@ -84,6 +84,34 @@ void leaf8_batch() {
   }
 }
 
+// The far field's launches go coarse to fine, groups at their coarsest level.
+void far_order() {
+  auto first = [](fmm_plan_t P, FarItem::Kind* kind) {
+    int ls[kMaxLevels], n = 0, seen = 0, last = 0;
+    for (int l = 2; l <= P->L; ++l)
+      if (!P->lev[l].tc && !(l == P->L && P->m2p)) ls[n++] = l;
+    const std::vector<FarItem> items = far_items(P, ls, n);
+    for (const FarItem& it : items) {
+      expect(it.ls[0] > last, "coarse to fine");
+      last = it.ls[0];
+      seen += (int)it.ls.size();
+    }
+    expect(seen == n, "every level once");
+    *kind = items[0].kind;
+    return items.size();
+  };
+  FarItem::Kind k;
+  // the levels of a mixed plan with FP64 coarse levels: two of those (one column
+  // per lane, split), then FP32 ones in a row group
+  Dry mixed(128, 128, 128, 0, 4, opts(FMM_FP32, 1));
+  for (int l : {2, 3}) mixed.P->lev[l].f64 = 1, mixed.P->m2l_choice[l].shape = 3;
+  for (int l = 2; l <= mixed.P->L; ++l) mixed.P->m2l_choice[l].dsplit = 27;
+  for (int l = 4; l <= mixed.P->L; ++l) mixed.P->m2l_choice[l].shape = 0;
+  expect(first(mixed.P, &k) == 3 && k == FarItem::kLevel, "FP64 levels ahead of the row group");
+  Dry fp32(64, 64, 64, 6, 4, opts(FMM_FP32, 1));
+  expect(first(fp32.P, &k) == 1 && k == FarItem::kRows, "levels of at most 512 rows in one group");
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
@@ -91,6 +119,7 @@ int main(int argc, char** argv) {
   if (what == "direct_gemm") direct_gemm();
   else if (what == "leaf8_streams") leaf8_streams();
   else if (what == "leaf8_batch") leaf8_batch();
+  else if (what == "far_order") far_order();
   else expect(false, "unknown check");
   return failures ? 1 : 0;
 }
