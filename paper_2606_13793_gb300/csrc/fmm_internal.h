@@ -19,6 +19,7 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstddef>
 #include <cstdint>
 
@@ -31,6 +32,25 @@ constexpr int kMaxCoef = 165;  // C(8+3, 3)
 constexpr int kMaxLevels = 24;
 constexpr int kNTile = 32;     // output columns per SIMT GEMM tile
 constexpr int kKChunk = 32;    // reduction values per SIMT GEMM stage
+
+// Raises a kernel's limit of dynamic shared memory, once per device: the limit
+// is the device's own, and a process may drive several.  One static object per
+// kernel; safe from several threads (a race sets the same value twice).
+class SmemOptIn {
+  std::atomic<unsigned long long> done_{0};  // bit: device ordinal (ordinals past 63 are set on every call)
+
+ public:
+  template <typename Kernel>
+  cudaError_t operator()(Kernel kernel, size_t bytes) {
+    int dev = 0;
+    if (cudaError_t e = cudaGetDevice(&dev)) return e;
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+    if (done_.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) done_.fetch_or(bit, std::memory_order_relaxed);
+    return e;
+  }
+};
 
 // Pair lists of the M2M / L2L shifts.  Entry: coefficient index `src`,
 // magnitude `coef`, and `mask`: bit q set when the shift exponent along

@@ -188,13 +188,8 @@ __global__ void __launch_bounds__(kRwRed) nbr_rows_reduce_kernel(const __grid_co
 
 cudaError_t launch_nbr_gemm_rows(const NbrGemm* gs, int n, cudaStream_t s) {
   if (n < 1 || n > kRowsGroupMax) return cudaErrorInvalidValue;
-  static bool attr = false;
-  if (!attr) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(nbr_gemm_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRwSmem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static SmemOptIn opt;
+  if (cudaError_t e = opt(nbr_gemm_rows_kernel, kRwSmem)) return e;
   RowsGroup G{};
   long long per_tile = 0;
   for (int i = 0; i < n; ++i) {

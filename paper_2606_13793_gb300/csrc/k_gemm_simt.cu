@@ -452,13 +452,8 @@ cudaError_t launch_nbr_gemm_tiny_multi(const NbrGemm* gs, const MultiGrid* grids
                                        cudaStream_t s, long long first, int nx) {
   if (n <= 0 || blocks <= 0) return cudaSuccess;
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  static bool attr = false;
-  if (!attr) {
-    const cudaError_t e = cudaFuncSetAttribute(nbr_gemm_tiny_multi_kernel<T>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTinySmem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static SmemOptIn opt;
+  if (cudaError_t e = opt(nbr_gemm_tiny_multi_kernel<T>, kTinySmem)) return e;
   nbr_gemm_tiny_multi_kernel<T><<<(unsigned)blocks, kTinyThreads, kTinySmem, s>>>(gs, grids, n, first, nx);
   return cudaGetLastError();
 }

@@ -385,13 +385,8 @@ template <typename T, int RZ>
 cudaError_t launch_rz_multi(const NbrGemm* gs, const MultiGrid* grids, int n, long long blocks, cudaStream_t s,
                             long long first, int ny, bool wide) {
   constexpr size_t smem = zrun_smem_bytes<T, RZ>();
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(nbr_gemm_zrun_multi_kernel<T, RZ>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static SmemOptIn opt;
+  if (cudaError_t e = opt(nbr_gemm_zrun_multi_kernel<T, RZ>, smem)) return e;
   if (n <= 0 || blocks <= 0) return cudaSuccess;
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   if constexpr (sizeof(T) == 4 && RZ % 2 == 0) {
@@ -407,13 +402,8 @@ cudaError_t launch_rz_multi(const NbrGemm* gs, const MultiGrid* grids, int n, lo
 template <typename T, int RZ>
 cudaError_t launch_rz(const NbrGemm& g, cudaStream_t s) {
   constexpr size_t smem = zrun_smem_bytes<T, RZ>();
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(nbr_gemm_zrun_kernel<T, RZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static SmemOptIn opt;
+  if (cudaError_t e = opt(nbr_gemm_zrun_kernel<T, RZ>, smem)) return e;
   const long long tiles = (long long)((g.grid[0] + kZrBX - 1) / kZrBX) * ((g.grid[1] + kZrBY - 1) / kZrBY) *
                           ((g.grid[2] + RZ - 1) / RZ);
   if (tiles <= 0 || g.ntiles <= 0) return cudaSuccess;

@@ -395,15 +395,9 @@ cudaError_t make_row_map(void* map_out, const void* base, int row_len, int elem_
 }
 
 cudaError_t launch_m2l_tc(const TcLaunch& L, const void* map_hi, const void* map_lo, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(m2l_tc_kernel<TC_BF16X3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kSmemBytes);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(m2l_tc_kernel<TC_TF32>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static SmemOptIn opt_bf16x3, opt_tf32;
+  if (cudaError_t e = opt_bf16x3(m2l_tc_kernel<TC_BF16X3>, kSmemBytes)) return e;
+  if (cudaError_t e = opt_tf32(m2l_tc_kernel<TC_TF32>, kSmemBytes)) return e;
   const int ntx = (L.grid[0] + kTcTileX - 1) / kTcTileX, nty = (L.grid[1] + kTcTileY - 1) / kTcTileY,
             ntz = (L.grid[2] + kTcTileZ - 1) / kTcTileZ;
   const int tiles = ntx * nty * ntz;

@@ -388,15 +388,9 @@ __global__ void __maxnreg__(96)
 }  // namespace
 
 cudaError_t launch_nbr_tc(const TpLaunch& L, const void* map_hi, const void* map_lo, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(nbr_tc_kernel<TC_BF16X3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kSmemBytes);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(nbr_tc_kernel<TC_TF32>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static SmemOptIn opt_bf16x3, opt_tf32;
+  if (cudaError_t e = opt_bf16x3(nbr_tc_kernel<TC_BF16X3>, kSmemBytes)) return e;
+  if (cudaError_t e = opt_tf32(nbr_tc_kernel<TC_TF32>, kSmemBytes)) return e;
   if (L.npass < 1 || L.npass > kTpMaxPasses || L.a_stages < 2 || L.a_stages > kTpMaxAStages || L.w_slots < 1 ||
       L.w_slots > kTpMaxSlots)
     return cudaErrorInvalidValue;

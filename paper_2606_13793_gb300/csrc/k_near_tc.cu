@@ -267,12 +267,8 @@ __global__ void __launch_bounds__(kNtThreads, 1)
 }  // namespace
 
 cudaError_t launch_near_tc4(const NearTcLaunch& L, const void* map_hi, const void* map_lo, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
-    const cudaError_t e = cudaFuncSetAttribute(near_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kNtSmem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static SmemOptIn opt;
+  if (cudaError_t e = opt(near_tc_kernel, kNtSmem)) return e;
   const int ntx = (L.grid[0] + kTcTileX - 1) / kTcTileX, nty = (L.grid[1] + kTcTileY - 1) / kTcTileY,
             ntz = (L.grid[2] + kTcTileZ - 1) / kTcTileZ;
   const long long items = ((long long)ntx * nty * ntz + kNtTiles - 1) / kNtTiles;

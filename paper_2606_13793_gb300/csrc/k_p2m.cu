@@ -342,13 +342,9 @@ cudaError_t p2m_multi_launch(const P2mArgs* args, const MultiGrid* grids, int n,
   constexpr size_t red = full + red0 <= 227 * 1024 ? red0 : 0;
   if (harm_rows && red == 0) return cudaErrorInvalidValue;
   const size_t smem = full + (harm_rows ? red : 0);
-  static bool attr = false;
-  if (!attr && full + red > 48 * 1024) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(p2m_multi_kernel<P, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(full + red));
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static SmemOptIn opt;
+  if (full + red > 48 * 1024)
+    if (cudaError_t e = opt(p2m_multi_kernel<P, T>, full + red)) return e;
   p2m_multi_kernel<P, T><<<(unsigned)blocks, kP2mThreads<T>, smem, s>>>(args, grids, n);
   return cudaGetLastError();
 }
@@ -358,13 +354,9 @@ cudaError_t p2m_launch_dip(unsigned blocks, size_t smem, size_t attr_bytes, cuda
                            int ny, int b, Level leaf, T* Mleaf, __nv_bfloat16* Mhi, __nv_bfloat16* Mlo, T* rho_box,
                            __nv_bfloat16* rhi, __nv_bfloat16* rlo, int* flag, int harm, T* Mfold, const T* dip,
                            long long ncell, int rho_soa) {
-  static bool attr = false;
-  if (!attr && attr_bytes > 48 * 1024) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(p2m_kernel<P, T, DIP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attr_bytes);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static SmemOptIn opt;
+  if (attr_bytes > 48 * 1024)
+    if (cudaError_t e = opt(p2m_kernel<P, T, DIP>, attr_bytes)) return e;
   p2m_kernel<P, T, DIP><<<blocks, kP2mThreads<T>, smem, s>>>(rho, nx, ny, b, leaf, Mleaf, Mhi, Mlo, rho_box, rhi, rlo, flag,
                                                        harm, Mfold, dip, ncell, rho_soa);
   return cudaGetLastError();

@@ -808,26 +808,18 @@ __global__ void __launch_bounds__(kSyThreads, 1)
   sym_near4_body<T, RZ>(g, multi_vblock_at(grids[i], b));
 }
 
-template <typename K>
-cudaError_t opt_in(K kernel, size_t smem, bool* done) {
-  if (*done) return cudaSuccess;
-  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess) *done = true;
-  return e;
-}
-
 template <typename T, int RZ>
 cudaError_t launch_zrun_form(const NbrGemm& g, cudaStream_t s) {
   const long long tiles = (long long)((g.grid[0] + 7) / 8) * ((g.grid[1] + 3) / 4) * ((g.grid[2] + RZ - 1) / RZ);
   if (tiles <= 0) return cudaSuccess;
   if (tiles > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   if (g.sym == kSymNear4) {
-    static bool done = false;
-    if (cudaError_t e = opt_in(sym_near4_kernel<T, RZ>, sym_near4_smem<T, RZ>(), &done)) return e;
+    static SmemOptIn opt;
+    if (cudaError_t e = opt(sym_near4_kernel<T, RZ>, sym_near4_smem<T, RZ>())) return e;
     sym_near4_kernel<T, RZ><<<dim3((unsigned)tiles, 1, (unsigned)g.dsplit), kSyThreads, sym_near4_smem<T, RZ>(), s>>>(g);
   } else {
-    static bool done = false;
-    if (cudaError_t e = opt_in(sym_m2l_kernel<T, RZ>, sym_m2l_smem<T, RZ>(), &done)) return e;
+    static SmemOptIn opt;
+    if (cudaError_t e = opt(sym_m2l_kernel<T, RZ>, sym_m2l_smem<T, RZ>())) return e;
     sym_m2l_kernel<T, RZ><<<dim3((unsigned)tiles, (unsigned)((g.n_cols / 8 + 7) / 8), (unsigned)g.dsplit), kSyThreads,
                             sym_m2l_smem<T, RZ>(), s>>>(g);
   }
@@ -836,8 +828,8 @@ cudaError_t launch_zrun_form(const NbrGemm& g, cudaStream_t s) {
 
 template <typename T, int RC, int P>
 cudaError_t launch_rows_form(const NbrGemm* gs, int n, cudaStream_t s) {
-  static bool done = false;
-  if (cudaError_t e = opt_in(sym_rows_kernel<T, RC, P>, 227 * 1024, &done)) return e;
+  static SmemOptIn opt;
+  if (cudaError_t e = opt(sym_rows_kernel<T, RC, P>, 227 * 1024)) return e;
   SymGroup G{};
   const int nk = gs[0].n_cols / 8, split = gs[0].dsplit;
   long long chunks = 0, blocks = 0;
@@ -873,12 +865,12 @@ template <typename T, int RZ>
 cudaError_t launch_multi_form(int kind, const NbrGemm* gs, const MultiGrid* grids, int n, long long blocks,
                               long long first, int ny, cudaStream_t s) {
   if (kind == kSymNear4) {
-    static bool done = false;
-    if (cudaError_t e = opt_in(sym_near4_multi_kernel<T, RZ>, sym_near4_smem<T, RZ>(), &done)) return e;
+    static SmemOptIn opt;
+    if (cudaError_t e = opt(sym_near4_multi_kernel<T, RZ>, sym_near4_smem<T, RZ>())) return e;
     sym_near4_multi_kernel<T, RZ><<<(unsigned)blocks, kSyThreads, sym_near4_smem<T, RZ>(), s>>>(gs, grids, n, first);
   } else {
-    static bool done = false;
-    if (cudaError_t e = opt_in(sym_m2l_multi_kernel<T, RZ>, sym_m2l_smem<T, RZ>(), &done)) return e;
+    static SmemOptIn opt;
+    if (cudaError_t e = opt(sym_m2l_multi_kernel<T, RZ>, sym_m2l_smem<T, RZ>())) return e;
     sym_m2l_multi_kernel<T, RZ><<<(unsigned)blocks, kSyThreads, sym_m2l_smem<T, RZ>(), s>>>(gs, grids, n, first, ny);
   }
   return cudaGetLastError();
@@ -923,8 +915,8 @@ cudaError_t launch_nbr_gemm_sym_multi(int shape, int kind, const NbrGemm* gs, co
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   if (shape == 3) {
     if (kind != kSymM2l) return cudaErrorInvalidValue;
-    static bool done = false;
-    if (cudaError_t e = opt_in(sym_tiny_multi_kernel<T>, sym_tiny_smem<T>(), &done)) return e;
+    static SmemOptIn opt;
+    if (cudaError_t e = opt(sym_tiny_multi_kernel<T>, sym_tiny_smem<T>())) return e;
     sym_tiny_multi_kernel<T><<<(unsigned)blocks, kSyTinyThreads, sym_tiny_smem<T>(), s>>>(gs, grids, n, first);
     return cudaGetLastError();
   }

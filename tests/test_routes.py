@@ -36,3 +36,20 @@ CHECKS = ["direct_gemm", "leaf8_streams", "leaf8_batch", "far_order"]
 def test_route(host_routes, check):
     r = subprocess.run([host_routes, check], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+def test_shared_memory_limits_are_raised_on_every_device(tmp_path):
+    """Kernels of more than 48 KB: the limit is per device (SmemOptIn), and no
+    launch sets it in any other way."""
+    for name in os.listdir(_build.CSRC):
+        text = open(os.path.join(_build.CSRC, name)).read()
+        assert text.count("cudaFuncSetAttribute(") == (1 if name == "fmm_internal.h" else 0), name
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not available")
+    exe = str(tmp_path / "host_smem")
+    r = subprocess.run([nvcc, *_build.ARCH, "-std=c++17", "-I", _build.CSRC,
+                        os.path.join(ROOT, "tests", "host_smem.cu"), "-o", exe], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
+    r = subprocess.run([exe], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
