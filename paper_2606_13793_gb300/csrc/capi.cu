@@ -1939,12 +1939,12 @@ fmm_status plan_init(fmm_plan_t P, const int d3[3], double dx, double G, int ord
       if (P->lev[l].rfold_off) want = std::max(want, 9 * one);
     }
     // room for the autotuner's neighbour-split candidates (M2L levels and the
-    // near field), up to 64 MiB each
+    // near field), up to 64 MiB each or what a split M2L level needs
+    if (!P->no_split) part = std::max(part, std::min(want, (size_t)64 << 20));
     if (!P->near_tc && !P->no_split)
       P->near_part_cap = std::min((size_t)27 * (size_t)P->lev[P->L].nbox * (size_t)(P->b * P->b * P->b) *
                                       (size_t)P->near_comps * P->esize(),
-                                  (size_t)64 << 20);
-    if (!P->no_split) part = std::max(part, std::min(want, (size_t)64 << 20));
+                                  std::max(part, (size_t)64 << 20));
     P->part_off = off;
     P->part_cap = part;
     off = align(off + part);

@@ -112,6 +112,25 @@ void far_order() {
   expect(first(fp32.P, &k) == 1 && k == FarItem::kRows, "levels of at most 512 rows in one group");
 }
 
+// The near field's own scratch takes every split that the M2L's, which it used
+// to share, held: 64 MiB or what a split M2L level needs.
+void near_scratch() {
+  struct {
+    int n[3], order, precision;
+  } cases[] = {{{96, 96, 64}, 6, FMM_FP64}, {{96, 96, 64}, 7, FMM_FP64}, {{64, 64, 64}, 6, FMM_FP64},
+               {{96, 112, 128}, 4, FMM_FP32}, {{32, 40, 24}, 3, FMM_FP32}};
+  for (const auto& c : cases) {
+    Dry d(c.n[0], c.n[1], c.n[2], c.order, 4, opts(c.precision, 1));
+    const size_t es = d.P->esize(), one = (size_t)d.P->ncell() * es;
+    const NbrGemm g = near_gemm(d.P);
+    for (int split : {27, 9, 3})
+      if (split * one <= std::max(d.P->part_cap, (size_t)64 << 20))
+        expect(choice_valid(d.P, g, d.P->h_near_tile_k, es, {split == 27 ? 0 : 1, split}), "a near-field split that fits");
+    expect(d.P->near_part_off >= d.P->part_off + d.P->part_cap &&
+               d.P->near_part_off + d.P->near_part_cap <= d.P->arena_bytes, "scratch of its own, inside the arena");
+  }
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
@@ -120,6 +139,7 @@ int main(int argc, char** argv) {
   else if (what == "leaf8_streams") leaf8_streams();
   else if (what == "leaf8_batch") leaf8_batch();
   else if (what == "far_order") far_order();
+  else if (what == "near_scratch") near_scratch();
   else expect(false, "unknown check");
   return failures ? 1 : 0;
 }

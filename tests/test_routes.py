@@ -29,7 +29,7 @@ def host_routes(tmp_path_factory):
     return exe
 
 
-CHECKS = ["direct_gemm", "leaf8_streams", "leaf8_batch", "far_order"]
+CHECKS = ["direct_gemm", "leaf8_streams", "leaf8_batch", "far_order", "near_scratch"]
 
 
 @pytest.mark.parametrize("check", CHECKS)
