@@ -304,7 +304,8 @@ fmm_status fmm_solve_static(const fmm_grid* grid, int order, int leaf, const voi
  *                         (the same operator, an eighth of the products)
  *                         with the same row tiles.
  *   fmm_plan_set_tuning : sets it; FMM_ERR_ARG if the variant does not apply
- *                         (level on the tensor cores, reduction lengths not a
+ *                         (level of a tensor-core precision that is or could
+ *                         be on the tensor cores, reduction lengths not a
  *                         multiple of 8, split scratch too small).
  * All variants compute the same sums; they differ in summation order only
  * through the neighbour split (partials added in a fixed order).
@@ -339,7 +340,8 @@ fmm_status fmm_plan_autotune(fmm_plan_t plan, void* stream);
  * rows each) do not fill the GPU run, in plans without the stencil force
  * (accel 0 or 2), in FP32 on the CUDA cores instead (sums
  * and differences over mirror pairs, 8 times fewer products), where that is
- * the faster one; selecting a schedule puts every such level on it.
+ * the faster one (fmm_plan_level_kind tells); selecting a schedule puts every
+ * such level on it for the rest of the plan's life.
  * The paper has no counterpart.
  */
 fmm_status fmm_plan_tc_schedule(fmm_plan_t plan, int what, int* prefix, int* available);
@@ -462,10 +464,10 @@ fmm_status fmm_debug_level(fmm_plan_t plan, int what, int level, double* host_ou
 /* Number of FMM levels minus one (index of the leaf level), or -1. */
 int fmm_plan_leaf_level(fmm_plan_t plan);
 
-/* How the M2L of one level runs: 0 none (levels 0, 1), 1 CUDA cores FP32,
- * 2 CUDA cores FP64, 3 tcgen05 tensor cores (a level too small to fill them
- * may run FP32 all the same, see fmm_plan_tc_schedule); -1 for a bad plan or
- * level. */
+/* How the M2L of one level runs: 0 none (levels 0, 1), 1 CUDA cores FP32
+ * (levels of a tensor-core precision too small for them too, see
+ * fmm_plan_tc_schedule), 2 CUDA cores FP64, 3 tcgen05 tensor cores; -1 for a
+ * bad plan or level. */
 int fmm_plan_level_kind(fmm_plan_t plan, int level);
 
 /* 1 when the near field runs on the tensor cores (bf16x3), else 0. */

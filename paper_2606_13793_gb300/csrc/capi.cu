@@ -272,6 +272,7 @@ struct fmm_plan_s {
   // until an M2L schedule is selected; refl_now: in the current (last) solve
   bool use_refl = true, refl_now = true;
   bool refl_on(int l) const { return lev[l].rfold_off != 0 && refl_now; }
+  bool on_tensor_cores(int l) const { return lev[l].tc && !(lev[l].rfold_off && use_refl); }
   // the dedicated near-field kernel of leaf 4 (k_near_tc.cu), used when
   // present unless another schedule is selected
   bool near4 = false, use_near4 = true;
@@ -3318,7 +3319,7 @@ int fmm_plan_level_kind(fmm_plan_t P, int level) {
   if (!P || level < 0 || level > P->L) return -1;
   if (level < 2) return 0;
   const Level& lv = P->lev[level];
-  return lv.tc ? 3 : (lv.f64 ? 2 : 1);
+  return P->on_tensor_cores(level) ? 3 : (lv.f64 ? 2 : 1);
 }
 
 int fmm_plan_near_on_tensor_cores(fmm_plan_t P) { return (P && P->near_tc) ? 1 : 0; }
@@ -4415,7 +4416,7 @@ fmm_status tuning_slot(fmm_plan_t P, int level, SimtChoice** c, NbrGemm* g, cons
     return FMM_OK;
   }
   if (level < 2 || level > P->L) return fail(FMM_ERR_ARG, "level %d outside 2..%d", level, P->L);
-  if (P->lev[level].tc) return fail(FMM_ERR_ARG, "level %d runs on the tensor cores", level);
+  if (P->on_tensor_cores(level)) return fail(FMM_ERR_ARG, "level %d runs on the tensor cores", level);
   *c = &P->m2l_choice[level];
   *g = m2l_gemm(P, level);
   *tk = &P->h_m2l_tile_k;
@@ -4441,6 +4442,8 @@ extern "C" fmm_status fmm_plan_set_tuning(fmm_plan_t P, int level, int shape, in
   const std::vector<int>* tk;
   size_t es;
   if (fmm_status st = tuning_slot(P, level, &c, &g, &tk, &es)) return st;
+  if (level >= 0 && P->lev[level].tc)  // on the CUDA cores by its size: the variant is fixed
+    return fail(FMM_ERR_ARG, "the variant of level %d is not selectable", level);
   const SimtChoice want{shape, dsplit};
   if (!choice_valid(P, g, *tk, es, want))
     return fail(FMM_ERR_ARG, "variant shape %d / split %d does not apply to this contraction (or its split scratch "

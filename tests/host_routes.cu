@@ -131,6 +131,25 @@ void near_scratch() {
   }
 }
 
+// A level of a tensor-core precision that runs on the CUDA cores says so, and
+// its variant can be read but not set.
+void level_kind() {
+  Dry d(64, 64, 64, 4, 4, opts(FMM_FP32, 0));
+  Level& lv = d.P->lev[d.P->L];
+  lv.tc = 1;
+  lv.rfold_off = lv.fold_off, lv.rred_off = lv.lred_off;
+  lv.fold_off = lv.lred_off = 0;
+  int shape = -1, split = -1;
+  expect(fmm_plan_level_kind(d.P, d.P->L) == 1, "kind of a small bf16x3 level: FP32 on the CUDA cores");
+  expect(fmm_plan_tuning(d.P, d.P->L, &shape, &split) == FMM_OK && shape == d.P->m2l_choice[d.P->L].shape,
+         "its variant reads");
+  expect(fmm_plan_set_tuning(d.P, d.P->L, 1, 1) == FMM_ERR_ARG, "and stays as it is");
+  d.P->use_refl = false;
+  expect(fmm_plan_level_kind(d.P, d.P->L) == 3, "with a schedule selected: the tensor cores");
+  expect(fmm_plan_tuning(d.P, d.P->L, &shape, &split) == FMM_ERR_ARG, "which have no variant");
+  expect(fmm_plan_level_kind(d.P, 2) == 1, "an FP32 level");
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
@@ -140,6 +159,7 @@ int main(int argc, char** argv) {
   else if (what == "leaf8_batch") leaf8_batch();
   else if (what == "far_order") far_order();
   else if (what == "near_scratch") near_scratch();
+  else if (what == "level_kind") level_kind();
   else expect(false, "unknown check");
   return failures ? 1 : 0;
 }

@@ -29,7 +29,7 @@ def host_routes(tmp_path_factory):
     return exe
 
 
-CHECKS = ["direct_gemm", "leaf8_streams", "leaf8_batch", "far_order", "near_scratch"]
+CHECKS = ["direct_gemm", "leaf8_streams", "leaf8_batch", "far_order", "near_scratch", "level_kind"]
 
 
 @pytest.mark.parametrize("check", CHECKS)
