@@ -427,13 +427,14 @@ size_t fmm_workspace_bytes(fmm_plan_t plan);
 int fmm_solve_launches(fmm_plan_t plan, int with_accel);
 
 /*
- * Per-stage timing with CUDA events recorded on the solve's own stream around
- * every kernel launch (for benchmarks; off by default).
+ * Per-stage timing with CUDA events recorded around every kernel launch on its
+ * stream (for benchmarks; off by default).  While it is on, levels that
+ * otherwise run beside one another follow one another, so that no two launches
+ * of a stage overlap; the levels' stream still runs beside the caller's.
  *   fmm_timing_enable : 1 starts recording (and clears totals), 0 stops.
  *                       Creates its event pool here, not during solves.
  *   fmm_timing_read   : synchronises, then writes for each stage i < nstages
- *                       the milliseconds ms[i] covered by its launches (those
- *                       that run side by side count once) and the launch count
+ *                       the summed milliseconds ms[i] and launch count
  *                       launches[i] since the last enable/read, and clears them.
  * Stages (index: name): see fmm_timing_stage_name().  Errors: FMM_ERR_ARG
  * (NULL plan or arrays), FMM_ERR_CUDA (event creation or timing failure).

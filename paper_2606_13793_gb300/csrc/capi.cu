@@ -2924,6 +2924,11 @@ std::vector<FarItem> far_items(fmm_plan_t P, const int* ls, int n) {
 cudaStream_t levels_stream(fmm_plan_t P, bool adj_g) {
   return !P->near_tc && P->b == 8 && !P->m2p && !adj_g ? P->side2 : P->side;
 }
+// Whether levels may run beside one another on `side2`: not while stages are
+// timed, whose launches then follow one another on one stream each, so that a
+// stage's time is its own launches' (512^3: 6.25 ms a solve so, 6.03 ms side by
+// side, where the tensor-core levels' spans held the near field's 1.1 ms).
+bool second_stream(fmm_plan_t P) { return P->side2 && !P->timing; }
 // Whether the near field runs on the levels' stream, after the final stage: a
 // split leaf-8 one, whose blocks and the direct M2P's (as long) only hold each
 // other up (FP64, 56 x 48 x 40, order 6: 29.9 ms so, 42.1 ms side by side).
@@ -3012,7 +3017,7 @@ fmm_status run_solve(fmm_plan_t P, const T* rho, T* phi, T* accel, cudaStream_t 
     if (!cc && tc_first < 0) tc_first = l;
     any2 |= cc ? !(l == L && P->m2p) && level2(l) : l != tc_first;
   }
-  const bool fork = P->side && any_simt, fork2 = P->side2 && any2;
+  const bool fork = P->side && any_simt, fork2 = any2 && second_stream(P);
   cudaStream_t sf = fork ? levels_stream(P, adj_g != nullptr) : s, s2 = fork2 ? P->side2 : s;
   if (fork || fork2) CUDA_TRY(cudaEventRecord(P->ev_fork, s));
   if (fork) CUDA_TRY(cudaStreamWaitEvent(sf, P->ev_fork, 0));
@@ -3383,31 +3388,14 @@ fmm_status fmm_timing_read(fmm_plan_t P, double* ms, int* launches, int nstages)
   if (!ms || !launches || nstages <= 0) return fail(FMM_ERR_ARG, "bad output arrays");
   CUDA_TRY(cudaDeviceSynchronize());
   for (int i = 0; i < nstages; ++i) ms[i] = 0.0, launches[i] = 0;
-  // Launches of a stage on two streams may overlap: the union of their spans.
-  // A span is kept from the first event of a run of overlapping launches.
-  struct Span {
-    cudaEvent_t from = nullptr;
-    float lo = 0.f, hi = 0.f;  // against `from`
-  };
-  std::vector<Span> open((size_t)nstages);
   for (const auto& r : P->recs) {
-    if (r.stage >= nstages) continue;
-    Span& sp = open[(size_t)r.stage];
-    launches[r.stage] += 1;
-    float a = 0.f, b = 0.f;
-    if (sp.from) {
-      CUDA_TRY(cudaEventElapsedTime(&a, sp.from, r.a));
-      CUDA_TRY(cudaEventElapsedTime(&b, sp.from, r.b));
-      if (a <= sp.hi && b >= sp.lo) {
-        sp.lo = std::min(sp.lo, a), sp.hi = std::max(sp.hi, b);
-        continue;
-      }
-      ms[r.stage] += sp.hi - sp.lo;
+    float t = 0.f;
+    CUDA_TRY(cudaEventElapsedTime(&t, r.a, r.b));
+    if (r.stage < nstages) {
+      ms[r.stage] += t;
+      launches[r.stage] += 1;
     }
-    sp.from = r.a, sp.lo = 0.f;
-    CUDA_TRY(cudaEventElapsedTime(&sp.hi, r.a, r.b));
   }
-  for (int i = 0; i < nstages; ++i) ms[i] += open[(size_t)i].hi - open[(size_t)i].lo;
   P->recs.clear();
   P->ev_used = 0;
   return FMM_OK;
