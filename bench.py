@@ -147,16 +147,18 @@ def mirror_products(leaf, fp64, harmonic, variant, near=False, accel_columns=Fal
 
 
 def batch_products(sizes, leaf, p, fp64):
-    """Flops of one fused batch step's contractions as multiplied: the leaf
-    level (every level in FP64) and the near field of leaf 4 an eighth of the
-    pairwise products, the other FP32 levels all of them."""
+    """Flops of one fused batch step's contractions as multiplied: an eighth of
+    the pairwise products where they run in the reflection basis (FP64: every
+    level; FP32: the leaf level, of leaf 2 and 4; near fields of leaf 4 of more
+    than 64 boxes), all of them elsewhere."""
     total = 0
     for s in sizes:
         lev = hierarchy((s, s, s), leaf)
         for l in range(2, len(lev)):
-            total += m2l_flop_level((s, s, s), leaf, p, l, p >= 2) * \
-                mirror_products(leaf, fp64, p >= 2, (1, 1) if l == len(lev) - 1 else (0, 1))
-        total += algorithmic_counts((s, s, s), leaf, p)["near_flop"] * mirror_products(leaf, fp64, False, (1, 1), near=True)
+            mirror = p >= 2 and (fp64 or (l == len(lev) - 1 and leaf != 8))
+            total += m2l_flop_level((s, s, s), leaf, p, l, p >= 2) * (1 / 8 if mirror else 1)
+        mirror = leaf == 4 and math.prod(lev[-1]) > 64
+        total += algorithmic_counts((s, s, s), leaf, p)["near_flop"] * (1 / 8 if mirror else 1)
     return total
 
 

@@ -150,6 +150,33 @@ void level_kind() {
   expect(fmm_plan_level_kind(d.P, 2) == 1, "an FP32 level");
 }
 
+// Prints 1 or 0 per contraction of a one-field fused batch, levels 2 to the
+// leaf level and the near field: reflection basis or direct.
+void batch_forms(int n, int order, int leaf, bool f64) {
+  Dry d(n, n, n, order, leaf, opts(f64 ? FMM_FP64 : FMM_FP32, 1));
+  fmm_batch_s B;
+  B.plans = {d.P};
+  if (f64)
+    build_fused<double>(&B, nullptr, nullptr, nullptr, false);
+  else
+    build_fused<float>(&B, nullptr, nullptr, nullptr, false);
+  std::vector<int> form(d.P->L, -1);  // level l at l - 2, the near field last
+  for (const MultiStep& st : B.steps) {
+    if (st.kind != MK_GEMM) continue;
+    const NbrGemm* g = reinterpret_cast<const NbrGemm*>(B.h_tab.data() + st.args_off);
+    for (int i = 0; i < st.n; ++i) {
+      const bool near = !g[i].skip_center;
+      int l = d.P->L;
+      while (!near && (long long)g[i].grid[0] * g[i].grid[1] * g[i].grid[2] != d.P->lev[l].npar) --l;
+      form[near ? d.P->L - 1 : l - 2] = i < st.kn[0] + st.kn[1];
+    }
+  }
+  for (int v : form) {
+    expect(v >= 0, "every contraction once");
+    std::printf("%d ", v);
+  }
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
@@ -160,6 +187,7 @@ int main(int argc, char** argv) {
   else if (what == "far_order") far_order();
   else if (what == "near_scratch") near_scratch();
   else if (what == "level_kind") level_kind();
+  else if (what == "batch_forms" && argc == 6) batch_forms(atoi(argv[2]), atoi(argv[3]), atoi(argv[4]), atoi(argv[5]) != 0);
   else expect(false, "unknown check");
   return failures ? 1 : 0;
 }
