@@ -2847,68 +2847,68 @@ size_t rows_partial(fmm_plan_t P, int l) {
   const Level& lv = P->lev[l];
   return ((size_t)27 * lv.npar * 8 * (lv.fold_off ? P->nr : P->nc) * (lv.f64 ? 8 : 4) + 255) & ~(size_t)255;
 }
-std::vector<std::vector<int>> row_groups(fmm_plan_t P, const int* ls, int n) {
-  std::vector<std::vector<int>> out;
-  for (int shape : {0, 3}) {
-    size_t used = 0;
-    bool open = false;
-    for (int i = 0; i < n; ++i) {
-      const int l = ls[i];
-      if (!rows_level(P, l) || P->m2l_choice[l].shape != shape) continue;
-      const size_t need = rows_partial(P, l);
-      if (!open || used + need > P->part_cap || (int)out.back().size() == std::min(kSymGroupMax, kRowsGroupMax) ||
-          P->lev[l].f64 != P->lev[out.back()[0]].f64 || sym_level(P, l) != sym_level(P, out.back()[0])) {
-        out.emplace_back();
-        open = true;
-        used = 0;
-      }
-      out.back().push_back(l);
-      used += need;
-    }
-  }
-  return out;
-}
-fmm_status do_m2l_rows(fmm_plan_t P, const std::vector<int>& ls, cudaStream_t s) {
-  NbrGemm g[std::max(kSymGroupMax, kRowsGroupMax)];
-  size_t used = 0;
-  for (size_t i = 0; i < ls.size(); ++i) {
-    g[i] = m2l_gemm(P, ls[i]);
-    g[i].partial = P->arena + P->part_off + used;
-    used += rows_partial(P, ls[i]);
-  }
-  CUDA_TRY(g[0].sym ? launch_nbr_gemm_sym_rows(g, (int)ls.size(), s)
-                    : launch_nbr_gemm_rows(g, (int)ls.size(), s));
-  return FMM_OK;
-}
-
 // The launches of the CUDA-core levels ls[0 .. n) (coarse to fine) on one
 // stream: a level by itself, a row group, the narrow group; coarse to fine, a
 // group at its coarsest level.  Where FP64 coarse levels come first, their
 // kernels (no shared memory) then run beside a tensor-core near field, which row
 // groups wait out (bf16x3 order 0 with M2P, 140 x 164 x 96: 0.403 ms so, 0.442 ms
-// with the groups first).
+// with the groups first).  No host allocation: solves call it.
+constexpr int kFarGroup = std::min({kSymGroupMax, kRowsGroupMax, kZrunGroupMax});
 struct FarItem {
   enum Kind { kLevel, kRows, kNarrow } kind;
-  std::vector<int> ls;
+  int n, ls[kFarGroup];
 };
-std::vector<FarItem> far_items(fmm_plan_t P, const int* ls, int n) {
-  std::vector<FarItem> out;
-  const std::vector<std::vector<int>> groups = row_groups(P, ls, n);
-  std::vector<int> narrow;
-  for (int i = 0; i < n && (int)narrow.size() < kZrunGroupMax; ++i)
-    if (narrow_level(P, ls[i])) narrow.push_back(ls[i]);
+int far_items(fmm_plan_t P, const int* ls, int n, FarItem (&out)[kMaxLevels]) {
+  int items = 0;
+  FarItem* rows[2] = {nullptr, nullptr};  // the open row group of shape 0 and 3
+  FarItem* narrow = nullptr;
+  size_t used[2] = {0, 0};
+  auto add = [&](FarItem::Kind kind, int l) {
+    FarItem& it = out[items++];
+    it.kind = kind;
+    it.n = 1;
+    it.ls[0] = l;
+    return &it;
+  };
   for (int i = 0; i < n; ++i) {
     const int l = ls[i];
     if (rows_level(P, l)) {
-      for (const std::vector<int>& gr : groups)
-        if (gr[0] == l) out.push_back({FarItem::kRows, gr});
-    } else if (std::find(narrow.begin(), narrow.end(), l) != narrow.end()) {
-      if (narrow[0] == l) out.push_back({FarItem::kNarrow, narrow});
+      const int s = P->m2l_choice[l].shape == 3;
+      const size_t need = rows_partial(P, l);
+      FarItem* g = rows[s];
+      if (!g || used[s] + need > P->part_cap || g->n == kFarGroup || P->lev[l].f64 != P->lev[g->ls[0]].f64 ||
+          sym_level(P, l) != sym_level(P, g->ls[0])) {
+        rows[s] = add(FarItem::kRows, l);
+        used[s] = need;
+      } else {
+        g->ls[g->n++] = l;
+        used[s] += need;
+      }
+    } else if (narrow_level(P, l) && (!narrow || narrow->n < kFarGroup)) {
+      if (narrow)
+        narrow->ls[narrow->n++] = l;
+      else
+        narrow = add(FarItem::kNarrow, l);
     } else {
-      out.push_back({FarItem::kLevel, {l}});
+      add(FarItem::kLevel, l);
     }
   }
-  return out;
+  return items;
+}
+fmm_status do_far_item(fmm_plan_t P, const FarItem& it, cudaStream_t s) {
+  if (it.kind == FarItem::kLevel) return do_m2l(P, it.ls[0], s);
+  NbrGemm g[kFarGroup];
+  size_t used = 0;
+  for (int i = 0; i < it.n; ++i) {
+    g[i] = m2l_gemm(P, it.ls[i]);
+    if (it.kind == FarItem::kNarrow) continue;
+    g[i].partial = P->arena + P->part_off + used;
+    used += rows_partial(P, it.ls[i]);
+  }
+  CUDA_TRY(it.kind == FarItem::kNarrow ? launch_nbr_gemm_zrun_group(g, it.n, s)
+           : g[0].sym                  ? launch_nbr_gemm_sym_rows(g, it.n, s)
+                                       : launch_nbr_gemm_rows(g, it.n, s));
+  return FMM_OK;
 }
 
 // Stream of the CUDA-core levels beside the near field (and of the final
@@ -3026,20 +3026,11 @@ fmm_status run_solve(fmm_plan_t P, const T* rho, T* phi, T* accel, cudaStream_t 
     int ls[kMaxLevels], n = 0;
     for (int l = 2; l <= L; ++l)
       if ((!P->lev[l].tc || P->refl_on(l)) && !(p2l && l == L) && !(l == L && P->m2p)) ls[n++] = l;
-    for (const FarItem& it : far_items(P, ls, n)) {
-      if (it.kind == FarItem::kLevel && fork2 && level2(it.ls[0])) continue;
+    FarItem items[kMaxLevels];
+    for (int i = 0, m = far_items(P, ls, n, items); i < m; ++i) {
+      if (items[i].kind == FarItem::kLevel && fork2 && level2(items[i].ls[0])) continue;
       StageTimer t(P, ST_M2L, sf);
-      if (it.kind == FarItem::kRows) {
-        st = do_m2l_rows(P, it.ls, sf);
-      } else if (it.kind == FarItem::kNarrow) {
-        NbrGemm ng[kZrunGroupMax];
-        for (size_t i = 0; i < it.ls.size(); ++i) ng[i] = m2l_gemm(P, it.ls[i]);
-        CUDA_TRY(launch_nbr_gemm_zrun_group(ng, (int)it.ls.size(), sf));
-        st = FMM_OK;
-      } else {
-        st = do_m2l(P, it.ls[0], sf);
-      }
-      if (st) return st;
+      if ((st = do_far_item(P, items[i], sf))) return st;
     }
     for (int i = n - 1; fork2 && i >= 0; --i) {
       if (!level2(ls[i])) continue;
@@ -3338,20 +3329,17 @@ int fmm_solve_launches(fmm_plan_t P, int with_accel) {
   if (L < 2) n += 1;                    // zero the leaf locals
   for (int l = 2; l <= L; ++l) {
     n += l >= 3 ? 2 : 1;                // M2L, and L2L below level 2
-    if (rows_level(P, l) && !(l == L && P->m2p)) n -= 2;  // grouped: counted below (M2L and its reduction)
     if (l == 2 && harmonic_m2l_level(P, 2)) n += 1;  // rebuild of the harmonic level-2 locals
     if (l == 2 && L == 2 && P->m2p) n += 1;          // zero leaf locals (final-stage M2P, no parent far field)
     if ((!P->lev[l].tc || P->refl_on(l)) && P->m2l_choice[l].dsplit > 1 && !(l == L && P->m2p)) n += 1;  // partial-sum reduction
   }
-  {
-    int ls[kMaxLevels], k = 0, nn = 0;
+  {  // one launch, and one reduction of row groups, for the levels of a group
+    int ls[kMaxLevels], k = 0;
     for (int l = 2; l <= L; ++l)
-      if (!P->lev[l].tc && !(l == L && P->m2p)) {
-        ls[k++] = l;
-        nn += narrow_level(P, l);
-      }
-    n += 2 * (int)row_groups(P, ls, k).size();
-    n -= std::max(0, std::min(nn, kZrunGroupMax) - 1);  // one launch for the narrow levels
+      if (!P->lev[l].tc && !(l == L && P->m2p)) ls[k++] = l;
+    FarItem items[kMaxLevels];
+    for (int i = 0, m = far_items(P, ls, k, items); i < m; ++i)
+      n -= (items[i].kind == FarItem::kRows ? 2 : 1) * (items[i].n - 1);
   }
   n += P->near_tc ? ((P->near4 && P->use_near4) || tc_prefix(P, TS_NEAR) ? 1 : (int)P->tcn.size()) + 1
                    : 2;  // near field + leaf finish

@@ -2,6 +2,17 @@
 // plans (no GPU): one check per name on the command line.
 #include "capi.cu"
 
+// Host allocations, counted.
+static size_t allocations = 0;
+void* operator new(size_t n) {
+#ifndef __CUDA_ARCH__
+  ++allocations;
+#endif
+  return malloc(n ? n : 1);
+}
+void operator delete(void* p) noexcept { free(p); }
+void operator delete(void* p, size_t) noexcept { free(p); }
+
 namespace {
 
 int failures = 0;
@@ -90,15 +101,19 @@ void far_order() {
     int ls[kMaxLevels], n = 0, seen = 0, last = 0;
     for (int l = 2; l <= P->L; ++l)
       if (!P->lev[l].tc && !(l == P->L && P->m2p)) ls[n++] = l;
-    const std::vector<FarItem> items = far_items(P, ls, n);
-    for (const FarItem& it : items) {
-      expect(it.ls[0] > last, "coarse to fine");
-      last = it.ls[0];
-      seen += (int)it.ls.size();
+    FarItem items[kMaxLevels];
+    const size_t before = allocations;
+    const int m = far_items(P, ls, n, items);
+    (void)fmm_solve_launches(P, 1);
+    expect(allocations == before, "no host allocation (an exception would cross the C interface)");
+    for (int i = 0; i < m; ++i) {
+      expect(items[i].ls[0] > last, "coarse to fine");
+      last = items[i].ls[0];
+      seen += items[i].n;
     }
     expect(seen == n, "every level once");
     *kind = items[0].kind;
-    return items.size();
+    return m;
   };
   FarItem::Kind k;
   // the levels of a mixed plan with FP64 coarse levels: two of those (one column
