@@ -315,8 +315,8 @@ struct fmm_plan_s {
   void* Lx(int l) const { return arena + lev[l].l_off; }
 
   // Device placement: cudaMalloc (plans) or a bump pointer inside a caller
-  // supplied region (the allocation-free solve), where the tables can be
-  // left as the previous call wrote them.
+  // supplied region (the allocation-free solve).  static_keep_tables: sizes
+  // only, no table is filled or uploaded.
   unsigned char* static_base = nullptr;
   size_t static_cap = 0, static_used = 0;
   bool static_keep_tables = false;
@@ -3741,7 +3741,6 @@ void build_fused(fmm_batch_t B, const void* const* rho, void* const* phi, void* 
     auto add = [&](NbrGemm x, const std::vector<int>& tile_k) {
       x.dsplit = 1;  // the batch fills the GPU: no neighbour split, no partial sums
       x.partial = nullptr;
-      x.max_blocks = 0;
       x.shape = batch_shape(x, tile_k, sizeof(T) == 4);
       std::array<unsigned, 3> gr;
       if (x.shape == 4)

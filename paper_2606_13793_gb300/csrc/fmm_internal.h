@@ -134,11 +134,10 @@ struct DirectGemm {
   void* partial;       // [dsplit][rows][n_cols] scratch when dsplit > 1
   int shape = 0;       // 0: 4x4x4 rows per CTA, 3: one column per lane (k_gemm_simt.cu);
                        // 1, 2: z-run tiles (k_gemm_zrun.cu)
-  int max_blocks = 0;  // shape 0: at most this many CTAs, each looping over work items (0: one per item)
   int skip_center = 0; // 1: W_d of the centre neighbour (d = 13) is all zero (the M2L: a parent's
                        // children are each other's near neighbours), and the kernels skip it
 };
-static_assert(sizeof(DirectGemm) == 96, "the fields of the direct form only");
+static_assert(sizeof(DirectGemm) == 88, "the fields of the direct form only");
 struct NbrGemm : DirectGemm {
   // reflection-basis form (k_sym.cu), SymKind.  kSymM2l: A is component-major,
   // [8 alpha + child][lda rows]; kSymNear4: A as above

@@ -24,13 +24,12 @@
 namespace fmmgb {
 namespace {
 
-constexpr int kRwWarps = 1;    // independent warps per CTA
 constexpr int kRwRows = 32;    // rows per warp
 constexpr int kRwTR = kRwRows / 8;  // rows per lane
 constexpr int kRwKC = 32;      // reduction values per stage
 constexpr int kRwPitch = kRwKC + 4;
 constexpr int kRwStage = kRwRows * kRwPitch + kRwKC * kNTile;  // floats
-constexpr size_t kRwSmem = sizeof(float) * (size_t)kRwWarps * 2 * kRwStage;
+constexpr size_t kRwSmem = sizeof(float) * 2 * kRwStage;
 
 struct RowsGroup {
   NbrGemm g[kRowsGroupMax];
@@ -79,12 +78,9 @@ __device__ __forceinline__ void rw_stage(const float* As, const float* Ws, int k
   }
 }
 
-__global__ void __launch_bounds__(32 * kRwWarps) nbr_gemm_rows_kernel(const __grid_constant__ RowsGroup G, int per_tile,
-                                                                      int items) {
+__global__ void __launch_bounds__(32) nbr_gemm_rows_kernel(const __grid_constant__ RowsGroup G, int per_tile) {
   extern __shared__ __align__(16) float rw_smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int item = (int)blockIdx.x * kRwWarps + warp;
-  if (item >= items) return;
+  const int lane = threadIdx.x, item = (int)blockIdx.x;
   const int tile = item / per_tile;  // longest reductions first
   int rem = item - tile * per_tile, li = 0;
   while (li + 1 < G.n && rem >= G.first[li + 1]) ++li;
@@ -98,7 +94,7 @@ __global__ void __launch_bounds__(32 * kRwWarps) nbr_gemm_rows_kernel(const __gr
   const int K = g.tile_k[tile];
   const float* W = static_cast<const float*>(g.W) + g.tile_w[tile] + (long long)d * K * kNTile;
   const float* A = static_cast<const float*>(g.A);
-  float* st = rw_smem + warp * 2 * kRwStage;
+  float* st = rw_smem;
 
   // this lane's 16-byte pieces: rows (lane / 8) + 4 i, piece lane % 8 of each
   const int q = lane & 7;
@@ -140,10 +136,8 @@ __global__ void __launch_bounds__(32 * kRwWarps) nbr_gemm_rows_kernel(const __gr
     const float* As = st + b * kRwStage;
     const float* Ws = As + kRwRows * kRwPitch;
     const int kn = min(kRwKC, K - kc);
-    if (live > 8 * (kRwTR / 2))
+    if (live > 16)
       rw_stage<kRwTR>(As, Ws, kn, rg, cg, acc);
-    else if (kRwTR > 4 && live > 16)
-      rw_stage<kRwTR < 4 ? kRwTR : 4>(As, Ws, kn, rg, cg, acc);
     else if (live > 8)
       rw_stage<2>(As, Ws, kn, rg, cg, acc);
     else
@@ -203,8 +197,7 @@ cudaError_t launch_nbr_gemm_rows(const NbrGemm* gs, int n, cudaStream_t s) {
   if (G.n == 0) return cudaSuccess;
   const long long items = per_tile * gs[0].ntiles;
   if (items > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  nbr_gemm_rows_kernel<<<(unsigned)((items + kRwWarps - 1) / kRwWarps), 32 * kRwWarps, kRwSmem, s>>>(
-      G, (int)per_tile, (int)items);
+  nbr_gemm_rows_kernel<<<(unsigned)items, 32, kRwSmem, s>>>(G, (int)per_tile);
   if (cudaError_t e = cudaGetLastError()) return e;
   long long blocks = 0;
   for (int i = 0; i < G.n; ++i) {

@@ -414,11 +414,10 @@ template <typename T>
 cudaError_t launch_nbr_gemm_simt(const NbrGemm& g, cudaStream_t s) {
   const long long tiles = (long long)((g.grid[0] + 3) / 4) * ((g.grid[1] + 3) / 4) * ((g.grid[2] + 3) / 4);
   if (tiles <= 0 || g.ntiles <= 0) return cudaSuccess;
-  long long items = tiles * g.ntiles * (g.dsplit > 1 ? 27 : 1);
-  if (g.max_blocks > 0 && items > g.max_blocks) items = g.max_blocks;
+  const long long items = tiles * g.ntiles * (g.dsplit > 1 ? 27 : 1);
   if (items > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   if constexpr (sizeof(T) == 4) {  // reduction lengths and columns are multiples of 8 (8 children, or b^3 cells)
-    if (g.dsplit == 27 && g.max_blocks == 0) return launch_nbr_gemm_rows(&g, 1, s);
+    if (g.dsplit == 27) return launch_nbr_gemm_rows(&g, 1, s);
   }
   nbr_gemm_simt_kernel<T><<<(unsigned)items, 64, 0, s>>>(g);
   cudaError_t e = cudaGetLastError();
