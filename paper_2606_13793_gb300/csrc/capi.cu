@@ -2920,8 +2920,13 @@ fmm_status do_far_item(fmm_plan_t P, const FarItem& it, cudaStream_t s) {
 // 96^3 with force columns 5.32 -> 4.54 ms, 160^3 4.46 -> 3.58 ms.  With the
 // final-stage M2P, itself as long, they keep `side` (adjoint at 208 x 216 x 136,
 // order 3: 14.0 ms, 21.3 ms on `side2`), and a split near field runs behind it
-// (near_behind).
-cudaStream_t levels_stream(fmm_plan_t P, bool adj_g) {
+// (near_behind).  The FP64 transpose of the analytic force has a direct near
+// field of one long wave at leaf 4, which levels beside it (0.1 to 1 ms) double:
+// there they run ahead of it on the caller's stream s (64^3, order 5: 8.04 ms so,
+// 12.5 to 14.4 ms beside it, 9.7 ms as direct levels beside it; FP32: no clear
+// winner, 0.66 and 0.82 ms at 64^3, 1.92 and 1.67 ms at 160^3).
+cudaStream_t levels_stream(fmm_plan_t P, bool adj_g, cudaStream_t s) {
+  if (adj_g && P->f64_data() && P->b == 4 && !P->m2p) return s;
   return !P->near_tc && P->b == 8 && !P->m2p && !adj_g ? P->side2 : P->side;
 }
 // Whether levels may run beside one another on `side2`: not while stages are
@@ -3017,8 +3022,9 @@ fmm_status run_solve(fmm_plan_t P, const T* rho, T* phi, T* accel, cudaStream_t 
     if (!cc && tc_first < 0) tc_first = l;
     any2 |= cc ? !(l == L && P->m2p) && level2(l) : l != tc_first;
   }
-  const bool fork = P->side && any_simt, fork2 = any2 && second_stream(P);
-  cudaStream_t sf = fork ? levels_stream(P, adj_g != nullptr) : s, s2 = fork2 ? P->side2 : s;
+  const cudaStream_t far = levels_stream(P, adj_g != nullptr, s);
+  const bool fork = P->side && any_simt && far != s, fork2 = any2 && second_stream(P);
+  cudaStream_t sf = fork ? far : s, s2 = fork2 ? P->side2 : s;
   if (fork || fork2) CUDA_TRY(cudaEventRecord(P->ev_fork, s));
   if (fork) CUDA_TRY(cudaStreamWaitEvent(sf, P->ev_fork, 0));
   if (fork2) CUDA_TRY(cudaStreamWaitEvent(s2, P->ev_fork, 0));

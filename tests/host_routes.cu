@@ -54,17 +54,20 @@ fmm_opts opts(int precision, int accel, int final_stage = 0) {
 
 // The levels beside a leaf-8 near field off the tensor cores run at its own
 // priority; with the final-stage M2P on the high-priority stream, a split near
-// field behind it; other leaves as ever.
+// field behind it.  The FP64 transpose of the analytic force at leaf 4: ahead of
+// the near field on the caller's stream.
 void leaf8_streams() {
   cudaStream_t hi = reinterpret_cast<cudaStream_t>(16), lo = reinterpret_cast<cudaStream_t>(32);
+  cudaStream_t own = reinterpret_cast<cudaStream_t>(48);
   for (int leaf : {2, 4, 8})
     for (int prec : {FMM_FP32, FMM_FP64})
       for (int m2p : {0, 1}) {
         Dry d(leaf * 12, leaf * 12, leaf * 12, 4, leaf, opts(prec, 1, m2p));
         d.P->side = hi, d.P->side2 = lo;
         const bool flat = leaf == 8 && !m2p;
-        expect(levels_stream(d.P, false) == (flat ? lo : hi), "levels' stream of a forward solve");
-        expect(levels_stream(d.P, true) == hi, "levels' stream of the transposed force");
+        expect(levels_stream(d.P, false, own) == (flat ? lo : hi), "levels' stream of a forward solve");
+        const bool ahead = leaf == 4 && prec == FMM_FP64 && !m2p;
+        expect(levels_stream(d.P, true, own) == (ahead ? own : hi), "levels' stream of the transposed force");
         for (int split : {1, 3}) {
           d.P->near_choice.dsplit = split;
           expect(near_behind(d.P, false) == (leaf == 8 && m2p && split > 1), "near field behind the final stage");
