@@ -2934,11 +2934,15 @@ cudaStream_t levels_stream(fmm_plan_t P, bool adj_g, cudaStream_t s) {
 // stage's time is its own launches' (512^3: 6.25 ms a solve so, 6.03 ms side by
 // side, where the tensor-core levels' spans held the near field's 1.1 ms).
 bool second_stream(fmm_plan_t P) { return P->side2 && !P->timing; }
-// Whether the near field runs on the levels' stream, after the final stage: a
-// split leaf-8 one, whose blocks and the direct M2P's (as long) only hold each
-// other up (FP64, 56 x 48 x 40, order 6: 29.9 ms so, 42.1 ms side by side).
-bool near_behind(fmm_plan_t P, bool adj_g) {
-  return !P->near_tc && P->b == 8 && P->m2p && P->near_choice.dsplit > 1 && !adj_g;
+// Whether the near field runs on the levels' stream, after them: a split one
+// (partial sums, so a small one) beside a tensor-core level that holds the
+// caller's stream (tc; TF32, leaf 2 with force columns, 64^3: 0.233 ms so, 0.253
+// behind that level; without one it is better beside the levels); and a split
+// leaf-8 one after the final stage, whose blocks and the direct M2P's (as long)
+// only hold each other up (FP64, 56 x 48 x 40, order 6: 29.9 ms so, 42.1 ms side
+// by side).
+bool near_behind(fmm_plan_t P, bool adj_g, bool tc) {
+  return !P->near_tc && P->near_choice.dsplit > 1 && !adj_g && (tc || (P->b == 8 && P->m2p));
 }
 
 // adjoint = true (fmm_solve_adjoint): the same chain on the adjoint source,
@@ -3023,7 +3027,8 @@ fmm_status run_solve(fmm_plan_t P, const T* rho, T* phi, T* accel, cudaStream_t 
     any2 |= cc ? !(l == L && P->m2p) && level2(l) : l != tc_first;
   }
   const cudaStream_t far = levels_stream(P, adj_g != nullptr, s);
-  const bool fork = P->side && any_simt && far != s, fork2 = any2 && second_stream(P);
+  const bool near_far = near_behind(P, adj_g != nullptr, tc_first >= 0);
+  const bool fork = P->side && (any_simt || near_far) && far != s, fork2 = any2 && second_stream(P);
   cudaStream_t sf = fork ? far : s, s2 = fork2 ? P->side2 : s;
   if (fork || fork2) CUDA_TRY(cudaEventRecord(P->ev_fork, s));
   if (fork) CUDA_TRY(cudaStreamWaitEvent(sf, P->ev_fork, 0));
@@ -3052,7 +3057,7 @@ fmm_status run_solve(fmm_plan_t P, const T* rho, T* phi, T* accel, cudaStream_t 
     StageTimer t(P, ST_M2L, sf);
     if ((st = do_p2l(P, sf))) return st;
   }
-  const bool behind = fork && near_behind(P, adj_g != nullptr);
+  const bool behind = fork && near_far;
   if (behind) {
     StageTimer t(P, ST_NEAR, sf);
     CUDA_TRY(launch_nbr_gemm<T>(near_gemm(P), sf));

@@ -70,8 +70,10 @@ void leaf8_streams() {
         expect(levels_stream(d.P, true, own) == (ahead ? own : hi), "levels' stream of the transposed force");
         for (int split : {1, 3}) {
           d.P->near_choice.dsplit = split;
-          expect(near_behind(d.P, false) == (leaf == 8 && m2p && split > 1), "near field behind the final stage");
-          expect(!near_behind(d.P, true), "the transposed force's near field is unsplit");
+          expect(near_behind(d.P, false, false) == (leaf == 8 && m2p && split > 1), "near field behind the final stage");
+          expect(near_behind(d.P, false, true) == (split > 1), "a split near field beside a tensor-core level");
+          expect(!near_behind(d.P, true, false) && !near_behind(d.P, true, true),
+                 "the transposed force's near field is unsplit");
         }
         d.P->side = d.P->side2 = nullptr;
       }
