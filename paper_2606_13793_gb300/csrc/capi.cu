@@ -2920,13 +2920,22 @@ fmm_status do_far_item(fmm_plan_t P, const FarItem& it, cudaStream_t s) {
 // 96^3 with force columns 5.32 -> 4.54 ms, 160^3 4.46 -> 3.58 ms.  With the
 // final-stage M2P, itself as long, they keep `side` (adjoint at 208 x 216 x 136,
 // order 3: 14.0 ms, 21.3 ms on `side2`), and a split near field runs behind it
-// (near_behind).  The FP64 transpose of the analytic force has a direct near
-// field of one long wave at leaf 4, which levels beside it (0.1 to 1 ms) double:
-// there they run ahead of it on the caller's stream s (64^3, order 5: 8.04 ms so,
-// 12.5 to 14.4 ms beside it, 9.7 ms as direct levels beside it; FP32: no clear
-// winner, 0.66 and 0.82 ms at 64^3, 1.92 and 1.67 ms at 160^3).
+// (near_behind).  The transpose of the analytic force off the tensor cores has a
+// direct near field too, at leaf 4 of one long wave of few blocks; levels beside
+// it lengthen it by more than they take, and run ahead of it on the caller's
+// stream s instead: in FP64 always, in FP32 from order 5 on with more than 16
+// blocks and at most one an SM (shorter levels, a handful of blocks or several
+// waves lose 5 to 15% so).  Measured ahead, beside it, and beside it as direct
+// levels (ms; the last two vary by a fifth from run to run): FP64 64^3, order 5
+// 8.04, 12.5, 9.7; 48 x 80 x 40 7.96, 12.4, 8.8; FP32 order 7, 68 x 32 x 112 (48
+// blocks) 0.72, 0.92 to 1.02, 0.86 to 1.11; order 6, 64^3 (32) 0.66, 0.84, 0.66 to
+// 0.90, 160^3 (500) 1.92, 1.67, 2.63; order 2, 20 x 24 x 124 (16) 0.63, 0.59, 0.60.
 cudaStream_t levels_stream(fmm_plan_t P, bool adj_g, cudaStream_t s) {
-  if (adj_g && P->f64_data() && P->b == 4 && !P->m2p) return s;
+  const int* n = P->lev[P->L].n;
+  const long long adj_blocks = (long long)((n[0] + 7) / 8) * ((n[1] + 3) / 4) * ((n[2] + 7) / 8) * P->near_adj_ntiles;
+  if (adj_g && P->tc_kind < 0 && P->b == 4 && !P->m2p &&
+      (P->f64_data() || (P->p >= 5 && adj_blocks > 16 && adj_blocks <= 152)))
+    return s;
   return !P->near_tc && P->b == 8 && !P->m2p && !adj_g ? P->side2 : P->side;
 }
 // Whether levels may run beside one another on `side2`: not while stages are

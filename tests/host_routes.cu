@@ -54,8 +54,8 @@ fmm_opts opts(int precision, int accel, int final_stage = 0) {
 
 // The levels beside a leaf-8 near field off the tensor cores run at its own
 // priority; with the final-stage M2P on the high-priority stream, a split near
-// field behind it.  The FP64 transpose of the analytic force at leaf 4: ahead of
-// the near field on the caller's stream.
+// field behind it.  The transpose of the analytic force at leaf 4: ahead of
+// the near field on the caller's stream (FP32: order 5 on, 17 to 152 blocks).
 void leaf8_streams() {
   cudaStream_t hi = reinterpret_cast<cudaStream_t>(16), lo = reinterpret_cast<cudaStream_t>(32);
   cudaStream_t own = reinterpret_cast<cudaStream_t>(48);
@@ -66,8 +66,14 @@ void leaf8_streams() {
         d.P->side = hi, d.P->side2 = lo;
         const bool flat = leaf == 8 && !m2p;
         expect(levels_stream(d.P, false, own) == (flat ? lo : hi), "levels' stream of a forward solve");
-        const bool ahead = leaf == 4 && prec == FMM_FP64 && !m2p;
-        expect(levels_stream(d.P, true, own) == (ahead ? own : hi), "levels' stream of the transposed force");
+        // the transposed force's near field: 12 tiles (2 x 3 x 2) times its column tiles
+        for (int order : {4, 5, 8})
+          for (int nt : {1, 2, 12, 13}) {
+            d.P->p = order;
+            d.P->near_adj_ntiles = nt;
+            const bool ahead = leaf == 4 && !m2p && (prec == FMM_FP64 || (order >= 5 && (nt == 2 || nt == 12)));
+            expect(levels_stream(d.P, true, own) == (ahead ? own : hi), "levels' stream of the transposed force");
+          }
         for (int split : {1, 3}) {
           d.P->near_choice.dsplit = split;
           expect(near_behind(d.P, false, false) == (leaf == 8 && m2p && split > 1), "near field behind the final stage");
