@@ -117,8 +117,10 @@ enum SymKind { kSymNone = 0, kSymM2l = 1, kSymNear4 = 2, kSymM2p = 3 };
 // The kernels of the direct form (k_gemm_simt.cu, k_gemm_zrun.cu) take this part
 // alone: with the reflection basis' fields in their parameters they compile to
 // other registers (the long FP32 z-run on a leaf-8 near field with force columns,
-// 12^3 boxes: 3.98 ms, 3.90 ms without).
-struct DirectGemm {
+// 12^3 boxes: 3.98 ms, 3.90 ms without).  Whole 16-byte units: batch kernels
+// copy it to shared memory ahead of their tiles (16 fields: 1.882 ms, 1.896 ms
+// with 88 bytes).
+struct alignas(16) DirectGemm {
   const void* A;       // [rows][row_len]
   int row_len;
   int grid[3];         // row grid extents
@@ -137,7 +139,7 @@ struct DirectGemm {
   int skip_center = 0; // 1: W_d of the centre neighbour (d = 13) is all zero (the M2L: a parent's
                        // children are each other's near neighbours), and the kernels skip it
 };
-static_assert(sizeof(DirectGemm) == 88, "the fields of the direct form only");
+static_assert(sizeof(DirectGemm) == 96, "the fields of the direct form only");
 struct NbrGemm : DirectGemm {
   // reflection-basis form (k_sym.cu), SymKind.  kSymM2l: A is component-major,
   // [8 alpha + child][lda rows]; kSymNear4: A as above
@@ -160,7 +162,7 @@ constexpr long long kZrunNarrowBlocks = 8 * 152;
 cudaError_t launch_nbr_gemm_zrun_group(const NbrGemm* gs, int n, cudaStream_t s);
 // Few rows, FP32, split over the 27 neighbours (k_gemm_rows.cu): up to
 // kRowsGroupMax levels of one plan in one launch, each with its own scratch
-// for the partial sums; the sums of the simt kernel, bit for bit.
+// for the partial sums; the sums in the 4 x 4 x 4 tile's order.
 constexpr int kRowsGroupMax = 8;
 cudaError_t launch_nbr_gemm_rows(const NbrGemm* gs, int n, cudaStream_t s);
 
