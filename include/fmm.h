@@ -283,7 +283,10 @@ fmm_status fmm_solve_static(const fmm_grid* grid, int order, int leaf, const voi
  *                         on the plan's own workspace (3 timed launches after
  *                         one warm-up) and keeps the fastest.  Overwrites the
  *                         workspace (no solve state survives a solve anyway);
- *                         synchronises `stream`.  Results are cached per
+ *                         synchronises `stream`.  Each launch is timed alone:
+ *                         beside the other launches of a solve another variant
+ *                         can be the faster one, and the defaults are chosen
+ *                         in whole solves.  Results are cached per
  *                         process by contraction geometry (grid of rows, row
  *                         length, columns, order, leaf), so further plans of
  *                         the same shape only look the choice up.
@@ -420,7 +423,12 @@ int fmm_batch_launches(fmm_batch_t batch, int with_accel);
  * a NULL plan, FMM_ERR_CUDA for an error the synchronisation returns. */
 fmm_status fmm_check(fmm_plan_t plan);
 
-/* Bytes of device memory the plan holds (tables + workspace arena). */
+/* Bytes of device memory the plan holds (tables + workspace arena).  Beside the
+ * expansions and box data the arena holds scratch for neighbour-split partial
+ * sums, one for the M2L levels and one for a near field off the tensor cores (up
+ * to 64 MiB each, or what a split coarse level needs), and with the final-stage
+ * M2P off the tensor cores at leaf 2 and 4 a folded copy of the leaf multipoles
+ * beside the full ones ((p+1)^2 values a box: 5.4 GB at 512^3, leaf 2, order 8). */
 size_t fmm_workspace_bytes(fmm_plan_t plan);
 
 /* Number of kernel launches one fmm_solve() enqueues for this plan. */

@@ -1804,9 +1804,10 @@ void sym_default(fmm_plan_t P, const NbrGemm& g, fmm_plan_s::SimtChoice* c, bool
 // rows 0.064, 32^3 0.34, 64^3 2.25 ms): it wins below ~14000 rows a wave at
 // p = 8; a full one has 19456, for which the two are close at p = 6.  Both sums are FP32, this one of unsplit operands.  A caller that
 // lowers n_fp64_levels asks for the tensor cores on small levels and gets them.
-// Plans with the stencil force stay on them too: the stencil amplifies what
-// the split operands round (512^3: level 5 alone is 2.5e-5 of the force), and
-// the force keeps to that of earlier releases.
+// Plans with the stencil force stay on them too, whether a solve asks for the
+// force or not: the stencil amplifies what the split operands round (512^3:
+// level 5 alone moves the force by 2.5e-5, about half its own error), and those
+// plans keep the same sums as before this form, by choice.
 bool reflect_tc_level(const Level& lv) {
   const long long tiles = (long long)((lv.np[0] + kTcTileX - 1) / kTcTileX) * ((lv.np[1] + kTcTileY - 1) / kTcTileY) *
                           lv.np[2];
@@ -1842,8 +1843,10 @@ fmm_status plan_init(fmm_plan_t P, const int d3[3], double dx, double G, int ord
   {
     // CUDA-core precisions only: in the mixed ones the CUDA-core (FP64) levels
     // run beside the tensor-core levels and, compressed, their denser DFMA
-    // work slows those (512^3 bf16x3 step 8.35 ms against 8.11 ms).  P2M
-    // stages a box row's full and folded components in shared memory.
+    // work slows those (512^3 bf16x3 step 8.35 ms against 8.11 ms).  P2M stages
+    // full and folded components in shared memory, priced here for its FP32
+    // blocks of 16 parents; that leaves FP64 order 8 on the Cartesian form,
+    // although its blocks of 4 parents would fit.
     const size_t esz = o.precision == FMM_FP64 ? 8 : 4;
     const size_t stage = (size_t)16 * (8 * P->nc + 8 + 8 * P->nr + 8) * esz;
     P->harm_cc = (!tcp || o.coarse_fp32) && !o.m2l_cartesian && order >= 2 && stage <= 227 * 1024;
@@ -3695,9 +3698,8 @@ void build_fused(fmm_batch_t B, const void* const* rho, void* const* phi, void* 
   // the reflection basis, except the levels above the leaf level of FP32
   // batches.  Their unsplit direct sums carry the largest rounding of a batch,
   // which the 5-point force amplifies (a change of it shows as 2.2e-5 to
-  // 3.7e-5 of the force, against 5e-6 for the leaf level's): the force would
-  // differ from earlier releases' by more than their FP32 solves of one field
-  // agree in.  FP32 fields of leaf 8 keep the direct form at the leaf level too:
+  // 3.7e-5 of the force, against 5e-6 for the leaf level's): they keep the same
+  // sums as before this form, by choice.  FP32 fields of leaf 8 keep the direct form at the leaf level too:
   // its blocks fill the gaps of the long direct near field, whose launch a
   // second form would have to wait for (below).
   auto reflect = [&](fmm_plan_t P, int l) {

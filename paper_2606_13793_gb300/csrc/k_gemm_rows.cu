@@ -3,10 +3,10 @@
 //
 //   part_d[r][n] = sum_{k < K(n)} A[r + d][k] W_d[k][n],  C = sum_d part_d
 //
-// Each sum runs over k in order and the partials are added in neighbour order
-// (one rounding per step, as in k_gemm_simt.cu, whose results it reproduces
-// bit for bit: those levels carry the bulk of phi, and the 5-point force
-// amplifies any change of their rounding).
+// Each sum runs over k in order and the partials are added in neighbour order,
+// one rounding per step: the order of the 4 x 4 x 4 tile's split form, which it
+// replaced (those levels carry the bulk of phi, and the 5-point force amplifies
+// any change of their rounding).
 //
 // These levels (8, 64, 512 rows) are bound by latency: a chain of up to
 // 8 (p+1)^2 multiply-adds per output, and a kernel each.  So: one launch for

@@ -278,7 +278,7 @@ __device__ __forceinline__ void p2m_block(const T* __restrict__ rho, int nx, int
   } else {
     for (int i = threadIdx.x; i < count; i += kP2mThreads<T>) Mleaf[g0 + i] = Ms[(i / ROW) * ROWP + i % ROW];
   }
-  if (Mfold && harm == 2) {  // component-major (CUDA-core harmonic M2L): runs of the block's 16 parents
+  if (Mfold && harm == 2) {  // component-major (CUDA-core harmonic M2L): runs of the block's parents
     for (int i = threadIdx.x; i < kP2mParents<T> * ROWR; i += kP2mThreads<T>) {
       const int pr = i % kP2mParents<T>, k = i / kP2mParents<T>;
       if (pr < np) Mfold[(long long)k * leaf.npar + p0 + pr] = Mr[pr * rp + k];
@@ -368,7 +368,7 @@ cudaError_t p2m_launch(unsigned blocks, cudaStream_t s, const T* rho, int nx, in
                 int harm, T* Mfold, const T* dip, long long ncell, int rho_soa) {
   constexpr size_t full = (size_t)kP2mParents<T> * (8 * ncoef_c(P) + 8) * sizeof(T);
   // staged harmonic rows, where they fit beside the full ones (the plan folds
-  // nothing at FP64 order 8, which would not)
+  // nothing at FP64 order 8)
   constexpr size_t red0 = (size_t)kP2mParents<T> * (8 * nred_c(P) + 32) * sizeof(T);
   constexpr size_t red = full + red0 <= 227 * 1024 ? red0 : 0;
   if (harm && (Mhi || Mfold) && red == 0) return cudaErrorInvalidValue;
