@@ -114,12 +114,14 @@ enum SymKind { kSymNone = 0, kSymM2l = 1, kSymNear4 = 2, kSymM2p = 3 };
 // Neighbour-contraction ("implicit GEMM") description for the SIMT kernel:
 //   C[row][n] (+)= sum_{d in 27 neighbours} sum_{k < K(tile(n))} A[row + d][k] * W_d[k][n]
 // rows live on a 3-D grid; a neighbour outside the grid contributes zero.
-// The kernels of the direct form (k_gemm_simt.cu, k_gemm_zrun.cu) take this part
-// alone: with the reflection basis' fields in their parameters they compile to
-// other registers (the long FP32 z-run on a leaf-8 near field with force columns,
-// 12^3 boxes: 3.98 ms, 3.90 ms without).  Whole 16-byte units: batch kernels
-// copy it to shared memory ahead of their tiles (16 fields: 1.882 ms, 1.896 ms
-// with 88 bytes).
+// The direct form's own part.  A kernel compiles to other registers with the
+// reflection basis' fields in its parameters, for better or worse: the FP32 z-run
+// tiles take this part for near fields (leaf 8 with force columns, 12^3 boxes:
+// 3.90 ms, 3.98 ms with the whole description), and so do the batch kernels;
+// the M2L's and the FP64 tiles and k_gemm_simt.cu's the whole (FP64 column form,
+// 64 registers, 72 with this part: TF32 with FP64 coarse levels, M2P, order 7, 32 x
+// 24 x 144 1.62 and 1.70 ms).  Whole 16-byte units: batch kernels copy it to shared
+// memory ahead of their tiles (16 fields: 1.876 ms, 1.896 ms with 88 bytes).
 struct alignas(16) DirectGemm {
   const void* A;       // [rows][row_len]
   int row_len;

@@ -76,8 +76,8 @@ constexpr size_t zrun_smem_bytes() {
   return sizeof(T) * ((size_t)kZrKC * ZrHalo<RZ>::stride + (size_t)27 * kZrKC * kNTile);
 }
 
-template <typename T, int RZ>
-__device__ __forceinline__ void nbr_gemm_zrun_body(const DirectGemm& g, const VBlock vb) {
+template <typename T, int RZ, typename Gemm>
+__device__ __forceinline__ void nbr_gemm_zrun_body(const Gemm& g, const VBlock vb) {
   using H = ZrHalo<RZ>;
   using V = typename Vec<T>::type;
   constexpr int VN = Vec<T>::n;
@@ -214,8 +214,8 @@ __device__ __forceinline__ void nbr_gemm_zrun_body(const DirectGemm& g, const VB
   }
 }
 
-template <typename T, int RZ>
-__global__ void __launch_bounds__(kZrThreads, 4) nbr_gemm_zrun_kernel(DirectGemm g) {
+template <typename T, int RZ, typename Gemm>
+__global__ void __launch_bounds__(kZrThreads, 4) nbr_gemm_zrun_kernel(Gemm g) {
   nbr_gemm_zrun_body<T, RZ>(g, native_vblock());
 }
 
@@ -402,14 +402,22 @@ cudaError_t launch_rz_multi(const NbrGemm* gs, const MultiGrid* grids, int n, lo
 template <typename T, int RZ>
 cudaError_t launch_rz(const NbrGemm& g, cudaStream_t s) {
   constexpr size_t smem = zrun_smem_bytes<T, RZ>();
-  static SmemOptIn opt;
-  if (cudaError_t e = opt(nbr_gemm_zrun_kernel<T, RZ>, smem)) return e;
   const long long tiles = (long long)((g.grid[0] + kZrBX - 1) / kZrBX) * ((g.grid[1] + kZrBY - 1) / kZrBY) *
                           ((g.grid[2] + RZ - 1) / RZ);
   if (tiles <= 0 || g.ntiles <= 0) return cudaSuccess;
   if (tiles > 0x7fffffffLL || g.ntiles > 65535) return cudaErrorInvalidConfiguration;
   dim3 grid((unsigned)tiles, (unsigned)g.ntiles, (unsigned)g.dsplit);
-  nbr_gemm_zrun_kernel<T, RZ><<<grid, kZrThreads, smem, s>>>(g);
+  if constexpr (sizeof(T) == 4) {
+    if (!g.skip_center) {
+      static SmemOptIn opt;
+      if (cudaError_t e = opt(nbr_gemm_zrun_kernel<T, RZ, DirectGemm>, smem)) return e;
+      nbr_gemm_zrun_kernel<T, RZ, DirectGemm><<<grid, kZrThreads, smem, s>>>(g);
+      return cudaGetLastError();
+    }
+  }
+  static SmemOptIn opt;
+  if (cudaError_t e = opt(nbr_gemm_zrun_kernel<T, RZ, NbrGemm>, smem)) return e;
+  nbr_gemm_zrun_kernel<T, RZ, NbrGemm><<<grid, kZrThreads, smem, s>>>(g);
   return cudaGetLastError();
 }
 
