@@ -2851,11 +2851,12 @@ size_t rows_partial(fmm_plan_t P, int l) {
   return ((size_t)27 * lv.npar * 8 * (lv.fold_off ? P->nr : P->nc) * (lv.f64 ? 8 : 4) + 255) & ~(size_t)255;
 }
 // The launches of the CUDA-core levels ls[0 .. n) (coarse to fine) on one
-// stream: a level by itself, a row group, the narrow group; coarse to fine, a
-// group at its coarsest level.  Where FP64 coarse levels come first, their
-// kernels (no shared memory) then run beside a tensor-core near field, which row
-// groups wait out (bf16x3 order 0 with M2P, 140 x 164 x 96: 0.403 ms so, 0.442 ms
-// with the groups first).  No host allocation: solves call it.
+// stream: a level by itself, a row group, the narrow group.  The groups go first,
+// but for the FP64 levels of a mixed plan, whose kernels (no shared memory) run
+// beside a tensor-core near field that row groups wait out (bf16x3 order 0 with
+// M2P, 140 x 164 x 96: 0.403 ms so, 0.442 ms with the groups first); the narrow
+// group ahead of a split coarser level (FP32 Cartesian 160^3: 1.92 ms so, 2.1 to
+// 2.3 ms in level order).  No host allocation: solves call it.
 constexpr int kFarGroup = std::min({kSymGroupMax, kRowsGroupMax, kZrunGroupMax});
 struct FarItem {
   enum Kind { kLevel, kRows, kNarrow } kind;
@@ -2873,29 +2874,35 @@ int far_items(fmm_plan_t P, const int* ls, int n, FarItem (&out)[kMaxLevels]) {
     it.ls[0] = l;
     return &it;
   };
+  auto first = [&](int l) { return P->tc_kind >= 0 && P->lev[l].f64 && !rows_level(P, l); };
+  for (int i = 0; i < n; ++i)
+    if (first(ls[i])) add(FarItem::kLevel, ls[i]);
   for (int i = 0; i < n; ++i) {
     const int l = ls[i];
-    if (rows_level(P, l)) {
-      const int s = P->m2l_choice[l].shape == 3;
-      const size_t need = rows_partial(P, l);
-      FarItem* g = rows[s];
-      if (!g || used[s] + need > P->part_cap || g->n == kFarGroup || P->lev[l].f64 != P->lev[g->ls[0]].f64 ||
-          sym_level(P, l) != sym_level(P, g->ls[0])) {
-        rows[s] = add(FarItem::kRows, l);
-        used[s] = need;
-      } else {
-        g->ls[g->n++] = l;
-        used[s] += need;
-      }
-    } else if (narrow_level(P, l) && (!narrow || narrow->n < kFarGroup)) {
-      if (narrow)
-        narrow->ls[narrow->n++] = l;
-      else
-        narrow = add(FarItem::kNarrow, l);
+    if (!rows_level(P, l)) continue;
+    const int s = P->m2l_choice[l].shape == 3;
+    const size_t need = rows_partial(P, l);
+    FarItem* g = rows[s];
+    if (!g || used[s] + need > P->part_cap || g->n == kFarGroup || P->lev[l].f64 != P->lev[g->ls[0]].f64 ||
+        sym_level(P, l) != sym_level(P, g->ls[0])) {
+      rows[s] = add(FarItem::kRows, l);
+      used[s] = need;
     } else {
-      add(FarItem::kLevel, l);
+      g->ls[g->n++] = l;
+      used[s] += need;
     }
   }
+  for (int i = 0; i < n; ++i) {
+    const int l = ls[i];
+    if (rows_level(P, l) || !narrow_level(P, l) || (narrow && narrow->n == kFarGroup)) continue;
+    if (narrow)
+      narrow->ls[narrow->n++] = l;
+    else
+      narrow = add(FarItem::kNarrow, l);
+  }
+  auto in_narrow = [&](int l) { return narrow && std::find(narrow->ls, narrow->ls + narrow->n, l) != narrow->ls + narrow->n; };
+  for (int i = 0; i < n; ++i)
+    if (!first(ls[i]) && !rows_level(P, ls[i]) && !in_narrow(ls[i])) add(FarItem::kLevel, ls[i]);
   return items;
 }
 fmm_status do_far_item(fmm_plan_t P, const FarItem& it, cudaStream_t s) {

@@ -106,10 +106,11 @@ void leaf8_batch() {
   }
 }
 
-// The far field's launches go coarse to fine, groups at their coarsest level.
+// The far field's launches: the FP64 levels of a mixed plan, the row groups, the
+// narrow group, the other levels; every level once, without a host allocation.
 void far_order() {
-  auto first = [](fmm_plan_t P, FarItem::Kind* kind) {
-    int ls[kMaxLevels], n = 0, seen = 0, last = 0;
+  auto kinds = [](fmm_plan_t P) {
+    int ls[kMaxLevels], n = 0, seen = 0;
     for (int l = 2; l <= P->L; ++l)
       if (!P->lev[l].tc && !(l == P->L && P->m2p)) ls[n++] = l;
     FarItem items[kMaxLevels];
@@ -117,25 +118,36 @@ void far_order() {
     const int m = far_items(P, ls, n, items);
     (void)fmm_solve_launches(P, 1);
     expect(allocations == before, "no host allocation (an exception would cross the C interface)");
+    std::string s;
+    bool once[kMaxLevels] = {};
     for (int i = 0; i < m; ++i) {
-      expect(items[i].ls[0] > last, "coarse to fine");
-      last = items[i].ls[0];
-      seen += items[i].n;
+      s += items[i].kind == FarItem::kRows ? 'r' : items[i].kind == FarItem::kNarrow ? 'n' : 'l';
+      for (int k = 0; k < items[i].n; ++k) {
+        expect(!once[items[i].ls[k]], "a level once");
+        once[items[i].ls[k]] = true;
+        ++seen;
+      }
     }
-    expect(seen == n, "every level once");
-    *kind = items[0].kind;
-    return m;
+    expect(seen == n, "every level");
+    return s;
   };
-  FarItem::Kind k;
+  Dry fp32(64, 64, 64, 6, 4, opts(FMM_FP32, 1));
+  expect(kinds(fp32.P) == "r", "levels of at most 512 rows in one group");
+  Dry mid(96, 96, 96, 6, 4, opts(FMM_FP32, 1));
+  expect(kinds(mid.P) == "rl", "the group ahead of the leaf level");
+  // Cartesian: the unsplit leaf level in the narrow form ahead of the split one above it
+  fmm_opts o = opts(FMM_FP32, 1);
+  o.m2l_cartesian = 1;
+  Dry cart(160, 160, 160, 6, 4, o);
+  expect(cart.P->m2l_choice[5].dsplit > 1 && narrow_level(cart.P, 6) && kinds(cart.P) == "rnl", "the narrow group second");
   // the levels of a mixed plan with FP64 coarse levels: two of those (one column
-  // per lane, split), then FP32 ones in a row group
+  // per lane, split), then FP32 ones in row groups
   Dry mixed(128, 128, 128, 0, 4, opts(FMM_FP32, 1));
+  mixed.P->tc_kind = TC_BF16X3;
   for (int l : {2, 3}) mixed.P->lev[l].f64 = 1, mixed.P->m2l_choice[l].shape = 3;
   for (int l = 2; l <= mixed.P->L; ++l) mixed.P->m2l_choice[l].dsplit = 27;
   for (int l = 4; l <= mixed.P->L; ++l) mixed.P->m2l_choice[l].shape = 0;
-  expect(first(mixed.P, &k) >= 3 && k == FarItem::kLevel, "FP64 levels ahead of the row group");
-  Dry fp32(64, 64, 64, 6, 4, opts(FMM_FP32, 1));
-  expect(first(fp32.P, &k) == 1 && k == FarItem::kRows, "levels of at most 512 rows in one group");
+  expect(kinds(mixed.P).substr(0, 3) == "llr", "the FP64 levels ahead of the row groups");
 }
 
 // The near field's own scratch takes every split that the M2L's, which it used
