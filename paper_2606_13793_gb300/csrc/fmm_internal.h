@@ -115,13 +115,15 @@ enum SymKind { kSymNone = 0, kSymM2l = 1, kSymNear4 = 2, kSymM2p = 3 };
 //   C[row][n] (+)= sum_{d in 27 neighbours} sum_{k < K(tile(n))} A[row + d][k] * W_d[k][n]
 // rows live on a 3-D grid; a neighbour outside the grid contributes zero.
 // The direct form's own part.  A kernel compiles to other registers with the
-// reflection basis' fields in its parameters, for better or worse: the FP32 z-run
-// tiles take this part for near fields (leaf 8 with force columns, 12^3 boxes:
-// 3.90 ms, 3.98 ms with the whole description), and so do the batch kernels;
-// the M2L's and the FP64 tiles and k_gemm_simt.cu's the whole (FP64 column form,
-// 64 registers, 72 with this part: TF32 with FP64 coarse levels, M2P, order 7, 32 x
-// 24 x 144 1.62 and 1.70 ms).  Whole 16-byte units: batch kernels copy it to shared
-// memory ahead of their tiles (16 fields: 1.876 ms, 1.896 ms with 88 bytes).
+// reflection basis' fields in its parameters, for better or worse.  This part:
+// the FP32 z-run tiles of near fields (leaf 8 with force columns, 12^3 boxes: 3.90
+// ms, 3.98 ms with the whole description), the column form (FP64 coarse levels of
+// a bf16x3 plan, 64^3, order 4: a solve 0.349 ms, 0.410 with the whole; TF32 M2P,
+// order 7, 32 x 24 x 144 the other way, 1.70 and 1.62 ms) and the batch kernels;
+// the whole: the z-run tiles otherwise (FP64 leaf-8 P2L, 32 x 16 x 24: 124.7 ms,
+// 125.3 with this part) and the 4 x 4 x 4 tile.  Whole 16-byte units: batch kernels
+// copy it to shared memory ahead of their tiles (16 fields: 1.876 ms, 1.896 ms with
+// 88 bytes).
 struct alignas(16) DirectGemm {
   const void* A;       // [rows][row_len]
   int row_len;

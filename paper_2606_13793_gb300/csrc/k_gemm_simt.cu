@@ -147,8 +147,8 @@ __global__ void __launch_bounds__(64) nbr_gemm_simt_multi_kernel(const NbrGemm* 
 // broadcast activation per row) are cheap beside the FMAs.
 constexpr int kColRows = 4;  // rows per warp
 
-template <typename T, typename Gemm>
-__device__ __forceinline__ void nbr_gemm_col_body(const Gemm& g, const VBlock vb) {
+template <typename T>
+__device__ __forceinline__ void nbr_gemm_col_body(const DirectGemm& g, const VBlock vb) {
   constexpr int R = kColRows;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long rows = (long long)g.grid[0] * g.grid[1] * g.grid[2];
@@ -207,7 +207,7 @@ __device__ __forceinline__ void nbr_gemm_col_body(const Gemm& g, const VBlock vb
 }
 
 template <typename T>
-__global__ void __launch_bounds__(128) nbr_gemm_col_kernel(NbrGemm g) {
+__global__ void __launch_bounds__(128) nbr_gemm_col_kernel(DirectGemm g) {
   nbr_gemm_col_body<T>(g, native_vblock());
 }
 
